@@ -1033,12 +1033,14 @@ cudaError_t run_backward(const lqt_problem& p, const Layout& L, size_t elem_byte
   // are recomputed there, segment by segment
   const bool one_segment = T <= adjoint_segment(T) && T <= kAdjSegment;
   if (one_segment) {
+    cf.uni = nullptr;  // every sub-interval's RK4 stages are recorded
     e = launch_build_stages_range(p, L, cf, 0, T, (double*)(ws + b.ys), st, el);
     if (e == cudaSuccess) e = launch_terminal_element(p, el, st);
   } else {
     e = launch_build(p, L, cf, el, st);
   }
   if (e != cudaSuccess) return e;
+  cf.uni = nullptr;
   double* maps = (double*)(ws + b.maps);
   e = launch_maps_from_values(p, el, S, v, maps, st);
   if (e != cudaSuccess) return e;

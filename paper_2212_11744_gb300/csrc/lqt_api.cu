@@ -73,6 +73,9 @@ static Layout make_layout(const lqt_problem& p) {
   L.off_Ku = off;
   const bool ku_const = p.L.mode == LQT_CONST && p.U.mode == LQT_CONST;
   off = align_up(off + (ku_const ? 1 : (size_t)p.T + 1) * (size_t)p.m * p.n * sizeof(double));
+  L.uniform = uniform_eligible(p);
+  L.off_uni = off;
+  if (L.uniform) off += uniform_table_bytes(p.n, L.M);
   L.coef_bytes = off;
   return L;
 }
@@ -527,6 +530,7 @@ lqt_status lqt_solve_host(const lqt_problem* hp, const double* x0, double* S, do
     double* qr = (double*)(base + L.off_qr);
     double* Ku = (double*)(base + L.off_Ku);
     const bool ku_const = d.L.mode == LQT_CONST && d.U.mode == LQT_CONST;
+    const double* uni = L.uniform ? (const double*)(base + L.off_uni) : nullptr;
     const ElemPtrs el = carve_elements(d, base + L.coef_bytes);
     const int64_t P = (d.T + chunk - 1) / chunk;
     for (int64_t c = 0; c < P && e == cudaSuccess; ++c) {
@@ -554,6 +558,9 @@ lqt_status lqt_solve_host(const lqt_problem* hp, const double* x0, double* S, do
                               st);
       const ElemPtrs elw{el.A + j0 * n * n, el.b + j0 * n, el.C + j0 * n * n, el.eta + j0 * n, el.J + j0 * n * n,
                          el.zeta + j0};
+      // one table for the whole grid (its time points were copied first)
+      cfw.uni = uni;
+      if (e == cudaSuccess && uni && c == 0) e = launch_uniform_master(d, cfw, st);
       if (e == cudaSuccess) e = launch_build_range(pw, Lw, cfw, elw, st);
     }
     if (e == cudaSuccess) e = launch_terminal_element(d, el, st);

@@ -126,13 +126,21 @@ __global__ void controls_cost_kernel(BatchDev bd, const double* S, const double*
 // Workspace layout of a batch.
 struct BatchLayout {
   int32_t B, n, m, K, M;
-  int64_t total, total_qr;
-  size_t off_probs, off_off, off_offqr, off_Lt, off_Ku, off_qr, off_el, off_team, off_inv, off_scan, bytes;
+  int64_t total, total_qr, maxT;
+  bool uniform;  // the constant-coefficient build applies to at least one problem
+  size_t off_probs, off_off, off_offqr, off_Lt, off_Ku, off_qr, off_el, off_team, off_inv, off_uni, off_scan, bytes;
 };
 
 static int32_t batch_factor_width(int n, int m) {
   if (n == 64) return 16;
   return padded_M(m);
+}
+
+// Whether problem p of a batch has a table of the constant-coefficient build.
+// A table costs one element's integration per problem, so short problems keep
+// the general build; n = 64 tables (MBs each) are left to single problems.
+static bool batch_uniform_member(const lqt_problem& p) {
+  return p.n <= 16 && p.T >= 64 && !p.c.ptr && (!p.r.ptr || p.r.mode != LQT_PER_STAGE);
 }
 
 static lqt_status batch_validate(const lqt_batch* bt, BatchLayout& L) {
@@ -149,6 +157,8 @@ static lqt_status batch_validate(const lqt_batch* bt, BatchLayout& L) {
   const int maxM = n == 1 ? 1 : n == 2 ? 2 : n <= 4 ? 4 : n == 8 ? 8 : 16;
   if (L.M > maxM) return LQT_EUNSUPPORTED;
   int64_t total = 0, total_qr = 0;
+  L.maxT = 0;
+  L.uniform = false;
   for (int32_t b = 0; b < bt->count; ++b) {
     const lqt_problem& p = bt->problems[b];
     if (p.n != n || p.m != p0.m || p.nr != n || p.K != p0.K || p.T < 1) return LQT_EINVAL;
@@ -160,6 +170,8 @@ static lqt_status batch_validate(const lqt_batch* bt, BatchLayout& L) {
     const int32_t rm0 = p0.r.ptr ? p0.r.mode : LQT_CONST;
     if (rm != rm0 || (rm != LQT_CONST && rm != LQT_PER_INTERVAL && rm != LQT_PER_STAGE)) return LQT_EINVAL;
     if (!bt->x0[b]) return LQT_EINVAL;
+    if (p.T > L.maxT) L.maxT = p.T;
+    L.uniform = L.uniform || batch_uniform_member(p);
     total += p.T + 1;
     total_qr += p.r.ptr ? sample_count(rm, p.T, p.K) : 1;
   }
@@ -179,6 +191,9 @@ static lqt_status batch_validate(const lqt_batch* bt, BatchLayout& L) {
   // per-problem tables of the time-invariant build (when it supports n)
   L.off_inv = off;
   if (invariant_supported(n, L.M)) off = bal(off + (size_t)L.B * invariant_table_bytes(n, L.M, L.K));
+  // per-problem tables of the constant-coefficient build
+  L.off_uni = off;
+  if (L.uniform) off = bal(off + (size_t)L.B * uniform_table_bytes(n, L.M));
   // The scans may run with any first-level chunk the caller's tuning picks;
   // the shortest chunk (2) needs the most level storage, so size for it.
   const int prev = scan_chunk_override();
@@ -265,6 +280,9 @@ lqt_status lqt_batch_plan(const lqt_batch* bt, void* ws, size_t ws_bytes, void* 
     P.cf.Ku = (const double*)(w + L.off_Ku) + (size_t)b * L.m * L.n;
     P.cf.Ku_per_boundary = 0;
     P.cf.M = L.M;
+    P.cf.uni = L.uniform && batch_uniform_member(p)
+                   ? (const double*)(w + L.off_uni + (size_t)b * uniform_table_bytes(L.n, L.M))
+                   : nullptr;
     off[b] = o;
     offqr[b] = oq;
     o += p.T + 1;
@@ -303,6 +321,7 @@ lqt_status lqt_solve_batched(const lqt_batch* bt, const lqt_tuning* tune, double
   set_scan_chunk(chunk);
   cudaError_t e = batch_prepare(bd, st);
   const ElemPtrs el = batch_elements(L, w);
+  if (e == cudaSuccess && !invariant && L.uniform) e = batch_uniform(bd, L.maxT, el, st);
   if (e == cudaSuccess)
     e = invariant ? batch_build_invariant(bd, el, (double*)(w + L.off_inv), st)
                   : batch_build(bd, el, w + L.off_team, st);

@@ -11,6 +11,7 @@
 
 #include "lqt_device.cuh"
 #include "lqt_internal.h"
+#include "lqt_uniform.cuh"
 
 namespace lqt {
 
@@ -316,12 +317,15 @@ Coefs coefs_view(const lqt_problem& p, const Layout& lay, double* Lt, double* Q,
   cf.Ku = Ku;
   cf.Ku_per_boundary = ku_const ? 0 : 1;
   cf.M = lay.M;
+  cf.uni = nullptr;
   return cf;
 }
 
 cudaError_t launch_prepare_coefs(const lqt_problem& p, const Layout& lay, char* ws, Coefs& cf, cudaStream_t st) {
-  return launch_prepare_into(p, lay, (double*)(ws + lay.off_Lt), (double*)(ws + lay.off_Q),
-                             (double*)(ws + lay.off_qr), (double*)(ws + lay.off_Ku), cf, st);
+  const cudaError_t e = launch_prepare_into(p, lay, (double*)(ws + lay.off_Lt), (double*)(ws + lay.off_Q),
+                                            (double*)(ws + lay.off_qr), (double*)(ws + lay.off_Ku), cf, st);
+  if (lay.uniform) cf.uni = (const double*)(ws + lay.off_uni);
+  return e;
 }
 
 // ---------------------------------------------------------------------------
@@ -557,7 +561,7 @@ __device__ __forceinline__ void build_one(const Coefs& cf, const double* t, int6
 template <int N, int M>
 __global__ void __launch_bounds__(128) build_kernel(BuildArgs a) {
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= a.T) return;
+  if (j >= a.T || uniform_near(a.cf.uni, a.t, j, a.K)) return;
   Elem<N> y;
   build_one<N, M>(a.cf, a.t, j, a.K, y);
   store_public<N>(a.out, j, y);
@@ -716,6 +720,7 @@ __global__ void __launch_bounds__(128) batch_build_kernel(BatchDev bd, ElemPtrs 
   const int64_t j = g - P.off;
   Elem<N> y;
   if (j < P.T) {
+    if (uniform_near(P.cf.uni, P.t, j, bd.K)) return;
     build_one<N, M>(P.cf, P.t, j, bd.K, y);
   } else {
 #pragma unroll
@@ -821,11 +826,16 @@ cudaError_t launch_build_stages_range(const lqt_problem& p, const Layout& lay, c
   }
 }
 
-// Elements 0..T-1 of p alone (no terminal element), n <= 8.
+// Elements 0..T-1 of p alone (no terminal element), n <= 8; cf.uni, when set,
+// holds a finished table.
 cudaError_t launch_build_range(const lqt_problem& p, const Layout& lay, const Coefs& cf, const ElemPtrs& out,
                                cudaStream_t st) {
   BuildArgs a;
   a.T = p.T; a.K = p.K; a.t = p.t; a.cf = cf; a.out = out;
+  if (cf.uni) {
+    const cudaError_t e = launch_uniform_expand(p, cf, out, st);
+    if (e != cudaSuccess) return e;
+  }
   switch (p.n) {
     case 1: return launch_build_n<1>(a, lay.M, st);
     case 2: return launch_build_n<2>(a, lay.M, st);
@@ -836,11 +846,21 @@ cudaError_t launch_build_range(const lqt_problem& p, const Layout& lay, const Co
   }
 }
 
-cudaError_t launch_build(const lqt_problem& p, const Layout& lay, const Coefs& cf, const ElemPtrs& out,
+cudaError_t launch_build(const lqt_problem& p, const Layout& lay, const Coefs& cf_in, const ElemPtrs& out,
                          cudaStream_t st, double* team_scratch) {
+  Coefs cf = cf_in;
+  // the mixed-precision path's FP32 products amplify a last-bit change of an
+  // element to their own rounding: its elements stay as the general build
+  // makes them
+  if (mixed_precision()) cf.uni = nullptr;
   BuildArgs a;
   a.T = p.T; a.K = p.K; a.t = p.t; a.cf = cf; a.out = out;
   cudaError_t e;
+  if (cf.uni) {
+    e = launch_uniform_master(p, cf, st);
+    if (e == cudaSuccess) e = launch_uniform_expand(p, cf, out, st);
+    if (e != cudaSuccess) return e;
+  }
   if (team_build_preferred(p.n, p.T)) {
     e = team_launch_build_small(p, lay, cf, 0, p.T, nullptr, out, st);
     if (e != cudaSuccess) return e;

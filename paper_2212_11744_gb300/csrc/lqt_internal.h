@@ -61,6 +61,9 @@ struct Coefs {
   const double* Ku;
   int32_t Ku_per_boundary;
   int32_t M;  // padded column count of Lt
+  // table of the constant-coefficient build (lqt_uniform.cu); NULL: the
+  // general build makes every element
+  const double* uni;
 };
 
 struct ElemPtrs {
@@ -73,7 +76,8 @@ struct Layout {
   int64_t T;
   int32_t mode_Lt, mode_Q, mode_qr;
   // byte offsets inside the workspace
-  size_t off_Lt, off_Q, off_qr, off_Ku, off_status;
+  size_t off_Lt, off_Q, off_qr, off_Ku, off_uni;
+  bool uniform;  // the constant-coefficient build applies (lqt_uniform.cu)
   size_t coef_bytes;  // end of the coefficient region
 };
 
@@ -103,6 +107,14 @@ cudaError_t launch_build_range(const lqt_problem& p, const Layout& lay, const Co
                                cudaStream_t st);
 cudaError_t launch_build_stages_range(const lqt_problem& p, const Layout& lay, const Coefs& cf, int64_t j0,
                                       int64_t cnt, double* stages, cudaStream_t st, const ElemPtrs& out);
+// Constant F, L, U, X without drift on a nearly uniform grid (lqt_uniform.cu):
+// the table (cf.uni) from the grid's mean step, then the elements of the
+// sub-intervals that have it; the general build makes the others.
+bool uniform_eligible(const lqt_problem& p);
+int64_t uniform_table_doubles(int n, int M);
+size_t uniform_table_bytes(int n, int M);
+cudaError_t launch_uniform_master(const lqt_problem& p, const Coefs& cf, cudaStream_t st);
+cudaError_t launch_uniform_expand(const lqt_problem& p, const Coefs& cf, const ElemPtrs& out, cudaStream_t st);
 cudaError_t launch_terminal_element(const lqt_problem& p, const ElemPtrs& out, cudaStream_t st);
 cudaError_t launch_build(const lqt_problem& p, const Layout& lay, const Coefs& cf, const ElemPtrs& out,
                          cudaStream_t s, double* team_scratch = nullptr);
@@ -226,6 +238,7 @@ __host__ __device__ __forceinline__ int32_t batch_find(const int64_t* off, int32
 
 cudaError_t batch_prepare(const BatchDev& bd, cudaStream_t st);
 cudaError_t batch_build(const BatchDev& bd, const ElemPtrs& el, char* team_scratch, cudaStream_t st);
+cudaError_t batch_uniform(const BatchDev& bd, int64_t maxT, const ElemPtrs& out, cudaStream_t st);
 cudaError_t batch_build_team(const BatchDev& bd, const ElemPtrs& el, double* gscratch, cudaStream_t st);
 cudaError_t batch_build_invariant(const BatchDev& bd, const ElemPtrs& el, double* tables, cudaStream_t st);
 void launch_inv_batch_build_warp(const BatchDev& bd, const double* tables, const ElemPtrs& out, cudaStream_t st);

@@ -12,6 +12,7 @@
 
 #include "lqt_device.cuh"
 #include "lqt_internal.h"
+#include "lqt_uniform.cuh"
 #include "lqt_team.cuh"
 #include "lqt_warp16.cuh"
 #include "lqt_warp8.cuh"
@@ -195,6 +196,7 @@ __global__ void __launch_bounds__(TeamCfg<N>::TEAM, TeamCfg<N>::BUILD_MIN) build
   double* P = AL + N * M;
   double* w = P + N * M;
   for (int64_t j = blockIdx.x; j < a.T; j += gridDim.x) {
+    if (uniform_near(a.cf.uni, a.t, j, a.K)) continue;  // written by the constant-coefficient build
     team_build_one<N, M>(lane, a.cf, a.t, j, a.K, yb, ynb, ytb, kb, AL, P, w);
     double zz = 0.0;
     Rec<N> dst = Rec<N>::pub(a.out, j, &zz);
@@ -223,6 +225,7 @@ __global__ void __launch_bounds__(TeamCfg<N>::TEAM) build_team_range_kernel(Team
   double* P = AL + N * M;
   double* w = P + N * M;
   for (int64_t jj = blockIdx.x; jj < a.T; jj += gridDim.x) {
+    if (uniform_near(a.cf.uni, a.t, j0 + jj, a.K)) continue;
     team_build_one<N, M>(lane, a.cf, a.t, j0 + jj, a.K, yb, ynb, ytb, kb, AL, P, w,
                          stages ? stages + jj * (int64_t)a.K * 4 * Rec<N>::SIZE : nullptr);
     if (a.out.A) {
@@ -252,6 +255,7 @@ __global__ void __launch_bounds__(TeamCfg<N>::TEAM, TeamCfg<N>::BUILD_MIN)
     const BatchProb& pb = bd.probs[b];
     const int64_t j = g - pb.off;
     if (j < pb.T) {
+      if (uniform_near(pb.cf.uni, pb.t, j, bd.K)) continue;
       team_build_one<N, M>(lane, pb.cf, pb.t, j, bd.K, yb, ynb, ytb, kb, AL, P, w);
     } else {
       const Rec<N> y = Rec<N>::packed(yb);
