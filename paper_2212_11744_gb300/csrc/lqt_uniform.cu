@@ -39,14 +39,15 @@ namespace lqt {
 
 static size_t ual(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Doubles of integrator state per step value: y and the RK4 sum (six n x n
-// blocks each), two buffers of the stage input's (A, J, E), AL, P, W.
+// Doubles of integrator state per step value: y, its low part and the RK4 sum
+// of the step (six n x n blocks each), two buffers of the stage input's (A, J,
+// E), AL, P, W.
 __host__ __device__ __forceinline__ int64_t uni_work_doubles(int n, int M) {
-  return 18 * (int64_t)n * n + 3 * (int64_t)n * M;
+  return 24 * (int64_t)n * n + 3 * (int64_t)n * M;
 }
 
 int64_t uniform_table_doubles(int n, int M) {
-  return kUniHeader + 18 * (int64_t)n * n + (n > 16 ? 3 * uni_work_doubles(n, M) : 0);
+  return kUniHeader + 24 * (int64_t)n * n + (n > 16 ? 3 * uni_work_doubles(n, M) : 0);
 }
 
 size_t uniform_table_bytes(int n, int M) { return ual((size_t)uniform_table_doubles(n, M) * sizeof(double)); }
@@ -90,6 +91,18 @@ __device__ __forceinline__ void tri_index(int e, int n, int& i, int& j) {
   j = i + e;
 }
 
+// (y, lo) += p + e exactly rounded to the pair (Knuth's two-sum): the element
+// serves every sub-interval, so a rounding of its RK4 sums would be the same
+// error in all of them and add up over the horizon, where the general build's
+// roundings differ from one sub-interval to the next.
+__device__ __forceinline__ void pair_add(double& y, double& lo, double p, double e) {
+  const double t = __dadd_rn(y, p), b = __dsub_rn(t, y);
+  const double err = __dadd_rn(__dsub_rn(y, __dsub_rn(t, b)), __dsub_rn(p, b));
+  const double l = __dadd_rn(lo, __dadd_rn(err, e));
+  y = __dadd_rn(t, l);
+  lo = __dsub_rn(l, __dsub_rn(y, t));
+}
+
 // One step value's integration: 256 threads of each CTA of the cluster own
 // entries of the six blocks (upper triangles of C, J, Z); two barriers per RK4
 // stage, before and after the entries that need AL, P, W of the stage input.
@@ -129,8 +142,9 @@ __global__ void __launch_bounds__(256) uniform_master_kernel(UniArgs a) {
   // F and Lt in shared memory; the state there too, or in the table's work area
   double* Fs = sm;
   double* Ls = Fs + nn;
-  double* y = kShared ? Ls + nM : tab + kUniHeader + 18 * (int64_t)nn + var * uni_work_doubles(n, M);
-  double* sum = y + 6 * nn;
+  double* y = kShared ? Ls + nM : tab + kUniHeader + 24 * (int64_t)nn + var * uni_work_doubles(n, M);
+  double* lo = y + 6 * nn;
+  double* sum = lo + 6 * nn;
   double* stg = sum + 6 * nn;  // two buffers of (A, J, E)
   double* AL = stg + 6 * nn;
   double* P = AL + nM;
@@ -140,12 +154,14 @@ __global__ void __launch_bounds__(256) uniform_master_kernel(UniArgs a) {
   for (int e = tid; e < 6 * nn; e += nth) {
     const double v = (e < nn && e % (n + 1) == 0) ? 1.0 : 0.0;
     y[e] = v;
-    sum[e] = v;
+    lo[e] = 0.0;
     if (e < 3 * nn) stg[e] = e < nn ? v : 0.0;
   }
   uni_sync(cl);
   const int tri = n * (n + 1) / 2;
   const int work = 3 * nn + 3 * tri;
+  // h / 6 to twice the precision
+  const double h6 = h / 6.0, h6l = fma(-6.0, h6, h) / 6.0;
   int cur = 0;
   for (int step = 0; step < 4 * K; ++step) {
     const int q = step & 3;
@@ -167,7 +183,6 @@ __global__ void __launch_bounds__(256) uniform_master_kernel(UniArgs a) {
       AL[e] = s;  // AL, P, W are contiguous
     }
     uni_sync(cl);
-    const double wk = -h * ((q == 0 || q == 3) ? 1.0 / 6.0 : 1.0 / 3.0);
     const double ak = -h * (q < 2 ? 0.5 : 1.0);
     for (int g = tid; g < work; g += nth) {
       int kind, i, j;
@@ -206,17 +221,20 @@ __global__ void __launch_bounds__(256) uniform_master_kernel(UniArgs a) {
       }
       const int e = kind * nn + i * n + j, et = kind * nn + j * n + i;
       const bool mirror = kind == 1 || kind == 2 || kind == 5;
-      const double ns = fma(wk, s, sum[e]);
-      sum[e] = ns;
       double nx;
       if (q == 3) {
-        y[e] = ns;
-        nx = ns;
+        const double k = -(sum[e] + s), p = h6 * k;
+        double ye = y[e], le = lo[e];
+        pair_add(ye, le, p, fma(h6, k, -p) + h6l * k);
+        nx = ye;
+        y[e] = ye;
+        lo[e] = le;
         if (mirror) {
-          y[et] = ns;
-          sum[et] = ns;
+          y[et] = ye;
+          lo[et] = le;
         }
       } else {
+        sum[e] = q == 0 ? s : fma(2.0, s, sum[e]);
         nx = fma(ak, s, y[e]);
       }
       // the next stage input's A, J, E
@@ -234,7 +252,9 @@ __global__ void __launch_bounds__(256) uniform_master_kernel(UniArgs a) {
   double* out = tab + kUniHeader + var * 6 * nn;
   for (int e = tid; e < 6 * nn; e += nth) {
     const int blk = e / nn, r = e - blk * nn, i = r / n, j = r - i * n;
-    out[e] = (blk == 3 || blk == 4) ? y[blk * nn + j * n + i] : y[e];
+    const int o = (blk == 3 || blk == 4) ? blk * nn + j * n + i : e;
+    out[e] = y[o];
+    if (var == 0) out[18 * nn + e] = lo[o];
   }
 }
 
@@ -291,6 +311,7 @@ __global__ void __launch_bounds__(256) uniform_expand_kernel(UniExpandArgs a) {
   const double* T0 = tab + kUniHeader;
   const double* Tp = T0 + 6 * NN;
   const double* Tm = Tp + 6 * NN;
+  const double* Tl = Tm + 6 * NN;  // low part of T0
   {
     constexpr int GR = NN >= 256 ? 1 : 256 / NN;  // threads that share an entry
     const int g = NN >= 256 ? 0 : tid / NN;
@@ -298,10 +319,10 @@ __global__ void __launch_bounds__(256) uniform_expand_kernel(UniExpandArgs a) {
 #pragma unroll
     for (int blk = 0; blk < 3; ++blk)
       for (int e = NN >= 256 ? tid : tid - g * NN; e < NN && g < GR; e += NN >= 256 ? 256 : NN) {
-        const double v = T0[blk * NN + e], d = Tp[blk * NN + e] - Tm[blk * NN + e];
+        const double v = T0[blk * NN + e], d = Tp[blk * NN + e] - Tm[blk * NN + e], l = Tl[blk * NN + e];
         double* o = dst[blk] + (off + j0) * NN + e;
         for (int k = g; k < cnt; k += GR)
-          if (near[k]) o[(int64_t)k * NN] = fma(cj[k], d, v);
+          if (near[k]) o[(int64_t)k * NN] = v + fma(cj[k], d, l);
       }
   }
   {
@@ -314,17 +335,17 @@ __global__ void __launch_bounds__(256) uniform_expand_kernel(UniExpandArgs a) {
       for (int r = 0; r < R; ++r) e[r] = b[r] = z[r] = 0.0;
       for (int c = 0; c < N; ++c) {
         const int o = c * N + i;
-        const double e0 = T0[3 * NN + o], de = Tp[3 * NN + o] - Tm[3 * NN + o];
-        const double b0 = T0[4 * NN + o], db = Tp[4 * NN + o] - Tm[4 * NN + o];
-        const double z0 = T0[5 * NN + o], dz = Tp[5 * NN + o] - Tm[5 * NN + o];
+        const double e0 = T0[3 * NN + o], de = Tp[3 * NN + o] - Tm[3 * NN + o], el = Tl[3 * NN + o];
+        const double b0 = T0[4 * NN + o], db = Tp[4 * NN + o] - Tm[4 * NN + o], bl = Tl[4 * NN + o];
+        const double z0 = T0[5 * NN + o], dz = Tp[5 * NN + o] - Tm[5 * NN + o], zl = Tl[5 * NN + o];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           const int k = g + r * GR;
           if (k < CH) {
             const double qc = qs[k * (N + 1) + c], w = cj[k];
-            e[r] = fma(fma(w, de, e0), qc, e[r]);
-            b[r] = fma(fma(w, db, b0), qc, b[r]);
-            z[r] = fma(fma(w, dz, z0), qc, z[r]);
+            e[r] = fma(e0 + fma(w, de, el), qc, e[r]);
+            b[r] = fma(b0 + fma(w, db, bl), qc, b[r]);
+            z[r] = fma(z0 + fma(w, dz, zl), qc, z[r]);
           }
         }
       }

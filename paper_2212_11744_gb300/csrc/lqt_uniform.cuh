@@ -8,7 +8,8 @@
 namespace lqt {
 
 // Table of one problem, in doubles: header (valid flag, step h, 1 / (h+ -
-// h-)), then A, C, J, E^T, Bq^T, Z (n x n each) at the steps h, h+, h-.
+// h-)), then A, C, J, E^T, Bq^T, Z (n x n each) at the steps h, h+, h-, then the
+// low parts of those at h.
 constexpr int kUniHeader = 16;
 constexpr double kUniStep = 1e-4;      // (h+- - h) / h
 constexpr double kUniNear = 1e-9;      // largest |h_j - h| / h served by the table
