@@ -153,6 +153,81 @@ __global__ void prepare_kernel(PrepArgs a) {
   }
 }
 
+// Lt and Ku of one (L, U) sample by a CTA of 128 threads (n <= 64): the
+// Cholesky factor in shared memory (R, kMaxM^2), its columns and updates over
+// the threads, then one thread per row of Lt (threads 0 .. 63) and per column
+// of Ku (64 .. 127).  The sums run in the order of prepare_kernel's.
+__device__ void prepare_sample_cta(int n, int m, int M, const double* __restrict__ L, const double* __restrict__ U,
+                                   double* __restrict__ Lt, double* __restrict__ Ku, double* R) {
+  const int tid = threadIdx.x;
+  for (int e = tid; e < m * m; e += blockDim.x) R[e] = U[e];
+  __syncthreads();
+  for (int j = 0; j < m; ++j) {
+    if (tid == 0) {
+      const double d = R[j * m + j];
+      if (!(d > 0.0)) flag(kStatusSingular);
+      R[j * m + j] = sqrt(d);
+    }
+    __syncthreads();
+    const double inv = 1.0 / R[j * m + j];
+    if (tid < j) R[tid * m + j] = 0.0;
+    if (tid > j && tid < m) R[tid * m + j] *= inv;
+    __syncthreads();
+    const int w = m - 1 - j;
+    for (int e = tid; e < w * w; e += blockDim.x) {
+      const int i = j + 1 + e / w, k = j + 1 + e % w;
+      if (k <= i) R[i * m + k] = fma(-R[i * m + j], R[k * m + j], R[i * m + k]);
+    }
+    __syncthreads();
+  }
+  if (tid < n) {  // Lt_i R^T = L_i
+    double row[kMaxM];
+#pragma unroll
+    for (int c = 0; c < kMaxM; ++c) {
+      row[c] = 0.0;
+      if (c < m) {
+        double v = L[tid * m + c];
+#pragma unroll
+        for (int k = 0; k < c; ++k) v = fma(-row[k], R[c * m + k], v);
+        row[c] = v / R[c * m + c];
+      }
+      if (c < M) Lt[tid * M + c] = row[c];
+    }
+  } else if (tid >= 64 && tid - 64 < n) {  // R y = L^T[:, col], R^T z = y
+    const int col = tid - 64;
+    double y[kMaxM];
+#pragma unroll
+    for (int i = 0; i < kMaxM; ++i) {
+      y[i] = 0.0;
+      if (i < m) {
+        double v = L[col * m + i];
+#pragma unroll
+        for (int k = 0; k < i; ++k) v = fma(-R[i * m + k], y[k], v);
+        y[i] = v / R[i * m + i];
+      }
+    }
+#pragma unroll
+    for (int i = kMaxM - 1; i >= 0; --i)
+      if (i < m) {
+        double v = y[i];
+#pragma unroll
+        for (int k = i + 1; k < kMaxM; ++k)
+          if (k < m) v = fma(-R[k * m + i], y[k], v);
+        y[i] = v / R[i * m + i];
+        Ku[i * n + col] = y[i];
+      }
+  }
+}
+
+// Constant L and U: their one sample by one CTA.  A thread alone took 21 us at
+// n = 4, m = 2, 163 us at n = 16, m = 8 and 1.49 ms at n = 64, m = 16, with the
+// rest of the GPU waiting.
+__global__ void __launch_bounds__(128) prepare_const_kernel(int n, int m, int M, const double* L, const double* U,
+                                                            double* Lt, double* Ku) {
+  __shared__ double R[kMaxM * kMaxM];
+  prepare_sample_cta(n, m, M, L, U, Lt, Ku, R);
+}
+
 // q = X r, rho = r^T X r per sample when H is the identity (one thread per
 // sample, loops unrolled for the compiled n).
 template <int N>
@@ -231,6 +306,35 @@ __global__ void __launch_bounds__(256) qr_rows_kernel(const double* __restrict__
   }
 }
 
+// The same with 64 threads per sample (N = 64), thread i forming row i of X r;
+// its row's lines stay in L1 over the row's 64 entries (one thread per sample:
+// 286 us at T = 4096).
+__global__ void __launch_bounds__(256) qr_rows64_kernel(const double* __restrict__ X, int32_t X_mode,
+                                                        const double* __restrict__ r, int32_t r_mode, int32_t dmode,
+                                                        int64_t cnt, int32_t K, int64_t T, double* __restrict__ qr) {
+  __shared__ double rs[4][64], part[8];
+  const int g = threadIdx.x >> 6, i = threadIdx.x & 63;
+  const int64_t s = (int64_t)blockIdx.x * 4 + g;
+  const bool live = s < cnt;
+  rs[g][i] = (live && r) ? r[input_index(r_mode, dmode, s, K, T) * 64 + i] : 0.0;
+  __syncthreads();
+  double q = 0.0;
+  if (live && r) {
+    const double* row = X + input_index(X_mode, dmode, s, K, T) * 4096 + i * 64;
+#pragma unroll 8
+    for (int l = 0; l < 64; ++l) q = fma(row[l], rs[g][l], q);
+  }
+  double rho = rs[g][i] * q;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) rho += __shfl_xor_sync(0xffffffffu, rho, o);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = rho;
+  __syncthreads();
+  if (live) {
+    qr[s * 65 + i] = q;
+    if (i == 0) qr[s * 65 + 64] = part[2 * g] + part[2 * g + 1];
+  }
+}
+
 template <int N>
 static void launch_qr_identity(const PrepArgs& a, cudaStream_t st) {
   const int threads = 256;
@@ -244,6 +348,9 @@ static void launch_qr_identity(const PrepArgs& a, cudaStream_t st) {
     else
       qr_rows_kernel<N, false><<<grid, threads, 0, st>>>(a.X.ptr, a.X.mode, a.r.ptr, a.r.mode, a.mode_qr, a.cnt_qr,
                                                           a.K, a.T, a.qr);
+  } else if constexpr (N == 64) {
+    qr_rows64_kernel<<<(unsigned)((a.cnt_qr + 3) / 4), threads, 0, st>>>(a.X.ptr, a.X.mode, a.r.ptr, a.r.mode,
+                                                                          a.mode_qr, a.cnt_qr, a.K, a.T, a.qr);
   } else {
     qr_identity_kernel<N><<<(unsigned)((a.cnt_qr + threads - 1) / threads), threads, 0, st>>>(
         a.X.ptr, a.X.mode, a.r.ptr, a.r.mode, a.mode_qr, a.cnt_qr, a.K, a.T, a.qr);
@@ -284,8 +391,10 @@ cudaError_t launch_prepare_into(const lqt_problem& p, const Layout& lay, double*
   const int threads = 128;
   const int64_t blocks = (most + threads - 1) / threads;
   if (h_identity) {
-    // which = 0 (Lt) and 3 (Ku): map blockIdx.y 0 -> 0, 1 -> 3
-    prepare_kernel<<<dim3((unsigned)blocks, 2), threads, 0, st>>>(a);
+    if (a.cnt_Lt == 1 && a.cnt_Ku == 1)
+      prepare_const_kernel<<<1, 128, 0, st>>>(a.n, a.m, a.M, a.L.ptr, a.U.ptr, a.Lt, a.Ku);
+    else  // which = 0 (Lt) and 3 (Ku): map blockIdx.y 0 -> 0, 1 -> 3
+      prepare_kernel<<<dim3((unsigned)blocks, 2), threads, 0, st>>>(a);
     count_launch();
     switch (p.n) {
       case 1: launch_qr_identity<1>(a, st); break;
@@ -582,62 +691,80 @@ __global__ void __launch_bounds__(128) build_stages_kernel(BuildArgs a, int64_t 
 }
 
 // Terminal element a_T: A = b = C = 0, J = Hf^T Xf Hf, eta = Hf^T Xf rf,
-// zeta = 1/2 rf^T Xf rf.  One thread per (i, j) entry of the n x n blocks.
-__device__ __forceinline__ double hf_at(const double* Hf, int k, int i, int n) {
-  return Hf ? Hf[k * n + i] : (k == i ? 1.0 : 0.0);
-}
-
+// zeta = 1/2 rf^T Xf rf.
 struct TermArgs {
   int32_t n, nr;
   const double *Hf, *Xf, *rf;
   double *A, *b, *C, *eta, *J, *zeta;  // the terminal record (any of A, b, C, zeta may be null)
 };
 
-__global__ void terminal_kernel(TermArgs a) {
-  const int n = a.n, nr = a.nr;
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n * n) return;
-  const int i = e / n, j = e % n;
-  double vij = 0.0, vji = 0.0;
-  for (int k = 0; k < nr; ++k) {
-    double xhj = 0.0, xhi = 0.0;
-    for (int l = 0; l < nr; ++l) {
-      xhj = fma(a.Xf[k * nr + l], hf_at(a.Hf, l, j, n), xhj);
-      xhi = fma(a.Xf[k * nr + l], hf_at(a.Hf, l, i, n), xhi);
+// One CTA: X_H = Xf Hf and Xf rf into shared memory, then J = sym(Hf' X_H), eta
+// = Hf' Xf rf, zeta (a thread per entry doing both sums was 0.97 ms at n = 64).
+__global__ void __launch_bounds__(256) terminal_kernel(TermArgs a) {
+  extern __shared__ double tsm[];
+  const int n = a.n, nr = a.nr, tid = threadIdx.x;
+  double* XH = tsm;              // nr x n
+  double* xr = XH + nr * n;      // nr
+  for (int e = tid; e < nr * n; e += 256) {
+    const int k = e / n, j = e % n;
+    double s = 0.0;
+    if (a.Hf) {
+      for (int l = 0; l < nr; ++l) s = fma(a.Xf[k * nr + l], a.Hf[l * n + j], s);
+    } else {
+      s = a.Xf[k * nr + j];
     }
-    vij = fma(hf_at(a.Hf, k, i, n), xhj, vij);
-    vji = fma(hf_at(a.Hf, k, j, n), xhi, vji);
+    XH[e] = s;
   }
-  a.J[e] = 0.5 * (vij + vji);
-  if (a.A) a.A[e] = 0.0;
-  if (a.C) a.C[e] = 0.0;
-  if (j == 0) {
+  for (int k = tid; k < nr; k += 256) {
+    double s = 0.0;
+    if (a.rf)
+      for (int l = 0; l < nr; ++l) s = fma(a.Xf[k * nr + l], a.rf[l], s);
+    xr[k] = s;
+  }
+  __syncthreads();
+  for (int e = tid; e < n * n; e += 256) {
+    const int i = e / n, j = e % n;
+    double vij = 0.0, vji = 0.0;
+    if (a.Hf) {
+      for (int k = 0; k < nr; ++k) {
+        vij = fma(a.Hf[k * n + i], XH[k * n + j], vij);
+        vji = fma(a.Hf[k * n + j], XH[k * n + i], vji);
+      }
+    } else {
+      vij = XH[i * n + j];
+      vji = XH[j * n + i];
+    }
+    a.J[e] = 0.5 * (vij + vji);
+    if (a.A) a.A[e] = 0.0;
+    if (a.C) a.C[e] = 0.0;
+  }
+  for (int i = tid; i < n; i += 256) {
     if (a.b) a.b[i] = 0.0;
     double et = 0.0;
-    if (a.rf)
-      for (int k = 0; k < nr; ++k) {
-        double xr = 0.0;
-        for (int l = 0; l < nr; ++l) xr = fma(a.Xf[k * nr + l], a.rf[l], xr);
-        et = fma(hf_at(a.Hf, k, i, n), xr, et);
-      }
+    if (a.Hf) {
+      for (int k = 0; k < nr; ++k) et = fma(a.Hf[k * n + i], xr[k], et);
+    } else {
+      et = xr[i];
+    }
     a.eta[i] = et;
   }
-  if (e == 0 && a.zeta) {
+  if (tid == 0 && a.zeta) {
     double rho = 0.0;
     if (a.rf)
-      for (int k = 0; k < nr; ++k) {
-        double xr = 0.0;
-        for (int l = 0; l < nr; ++l) xr = fma(a.Xf[k * nr + l], a.rf[l], xr);
-        rho = fma(a.rf[k], xr, rho);
-      }
+      for (int k = 0; k < nr; ++k) rho = fma(a.rf[k], xr[k], rho);
     *a.zeta = 0.5 * rho;
   }
 }
 
+static void launch_terminal(const TermArgs& t, cudaStream_t st) {
+  // nr <= 64, n <= 64: at most 33 KB
+  terminal_kernel<<<1, 256, ((size_t)t.nr * t.n + t.nr) * sizeof(double), st>>>(t);
+  count_launch();
+}
+
 cudaError_t launch_terminal_values(const lqt_problem& p, double* J, double* eta, double* zeta, cudaStream_t st) {
   TermArgs t{p.n, p.nr, p.Hf, p.Xf, p.rf, nullptr, nullptr, nullptr, eta, J, zeta};
-  terminal_kernel<<<(p.n * p.n + 255) / 256, 256, 0, st>>>(t);
-  count_launch();
+  launch_terminal(t, st);
   return cudaGetLastError();
 }
 
@@ -645,65 +772,38 @@ cudaError_t launch_terminal_values(const lqt_problem& p, double* J, double* eta,
 // batches: coefficient preparation and element build over the concatenation
 // ---------------------------------------------------------------------------
 
-// which = 0: Lt and Ku of every problem (constant L, U); which = 1: q = X r,
-// rho = r'Xr of every qr sample (X constant, H = identity).
-__global__ void batch_prepare_kernel(BatchDev bd, int which) {
+// Lt and Ku of every problem (constant L, U), one CTA each.
+__global__ void __launch_bounds__(128) batch_prepare_kernel(BatchDev bd) {
+  __shared__ double R[kMaxM * kMaxM];
+  const BatchProb& P = bd.probs[blockIdx.x];
+  prepare_sample_cta(bd.n, bd.m, bd.M, P.L, P.U, const_cast<double*>(P.cf.Lt.ptr), const_cast<double*>(P.cf.Ku), R);
+}
+
+// q = X r, rho = r'Xr of every qr sample (X constant, H = identity).
+__global__ void batch_qr_kernel(BatchDev bd) {
   const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int n = bd.n, m = bd.m;
-  if (which == 0) {
-    if (g >= bd.B) return;
-    const BatchProb& P = bd.probs[g];
-    double R[kMaxM * kMaxM];
-    for (int i = 0; i < m * m; ++i) R[i] = P.U[i];
-    cholesky_lower(R, m);
-    double* Lt = const_cast<double*>(P.cf.Lt.ptr);
-    for (int i = 0; i < n; ++i) {
-      double row[kMaxM];
-      for (int c = 0; c < m; ++c) {
-        double v = P.L[i * m + c];
-        for (int k = 0; k < c; ++k) v -= row[k] * R[c * m + k];
-        row[c] = v / R[c * m + c];
-      }
-      for (int c = 0; c < bd.M; ++c) Lt[i * bd.M + c] = c < m ? row[c] : 0.0;
-    }
-    double* Ku = const_cast<double*>(P.cf.Ku);
-    for (int col = 0; col < n; ++col) {
-      double y[kMaxM];
-      for (int i = 0; i < m; ++i) {
-        double v = P.L[col * m + i];
-        for (int k = 0; k < i; ++k) v -= R[i * m + k] * y[k];
-        y[i] = v / R[i * m + i];
-      }
-      for (int i = m - 1; i >= 0; --i) {
-        double v = y[i];
-        for (int k = i + 1; k < m; ++k) v -= R[k * m + i] * y[k];
-        y[i] = v / R[i * m + i];
-      }
-      for (int i = 0; i < m; ++i) Ku[i * n + col] = y[i];
-    }
-  } else {
-    if (g >= bd.total_qr) return;
-    const int32_t b = batch_find(bd.off_qr, bd.B, g);
-    const BatchProb& P = bd.probs[b];
-    const int64_t s = g - bd.off_qr[b];
-    const double* r = P.r ? P.r + (P.r_mode == kConst ? 0 : s) * n : nullptr;
-    double* out = const_cast<double*>(P.cf.qr.ptr) + s * (n + 1);
-    double rho = 0.0;
-    for (int i = 0; i < n; ++i) {
-      double v = 0.0;
-      if (r)
-        for (int l = 0; l < n; ++l) v = fma(P.X[i * n + l], r[l], v);
-      out[i] = v;
-      if (r) rho = fma(r[i], v, rho);
-    }
-    out[n] = rho;
+  const int n = bd.n;
+  if (g >= bd.total_qr) return;
+  const int32_t b = batch_find(bd.off_qr, bd.B, g);
+  const BatchProb& P = bd.probs[b];
+  const int64_t s = g - bd.off_qr[b];
+  const double* r = P.r ? P.r + (P.r_mode == kConst ? 0 : s) * n : nullptr;
+  double* out = const_cast<double*>(P.cf.qr.ptr) + s * (n + 1);
+  double rho = 0.0;
+  for (int i = 0; i < n; ++i) {
+    double v = 0.0;
+    if (r)
+      for (int l = 0; l < n; ++l) v = fma(P.X[i * n + l], r[l], v);
+    out[i] = v;
+    if (r) rho = fma(r[i], v, rho);
   }
+  out[n] = rho;
 }
 
 cudaError_t batch_prepare(const BatchDev& bd, cudaStream_t st) {
-  batch_prepare_kernel<<<(unsigned)((bd.B + 127) / 128), 128, 0, st>>>(bd, 0);
+  batch_prepare_kernel<<<(unsigned)bd.B, 128, 0, st>>>(bd);
   count_launch();
-  batch_prepare_kernel<<<(unsigned)((bd.total_qr + 127) / 128), 128, 0, st>>>(bd, 1);
+  batch_qr_kernel<<<(unsigned)((bd.total_qr + 127) / 128), 128, 0, st>>>(bd);
   count_launch();
   return cudaGetLastError();
 }
@@ -886,8 +986,7 @@ cudaError_t launch_terminal_element(const lqt_problem& p, const ElemPtrs& out, c
   const int n = p.n;
   TermArgs t{p.n, p.nr, p.Hf, p.Xf, p.rf, out.A + T * n * n, out.b + T * n, out.C + T * n * n,
              out.eta + T * n, out.J + T * n * n, out.zeta ? out.zeta + T : nullptr};
-  terminal_kernel<<<(n * n + 255) / 256, 256, 0, st>>>(t);
-  count_launch();
+  launch_terminal(t, st);
   return cudaGetLastError();
 }
 
