@@ -8,6 +8,8 @@
 // (forward-ODE elements, prefix scan, states) for n = 16 and 64, the
 // warp-per-element build of n = 4 and 8 at short horizons, and the warp-per-pair
 // upper scan levels of n = 4 and 8 (lqt_warp8.cuh).
+#include <algorithm>
+
 #include <cuda_runtime.h>
 
 #include "lqt_device.cuh"
@@ -16,6 +18,7 @@
 #include "lqt_team.cuh"
 #include "lqt_warp16.cuh"
 #include "lqt_warp8.cuh"
+#include "lqt_split64.cuh"
 
 namespace lqt {
 
@@ -348,17 +351,9 @@ __global__ void __launch_bounds__(TeamCfg<N>::TEAM) build_forward_team_kernel(Te
 // The FP32 products of the n = 64 combinations run on the tensor core.
 template <int N, typename GT>
 constexpr bool kTensorProducts = (N == 64 && std::is_same<GT, float>::value);
-// The FP64 n = 64 combinations keep their scratch (W, R = [K1 | MC1 | z0],
-// T1, vectors; 131 KB) in dynamic shared memory: the 64 dependent pivot steps
-// of the LU then wait on shared memory instead of L2.
+// The FP64 combinations of n = 64 run on split products (lqt_split64.cuh).
 template <int N, typename GT>
-constexpr bool kSharedScratch = (N == 64 && !kTensorProducts<N, GT>);
-// After the scratch: the A and C blocks of the element being combined, staged
-// by the TMA unit at level 0 (stage_ac).
-template <int N>
-constexpr size_t kReduceSmemBytes = sizeof(double) * (team::combine_scratch_doubles<N>() + 2 * N * N);
-template <int N>
-constexpr size_t kDownSmemBytes = sizeof(double) * (team::value_scratch_doubles<N>() + N * N + N + 2 * N * N);
+constexpr bool kSplit64 = (N == 64 && std::is_same<GT, double>::value);
 // The tensor-core instances: the operand tiles, then W, R and the vectors
 // (and the map Psi, alpha in the down-sweep); T1 stays in the slot.
 template <int N>
@@ -384,37 +379,12 @@ struct TeamScanArgs {
   int64_t T;
   double* gscratch;
   int zeta_inc;          // level 0 of a batch: zeta[k] receives the element's own share (see DownOut)
-  int bulk;              // FP64 n = 64, level 0: stage A, C of each element by TMA
 };
 
 template <int N>
 __device__ __forceinline__ Rec<N> level_elem(const TeamScanArgs& a, int64_t k, double* zero) {
   if (a.src) return Rec<N>::packed(const_cast<double*>(a.src) + k * Rec<N>::SIZE);
   return Rec<N>::pub(a.el, k, zero);
-}
-
-// Element k of the public arrays with its A and C blocks (N x N each, 32 KB at
-// n = 64) copied into shared memory sA, sC by the TMA unit (cp.async.bulk,
-// completion on the mbarrier `bar` with a bounded wait); every thread of the
-// CTA calls it after its last read of sA, sC.  The arrays must be 16-byte
-// aligned (bulk_ok).
-template <int N>
-__device__ __forceinline__ Rec<N> stage_ac(const ElemPtrs& el, int64_t k, double* sA, double* sC,
-                                           unsigned long long* bar, unsigned& phase, double* zero) {
-  constexpr unsigned kBytes = N * N * sizeof(double);
-  w16::fence_proxy_async();  // this thread's reads of sA, sC before the copies' writes
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    w16::mbar_expect_tx(bar, 2 * kBytes);
-    w16::bulk_g2s(sA, el.A + k * N * N, kBytes, bar);
-    w16::bulk_g2s(sC, el.C + k * N * N, kBytes, bar);
-  }
-  w16::mbar_wait_bounded(bar, phase);
-  phase ^= 1u;
-  Rec<N> e = Rec<N>::pub(el, k, zero);
-  e.a_ = sA;
-  e.c_ = sC;
-  return e;
 }
 
 template <int N, typename GT = double>
@@ -431,16 +401,6 @@ __global__ void __launch_bounds__(TeamCfg<N>::TEAM, TeamCfg<N>::SCAN_MIN) reduce
   double* bufB = bufA + Rec<N>::SIZE;
   double* scr = bufB + Rec<N>::SIZE;
   double* t1 = nullptr;
-  double *sA = nullptr, *sC = nullptr;
-  __shared__ unsigned long long st_bar;
-  unsigned st_phase = 0;
-  if constexpr (kSharedScratch<N, GT>) {
-    extern __shared__ __align__(16) double scr_smem[];
-    scr = scr_smem;
-    sA = scr + team::combine_scratch_doubles<N>();
-    sC = sA + N * N;
-    if (lane == 0) w16::mbar_init(&st_bar, 1);
-  }
   tc::Ctx* tcx = nullptr;
   tc::Ctx tc_ctx;
   if constexpr (kTensorProducts<N, GT>) {
@@ -460,10 +420,7 @@ __global__ void __launch_bounds__(TeamCfg<N>::TEAM, TeamCfg<N>::SCAN_MIN) reduce
     Rec<N> acc = Rec<N>::packed(bufA), nxt = Rec<N>::packed(bufB);
     team::copy_rec<N, TEAM>(lane, acc, level_elem<N>(a, last, &zero));
     for (int64_t k = last - 1; k >= first; --k) {
-      Rec<N> e1 = level_elem<N>(a, k, &zero);
-      if constexpr (kSharedScratch<N, GT>)
-        if (a.bulk) e1 = stage_ac<N>(a.el, k, sA, sC, &st_bar, st_phase, &zero);
-      team::combine<N, TEAM, GT>(lane, e1, acc, nxt, scr, fs, is, tcx, t1);
+      team::combine<N, TEAM, GT>(lane, level_elem<N>(a, k, &zero), acc, nxt, scr, fs, is, tcx, t1);
       const Rec<N> t = acc;
       acc = nxt;
       nxt = t;
@@ -495,20 +452,6 @@ __global__ void __launch_bounds__(TeamCfg<N>::TEAM, TeamCfg<N>::SCAN_MIN) down_t
   double* pv = P + N * N;
   double* Tm = pv + N;
   double* t1 = nullptr;
-  double *sA = nullptr, *sC = nullptr;
-  __shared__ unsigned long long st_bar;
-  unsigned st_phase = 0;
-  if constexpr (kSharedScratch<N, GT>) {
-    // the combination's scratch, its map (Psi, alpha) and the staged A, C in
-    // shared memory; the chunk composite (P, pv, Tm) stays in the slot
-    extern __shared__ __align__(16) double scr_smem[];
-    scr = scr_smem;
-    Psi = scr + team::value_scratch_doubles<N>();
-    alpha = Psi + N * N;
-    sA = alpha + N;
-    sC = sA + N * N;
-    if (lane == 0) w16::mbar_init(&st_bar, 1);
-  }
   tc::Ctx* tcx = nullptr;
   tc::Ctx tc_ctx;
   if constexpr (kTensorProducts<N, GT>) {
@@ -538,10 +481,7 @@ __global__ void __launch_bounds__(TeamCfg<N>::TEAM, TeamCfg<N>::SCAN_MIN) down_t
       }
     team::sync<TEAM>();
     for (int64_t k = last; k >= first; --k) {
-      Rec<N> e = level_elem<N>(a, k, &zero);
-      if constexpr (kSharedScratch<N, GT>)
-        if (a.bulk) e = stage_ac<N>(a.el, k, sA, sC, &st_bar, st_phase, &zero);
-      team::combine_value<N, TEAM, GT>(lane, e, carry, nv, Psi, alpha, scr, fs, is, &zinc, tcx, t1);
+      team::combine_value<N, TEAM, GT>(lane, level_elem<N>(a, k, &zero), carry, nv, Psi, alpha, scr, fs, is, &zinc, tcx, t1);
       if (Level0) {
         bool ok = true;
         for (int e = lane; e < VS; e += TEAM) {
@@ -571,30 +511,127 @@ __global__ void __launch_bounds__(TeamCfg<N>::TEAM, TeamCfg<N>::SCAN_MIN) down_t
   if constexpr (kTensorProducts<N, GT>) tc::release(tc_ctx);
 }
 
-// n = 16: one warp per combination with the register Gauss-Jordan solve and
-// TMA-staged element operands (lqt_warp16.cuh).  Same levels, groups and
-// records as the kernels above.
-constexpr int kW16ReduceSmem = 2 * w16::kRecPad + w16::kScratch;
-constexpr int kW16DownSmem = 2 * 276 + w16::kRecPad + w16::kVScratch + 256 + 16 + 256 + 16 + 16 * w16::kWld;
-
 __device__ __forceinline__ bool finite_bits(double x) {
   return (__double_as_longlong(x) & 0x7ff0000000000000ll) != 0x7ff0000000000000ll;
 }
 
+// n = 64 in FP64: one CTA per combination on split products; the running
+// records live in the CTA's workspace slot (L2).
+__global__ void __launch_bounds__(s64::kThreads, 1) reduce_s64_kernel(TeamScanArgs a) {
+  extern __shared__ __align__(16) unsigned char s64_smem[];
+  s64::Shared& sm = *reinterpret_cast<s64::Shared*>(s64_smem);
+  __shared__ double zero;
+  constexpr int N = 64, NT = s64::kThreads;
+  const int tid = threadIdx.x;
+  if (tid == 0) zero = 0.0;
+  __syncthreads();
+  double* base = slot_base<N>(a.gscratch, reduce_slot_doubles<N>());
+  const int64_t groups = tdiv(a.cnt, a.G);
+  for (int64_t g = blockIdx.x; g < groups; g += gridDim.x) {
+    const int64_t first = g * a.G;
+    const int64_t last = (first + a.G < a.cnt ? first + a.G : a.cnt) - 1;
+    Rec<N> acc = Rec<N>::packed(base), nxt = Rec<N>::packed(base + Rec<N>::SIZE);
+    team::copy_rec<N, NT>(tid, acc, level_elem<N>(a, last, &zero));
+    for (int64_t k = last - 1; k >= first; --k) {
+      s64::combine(sm, level_elem<N>(a, k, &zero), acc, nxt);
+      const Rec<N> t = acc;
+      acc = nxt;
+      nxt = t;
+    }
+    team::copy_rec<N, NT>(tid, Rec<N>::packed(a.agg + g * Rec<N>::SIZE), acc);
+  }
+}
+
+template <bool Level0>
+__global__ void __launch_bounds__(s64::kThreads, 1) down_s64_kernel(TeamScanArgs a) {
+  extern __shared__ __align__(16) unsigned char s64_smem[];
+  s64::Shared& sm = *reinterpret_cast<s64::Shared*>(s64_smem);
+  __shared__ double zero, zinc;
+  constexpr int N = 64, NT = s64::kThreads, VS = team::val_doubles<N>(), PM = N * N + N;
+  const int tid = threadIdx.x;
+  if (tid == 0) zero = 0.0;
+  __syncthreads();
+  double* c0 = slot_base<N>(a.gscratch, down_slot_doubles<N>());
+  double* c1 = c0 + VS;
+  double* P = c1 + VS;
+  double* pv = P + N * N;
+  const int64_t groups = tdiv(a.cnt, a.G);
+  for (int64_t g = blockIdx.x; g < groups; g += gridDim.x) {
+    const int64_t first = g * a.G;
+    const int64_t last = (first + a.G < a.cnt ? first + a.G : a.cnt) - 1;
+    double* carry = c0;
+    double* nv = c1;
+    for (int e = tid; e < VS; e += NT)
+      carry[e] = (a.above != nullptr && g + 1 < a.cnt_above) ? a.above[(g + 1) * VS + e] : 0.0;
+    if (Level0)
+      for (int e = tid; e < PM; e += NT) P[e] = (e < N * N && e % (N + 1) == 0) ? 1.0 : 0.0;  // P, then pv
+    __syncthreads();
+    for (int64_t k = last; k >= first; --k) {
+      s64::combine_value(sm, level_elem<N>(a, k, &zero), carry, nv, &zinc);
+      if (Level0) {
+        bool ok = true;
+        for (int e = tid; e < VS; e += NT) {
+          const double x = nv[e];
+          ok = ok && finite_bits(x);
+          if (e < N * N) a.S[k * N * N + e] = x;
+          else if (e < N * N + N) a.v[k * N + e - N * N] = x;
+          else if (a.zeta) a.zeta[k] = a.zeta_inc ? zinc : x;
+        }
+        if (!ok) flag(kStatusNonFinite);
+        if (a.maps != nullptr && k < a.T) {
+          for (int e = tid; e < PM; e += NT)
+            a.maps[k * PM + e] = e < N * N ? sm.K1[(e >> 6) * s64::kLd + (e & 63)] : sm.vec[4][e - N * N];
+          s64::compose_right(sm, P, pv);
+        }
+      } else {
+        for (int e = tid; e < VS; e += NT) a.vals[k * VS + e] = nv[e];
+      }
+      __syncthreads();
+      double* t = carry;
+      carry = nv;
+      nv = t;
+    }
+    if (Level0 && a.comp != nullptr && last + 1 <= a.T)
+      for (int e = tid; e < PM; e += NT) a.comp[g * PM + e] = P[e];
+    __syncthreads();
+  }
+}
+
+// n = 16: one warp per combination with the register Gauss-Jordan solve and
+// TMA-staged element operands (lqt_warp16.cuh).  Same levels, groups and
+// records as the kernels above.
 template <typename GT>
-__global__ void __launch_bounds__(32, 10) reduce_w16_kernel(TeamScanArgs a, int bulk) {
+constexpr bool kSplit16 = std::is_same<GT, double>::value;  // FP64: split products (lqt_split.cuh)
+template <typename GT>
+constexpr int kW16ReduceSmem = 2 * w16::kRecPad + (kSplit16<GT> ? w16::kSplitScratch : w16::kScratch);
+template <typename GT>
+constexpr int kW16DownSmem = 2 * 276 + w16::kRecPad + 256 + 16 + 256 + 16 +
+                             (kSplit16<GT> ? w16::kVSplitScratch : w16::kVScratch + 16 * w16::kWld);
+// CTAs per SM that the shared memory of each allows, and their warps: a split
+// combination is integer work in long dependent chains, and two warps on one
+// combination double the warps in flight for the same shared memory (one warp:
+// 64 k cycles a combination alone, 1960 cycles a product per sub-partition
+// with nine of them on an SM, against 810 with sixteen)
+template <typename GT>
+constexpr int kW16Ctas = kSplit16<GT> ? 8 : 10;
+template <typename GT>
+constexpr int kW16Nw = kSplit16<GT> ? 2 : 1;
+
+template <typename GT>
+__global__ void __launch_bounds__(32 * kW16Nw<GT>, kW16Ctas<GT>) reduce_w16_kernel(TeamScanArgs a, int bulk) {
   extern __shared__ __align__(16) double w16_smem[];
   __shared__ unsigned long long bar;
   __shared__ double zero;
-  const int lane = threadIdx.x;
+  constexpr int NW = kW16Nw<GT>, NT = 32 * NW;
+  const int tid = threadIdx.x;
   double* bufA = w16_smem;
   double* bufB = bufA + w16::kRecPad;
   double* scr = bufB + w16::kRecPad;
-  if (lane == 0) {
+  if (tid == 0) {
     zero = 0.0;
     w16::mbar_init(&bar, 1);
   }
-  __syncwarp();
+  split::sync16<NW>();
   unsigned phase = 0;
   const w16::ElemSrc src{a.el, a.src, bulk != 0};
   const int64_t groups = tdiv(a.cnt, a.G);
@@ -603,42 +640,45 @@ __global__ void __launch_bounds__(32, 10) reduce_w16_kernel(TeamScanArgs a, int 
     const int64_t last = (first + a.G < a.cnt ? first + a.G : a.cnt) - 1;
     double* acc = bufA;
     double* nxt = bufB;
-    w16::stage(lane, src, last, acc, &bar, phase, &zero);
+    w16::stage<NW>(tid, src, last, acc, &bar, phase, &zero);
     for (int64_t k = last - 1; k >= first; --k) {
-      w16::stage(lane, src, k, nxt, &bar, phase, &zero);
-      w16::combine<GT>(lane, nxt, acc, scr);
+      w16::stage<NW>(tid, src, k, nxt, &bar, phase, &zero);
+      if constexpr (kSplit16<GT>)
+        w16::combine_split<NW>(nxt, acc, scr);
+      else
+        w16::combine<GT>(tid, nxt, acc, scr);
       double* t = acc;
       acc = nxt;
       nxt = t;
     }
     double* out = a.agg + g * w16::kRec;
-    for (int e = lane; e < w16::kRec; e += 32) out[e] = acc[e];
-    __syncwarp();
+    for (int e = tid; e < w16::kRec; e += NT) out[e] = acc[e];
+    split::sync16<NW>();
   }
 }
 
 template <bool Level0, typename GT>
-__global__ void __launch_bounds__(32, 10) down_w16_kernel(TeamScanArgs a, int bulk) {
+__global__ void __launch_bounds__(32 * kW16Nw<GT>, kW16Ctas<GT>) down_w16_kernel(TeamScanArgs a, int bulk) {
   extern __shared__ __align__(16) double w16_smem[];
   __shared__ unsigned long long bar;
   __shared__ double zero;
   __shared__ double zinc;
+  constexpr int NW = kW16Nw<GT>, NT = 32 * NW;
   constexpr int VS = w16::kVal;
-  const int lane = threadIdx.x;
+  const int tid = threadIdx.x;
   double* c0 = w16_smem;
   double* c1 = c0 + 276;
   double* E = c1 + 276;
-  double* scr = E + w16::kRecPad;
-  double* Psi = scr + w16::kVScratch;
+  double* Psi = E + w16::kRecPad;
   double* alpha = Psi + 256;
   double* P = alpha + 16;
   double* pv = P + 256;
-  double* Tm = pv + 16;
-  if (lane == 0) {
+  double* scr = pv + 16;
+  if (tid == 0) {
     zero = 0.0;
     w16::mbar_init(&bar, 1);
   }
-  __syncwarp();
+  split::sync16<NW>();
   unsigned phase = 0;
   const w16::ElemSrc src{a.el, a.src, bulk != 0};
   const int64_t groups = tdiv(a.cnt, a.G);
@@ -647,19 +687,22 @@ __global__ void __launch_bounds__(32, 10) down_w16_kernel(TeamScanArgs a, int bu
     const int64_t last = (first + a.G < a.cnt ? first + a.G : a.cnt) - 1;
     double* carry = c0;
     double* nv = c1;
-    for (int e = lane; e < VS; e += 32)
+    for (int e = tid; e < VS; e += NT)
       carry[e] = (a.above != nullptr && g + 1 < a.cnt_above) ? a.above[(g + 1) * VS + e] : 0.0;
     if (Level0) {
-      for (int e = lane; e < 256; e += 32) P[e] = ((e >> 4) == (e & 15)) ? 1.0 : 0.0;
-      if (lane < 16) pv[lane] = 0.0;
+      for (int e = tid; e < 256; e += NT) P[e] = ((e >> 4) == (e & 15)) ? 1.0 : 0.0;
+      if (tid < 16) pv[tid] = 0.0;
     }
-    __syncwarp();
+    split::sync16<NW>();
     for (int64_t k = last; k >= first; --k) {
-      w16::stage(lane, src, k, E, &bar, phase, &zero);
-      w16::combine_value<GT>(lane, E, carry, nv, Psi, alpha, scr, &zinc);
+      w16::stage<NW>(tid, src, k, E, &bar, phase, &zero);
+      if constexpr (kSplit16<GT>)
+        w16::combine_value_split(E, carry, nv, Psi, alpha, scr, &zinc);
+      else
+        w16::combine_value<GT>(tid, E, carry, nv, Psi, alpha, scr, &zinc);
       if (Level0) {
         bool ok = true;
-        for (int e = lane; e < VS; e += 32) {
+        for (int e = tid; e < VS; e += NT) {
           const double x = nv[e];
           ok = ok && finite_bits(x);
           if (e < 256) a.S[k * 256 + e] = x;
@@ -668,20 +711,23 @@ __global__ void __launch_bounds__(32, 10) down_w16_kernel(TeamScanArgs a, int bu
         }
         if (!ok) flag(kStatusNonFinite);
         if (a.maps != nullptr && k < a.T) {
-          for (int e = lane; e < 272; e += 32) a.maps[k * 272 + e] = e < 256 ? Psi[e] : alpha[e - 256];
-          w16::compose_right(lane, P, pv, Psi, alpha, Tm);
+          for (int e = tid; e < 272; e += NT) a.maps[k * 272 + e] = e < 256 ? Psi[e] : alpha[e - 256];
+          if constexpr (kSplit16<GT>)
+            w16::compose_right_split(P, pv, Psi, alpha);
+          else
+            w16::compose_right(tid, P, pv, Psi, alpha, scr + w16::kVScratch);
         }
       } else {
-        for (int e = lane; e < VS; e += 32) a.vals[k * VS + e] = nv[e];
+        for (int e = tid; e < VS; e += NT) a.vals[k * VS + e] = nv[e];
       }
-      __syncwarp();
+      split::sync16<NW>();
       double* t = carry;
       carry = nv;
       nv = t;
     }
     if (Level0 && a.comp != nullptr && last + 1 <= a.T)
-      for (int e = lane; e < 272; e += 32) a.comp[g * 272 + e] = e < 256 ? P[e] : pv[e - 256];
-    __syncwarp();
+      for (int e = tid; e < 272; e += NT) a.comp[g * 272 + e] = e < 256 ? P[e] : pv[e - 256];
+    split::sync16<NW>();
   }
 }
 
@@ -816,13 +862,23 @@ __global__ void __launch_bounds__(TeamCfg<N>::TEAM) final_team_kernel(TeamFinalA
 // host side
 // ---------------------------------------------------------------------------
 
+// Level-0 chunk length: one chunk per resident team, so that the level is one
+// wave of equally long chunks (a power of two left a second, mostly empty wave:
+// at n = 64, T = 4096, 257 chunks of 16 on 152 slots took the time of 32
+// elements instead of 27), at most 32 elements.  The mixed path keeps its
+// power-of-two chunks: its results depend on the grouping to FP32 rounding.
 template <int N>
-static int team_group0(int64_t T) {
+static int team_group0(int64_t T, bool mixed) {
   if (scan_chunk_override() >= 2) return scan_chunk_override();
-  const int64_t want = TeamCfg<N>::SLOTS;  // chunks that keep every slot busy
-  int g = 2;
-  while (g < 32 && (T + 1) / (2 * g) >= want) g *= 2;
-  return g;
+  if (mixed) {
+    const int64_t want = TeamCfg<N>::SLOTS;
+    int g = 2;
+    while (g < 32 && (T + 1) / (2 * g) >= want) g *= 2;
+    return g;
+  }
+  const int64_t slots = N == 16 ? 152 * kW16Ctas<double> : TeamCfg<N>::SCAN_SLOTS;
+  const int64_t g = tdiv(T + 1, slots);
+  return g < 2 ? 2 : g > 32 ? 32 : (int)g;
 }
 
 template <int N>
@@ -840,9 +896,9 @@ struct TeamPlan {
 };
 
 template <int N>
-static TeamPlan<N> team_plan(int64_t T, bool with_traj) {
+static TeamPlan<N> team_plan(int64_t T, bool with_traj, bool mixed = false) {
   TeamPlan<N> pl{};
-  pl.G0 = team_group0<N>(T);
+  pl.G0 = team_group0<N>(T, mixed);
   size_t off = 0;
   const size_t PE = sizeof(double) * Rec<N>::SIZE;
   const size_t PV = sizeof(double) * team::val_doubles<N>();
@@ -905,16 +961,18 @@ static int bulk_ok(const ElemPtrs& el) {
 template <int N, typename GT>
 static void launch_reduce(const TeamScanArgs& a, int64_t groups, cudaStream_t st) {
   if constexpr (N == 16) {
-    reduce_w16_kernel<GT><<<(unsigned)(groups < TeamCfg<16>::SCAN_SLOTS ? (groups > 0 ? groups : 1)
-                                                                         : TeamCfg<16>::SCAN_SLOTS),
-                            32, kW16ReduceSmem * sizeof(double), st>>>(a, a.src == nullptr ? bulk_ok(a.el) : 0);
+    constexpr int64_t slots = 152 * kW16Ctas<GT>;
+    reduce_w16_kernel<GT><<<(unsigned)(groups < slots ? (groups > 0 ? groups : 1) : slots), 32 * kW16Nw<GT>,
+                            kW16ReduceSmem<GT> * sizeof(double), st>>>(a, a.src == nullptr ? bulk_ok(a.el) : 0);
     count_launch();
-  } else if constexpr (kTensorProducts<N, GT> || kSharedScratch<N, GT>) {
-    const size_t smem = kTensorProducts<N, GT> ? kTcReduceSmemBytes<N> : kReduceSmemBytes<N>;
-    TeamScanArgs b = a;
-    b.bulk = (kSharedScratch<N, GT> && a.src == nullptr) ? bulk_ok(a.el) : 0;
+  } else if constexpr (kSplit64<N, GT>) {
+    cudaFuncSetAttribute(reduce_s64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(s64::Shared));
+    reduce_s64_kernel<<<team_grid<N>(groups, TeamCfg<N>::SCAN_SLOTS), s64::kThreads, sizeof(s64::Shared), st>>>(a);
+    count_launch();
+  } else if constexpr (kTensorProducts<N, GT>) {
+    constexpr size_t smem = kTcReduceSmemBytes<N>;
     cudaFuncSetAttribute(reduce_team_kernel<N, GT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    reduce_team_kernel<N, GT><<<team_grid<N>(groups, TeamCfg<N>::SCAN_SLOTS), TeamCfg<N>::TEAM, smem, st>>>(b);
+    reduce_team_kernel<N, GT><<<team_grid<N>(groups, TeamCfg<N>::SCAN_SLOTS), TeamCfg<N>::TEAM, smem, st>>>(a);
     count_launch();
   } else {
     team_launch<N>(reduce_team_kernel<N, GT>, groups, reduce_slot_doubles<N>(), a, st, TeamCfg<N>::SCAN_SLOTS);
@@ -924,16 +982,20 @@ static void launch_reduce(const TeamScanArgs& a, int64_t groups, cudaStream_t st
 template <int N, bool Level0, typename GT>
 static void launch_down(const TeamScanArgs& a, int64_t groups, cudaStream_t st) {
   if constexpr (N == 16) {
-    down_w16_kernel<Level0, GT><<<(unsigned)(groups < TeamCfg<16>::SCAN_SLOTS ? (groups > 0 ? groups : 1)
-                                                                              : TeamCfg<16>::SCAN_SLOTS),
-                                  32, kW16DownSmem * sizeof(double), st>>>(a, a.src == nullptr ? bulk_ok(a.el) : 0);
+    constexpr int64_t slots = 152 * kW16Ctas<GT>;
+    down_w16_kernel<Level0, GT><<<(unsigned)(groups < slots ? (groups > 0 ? groups : 1) : slots), 32 * kW16Nw<GT>,
+                                  kW16DownSmem<GT> * sizeof(double), st>>>(a, a.src == nullptr ? bulk_ok(a.el) : 0);
     count_launch();
-  } else if constexpr (kTensorProducts<N, GT> || kSharedScratch<N, GT>) {
-    const size_t smem = kTensorProducts<N, GT> ? kTcDownSmemBytes<N> : kDownSmemBytes<N>;
-    TeamScanArgs b = a;
-    b.bulk = (kSharedScratch<N, GT> && a.src == nullptr) ? bulk_ok(a.el) : 0;
+  } else if constexpr (kSplit64<N, GT>) {
+    cudaFuncSetAttribute(down_s64_kernel<Level0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)sizeof(s64::Shared));
+    down_s64_kernel<Level0>
+        <<<team_grid<N>(groups, TeamCfg<N>::SCAN_SLOTS), s64::kThreads, sizeof(s64::Shared), st>>>(a);
+    count_launch();
+  } else if constexpr (kTensorProducts<N, GT>) {
+    constexpr size_t smem = kTcDownSmemBytes<N>;
     cudaFuncSetAttribute(down_team_kernel<N, Level0, GT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    down_team_kernel<N, Level0, GT><<<team_grid<N>(groups, TeamCfg<N>::SCAN_SLOTS), TeamCfg<N>::TEAM, smem, st>>>(b);
+    down_team_kernel<N, Level0, GT><<<team_grid<N>(groups, TeamCfg<N>::SCAN_SLOTS), TeamCfg<N>::TEAM, smem, st>>>(a);
     count_launch();
   } else {
     team_launch<N>(down_team_kernel<N, Level0, GT>, groups, down_slot_doubles<N>(), a, st, TeamCfg<N>::SCAN_SLOTS);
@@ -952,7 +1014,7 @@ template <int N, typename GT>
 static cudaError_t team_run_g(const lqt_problem& p, const Coefs& cf, const ElemPtrs& el, double* S, double* v,
                             double* zeta, const double* x0, double* x, double* u, double* cost, bool do_value,
                             bool do_traj, char* ws, cudaStream_t st) {
-  const TeamPlan<N> pl = team_plan<N>(p.T, do_traj);
+  const TeamPlan<N> pl = team_plan<N>(p.T, do_traj, std::is_same<GT, float>::value);
   double* gs = TeamCfg<N>::SMEM ? nullptr : (double*)(ws + pl.off_scratch);
   double* maps0 = (double*)(ws + pl.off_maps);
   double* comp1 = pl.tlev > 0 ? (double*)(ws + pl.off_tmap[0]) : nullptr;
@@ -1185,7 +1247,7 @@ struct TeamM2Args {
 template <int N>
 constexpr int m2_rec_doubles() { return N == 16 ? w16::kRecPad : Rec<N>::SIZE; }
 template <int N>
-constexpr int m2_scratch_doubles() { return N == 16 ? w16::kScratch : team::combine_scratch_doubles<N>(); }
+constexpr int m2_scratch_doubles() { return N == 16 ? w16::kSplitScratch : team::combine_scratch_doubles<N>(); }
 template <int N>
 constexpr int m2_slot_doubles() { return 2 * m2_rec_doubles<N>() + m2_scratch_doubles<N>() + N * N + 2 * N + 8; }
 
@@ -1273,7 +1335,7 @@ __global__ void __launch_bounds__(TeamCfg<N>::TEAM) method2_team_kernel(TeamM2Ar
       m2_state<N, TEAM>(lane, a, k, P, W, r, ev, fs, is);
       if constexpr (N == 16) {
         w16::stage(lane, w16::ElemSrc{a.el, nullptr, a.bulk != 0}, k, Pn, &bar, phase, &zero);
-        w16::combine<double>(lane, P, Pn, scr);
+        w16::combine_split<1>(P, Pn, scr);
       } else {
         team::combine<N, TEAM>(lane, Rec<N>::packed(P), Rec<N>::pub(a.el, k, &zero), Rec<N>::packed(Pn), scr, fs,
                                is);
@@ -1309,7 +1371,7 @@ struct TeamPrefixPlan {
 template <int N>
 static TeamPrefixPlan<N> team_prefix_plan(int64_t T) {
   TeamPrefixPlan<N> pl{};
-  pl.G0 = team_group0<N>(T - 1);
+  pl.G0 = team_group0<N>(T - 1, false);
   const size_t PE = sizeof(double) * Rec<N>::SIZE;
   size_t off = 0;
   int64_t c = T;
@@ -1704,8 +1766,9 @@ cudaError_t team_launch_build_small(const lqt_problem& p, const Layout& lay, con
 
 size_t team_scan_workspace_bytes(int32_t n, int64_t T, bool with_traj) {
   switch (n) {
-    case 16: return team_plan<16>(T, with_traj).bytes;
-    case 64: return team_plan<64>(T, with_traj).bytes;
+    // lqt_solve and lqt_solve_mixed share one size
+    case 16: return std::max(team_plan<16>(T, with_traj).bytes, team_plan<16>(T, with_traj, true).bytes);
+    case 64: return std::max(team_plan<64>(T, with_traj).bytes, team_plan<64>(T, with_traj, true).bytes);
     default: return 0;
   }
 }

@@ -23,6 +23,7 @@
 
 #include "lqt_device.cuh"
 #include "lqt_internal.h"
+#include "lqt_split.cuh"
 
 namespace lqt {
 namespace w16 {
@@ -102,15 +103,17 @@ struct ElemSrc {
   bool bulk;           // public arrays 16-byte aligned: stage by TMA
 };
 
-// Stages element k into the shared record `dst` (kRec doubles).  The whole warp
-// calls it; on return (after a __syncwarp) the record is complete.  `bar` is
-// this warp's mbarrier and `phase` its parity, flipped per use.
-__device__ __forceinline__ void stage(int lane, const ElemSrc& s, int64_t k, double* dst, unsigned long long* bar,
+// Stages element k into the shared record `dst` (kRec doubles).  The warp, or
+// the CTA of NW warps, calls it with its thread index; on return the record is
+// complete.  `bar` is its mbarrier and `phase` its parity, flipped per use.
+template <int NW = 1>
+__device__ __forceinline__ void stage(int tid, const ElemSrc& s, int64_t k, double* dst, unsigned long long* bar,
                                       unsigned& phase, const double* zero_zeta) {
+  constexpr int NT = 32 * NW;
   if (s.rec == nullptr && s.bulk) {
-    fence_proxy_async();  // this lane's earlier reads of dst before the copy's writes
-    __syncwarp();
-    if (lane == 0) {
+    fence_proxy_async();  // this thread's earlier reads of dst before the copy's writes
+    split::sync16<NW>();
+    if (tid == 0) {
       mbar_expect_tx(bar, (3 * 256 + 2 * 16) * 8);
       bulk_g2s(dst + kOffA, s.el.A + k * 256, 256 * 8, bar);
       bulk_g2s(dst + kOffB, s.el.b + k * 16, 16 * 8, bar);
@@ -122,21 +125,21 @@ __device__ __forceinline__ void stage(int lane, const ElemSrc& s, int64_t k, dou
     mbar_wait_bounded(bar, phase);
     phase ^= 1u;
   } else if (s.rec == nullptr) {
-    for (int e = lane; e < 256; e += 32) {
+    for (int e = tid; e < 256; e += NT) {
       dst[kOffA + e] = s.el.A[k * 256 + e];
       dst[kOffC + e] = s.el.C[k * 256 + e];
       dst[kOffJ + e] = s.el.J[k * 256 + e];
     }
-    if (lane < 16) {
-      dst[kOffB + lane] = s.el.b[k * 16 + lane];
-      dst[kOffEta + lane] = s.el.eta[k * 16 + lane];
+    if (tid < 16) {
+      dst[kOffB + tid] = s.el.b[k * 16 + tid];
+      dst[kOffEta + tid] = s.el.eta[k * 16 + tid];
     }
-    if (lane == 0) dst[kOffZeta] = s.el.zeta ? s.el.zeta[k] : *zero_zeta;
+    if (tid == 0) dst[kOffZeta] = s.el.zeta ? s.el.zeta[k] : *zero_zeta;
   } else {
     const double* r = s.rec + k * kRec;
-    for (int e = lane; e < kRec; e += 32) dst[e] = r[e];
+    for (int e = tid; e < kRec; e += NT) dst[e] = r[e];
   }
-  __syncwarp();
+  split::sync16<NW>();
 }
 
 // ---------------------------------------------------------------------------
@@ -472,6 +475,407 @@ __device__ __forceinline__ void compose_right(int lane, double* P, double* p, co
   for (int q = lane; q < 256; q += 32) P[q] = Tm[(q >> 4) * kWld + (q & 15)];
   if (lane < 16) p[lane] = pa;
   __syncwarp();
+}
+
+// ---------------------------------------------------------------------------
+// the FP64 combinations: split products (lqt_split.cuh) and an inverse
+// ---------------------------------------------------------------------------
+//
+// What bounds a combination is the FP64 pipe, at 64 cycles a warp
+// instruction: five to six 16^3 products took 128 instructions each and the
+// elimination of 2 n + 1 right-hand sides 530.  The products now run on the
+// tensor core (about 800 cycles of a sub-partition each, integer work, against
+// 8192), and W is inverted instead of eliminated: a Gauss-Jordan inverse in
+// FP32 and Newton steps M <- M - M (W M - I), whose residual the split product
+// forms to 2^-57 of |W| |M|.  A residual below 2^-28 makes the step that
+// follows exact to FP64 rounding, so M is as accurate as its own rounding.
+// Where an FP32 pivot falls below 2^-10 of its row or the residual does not
+// shrink (cond(W) beyond some 1e5), the inverse is made in FP64 with the
+// pivots and the SINGULAR test of gauss_jordan, and the Newton step polishes
+// that one.
+
+// x[k], k = 0..7, without indexing a local array.
+template <typename X>
+__device__ __forceinline__ X pick8(const X (&x)[8], int k) {
+  const X a = (k & 1) ? x[1] : x[0], b = (k & 1) ? x[3] : x[2], c = (k & 1) ? x[5] : x[4], d = (k & 1) ? x[7] : x[6];
+  const X e = (k & 2) ? b : a, f = (k & 2) ? d : c;
+  return (k & 4) ? f : e;
+}
+
+// The FP32 inverse: layout as invert16 below; scale: the largest magnitude of
+// row (lane & 15), at least 1.  False when a pivot is not safely away from 0.
+__device__ __forceinline__ bool invert16_f32(int lane, float (&m)[8], float scale, int& perm) {
+  const int j = lane & 15, h = lane >> 4;
+  perm = j;
+  bool ok = true;
+#pragma unroll 1
+  for (int k = 0; k < 16; ++k) {
+    // largest magnitude of column k below the diagonal, to 2^-19, with its row
+    unsigned best = 0;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const unsigned key = (__float_as_uint(m[r]) & 0x7ffffff0u) | (unsigned)(15 - 8 * h - r);
+      best = (8 * h + r >= k) ? max(best, key) : best;
+    }
+    best = max(__shfl_sync(kFull, best, k), __shfl_sync(kFull, best, k + 16));
+    const int p = 15 - (int)(best & 15u);
+    const float sk = __shfl_sync(kFull, scale, k), sp = __shfl_sync(kFull, scale, p);
+    const int pk = __shfl_sync(kFull, perm, k), pp = __shfl_sync(kFull, perm, p);
+    scale = j == k ? sp : (j == p ? sk : scale);
+    perm = j == k ? pp : (j == p ? pk : perm);
+    const float vk = __shfl_sync(kFull, pick8(m, k & 7), j + 16 * (k >> 3));
+    const float vp = __shfl_sync(kFull, pick8(m, p & 7), j + 16 * (p >> 3));
+    const float d = __shfl_sync(kFull, vp, k);
+    ok = ok && fabsf(d) > 0x1p-10f * sp && fabsf(d) < 0x1p100f;
+    const float pr = (j == k ? 1.0f : vp) * __frcp_rn(d);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) m[r] = (8 * h + r == p) ? vk : m[r];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const float f = __shfl_sync(kFull, m[r], k + 16 * h);
+      const float v = fmaf(-f, pr, j == k ? 0.0f : m[r]);
+      m[r] = (8 * h + r == k) ? pr : v;
+    }
+  }
+  return ok;
+}
+
+// Inverse of W in place with partial pivoting: lane (j = lane & 15, h = lane
+// >> 4) holds rows 8h .. 8h + 7 of column j in m; rk as in gauss_jordan.  On
+// return m holds column j of (P W)^-1, which is column perm of W^-1.  Pivots
+// as in gauss_jordan (the same rows, the same SINGULAR test).
+__device__ __forceinline__ int invert16(int lane, double (&m)[8], unsigned long long rk) {
+  const int j = lane & 15, h = lane >> 4;
+  int perm = j;
+#pragma unroll 1
+  for (int k = 0; k < 16; ++k) {
+    unsigned long long best = 0;
+    int p = k;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const unsigned long long key = (8 * h + r >= k) ? mag_key(m[r]) : 0ull;
+      if (key > best) {
+        best = key;
+        p = 8 * h + r;
+      }
+    }
+    {
+      const unsigned long long ob = __shfl_xor_sync(kFull, best, 16);
+      const int op = __shfl_xor_sync(kFull, p, 16);
+      if (ob > best || (ob == best && op < p)) {
+        best = ob;
+        p = op;
+      }
+    }
+    p = __shfl_sync(kFull, p, k);
+    best = __shfl_sync(kFull, best, k);
+    const unsigned long long rk_k = __shfl_sync(kFull, rk, k), rk_p = __shfl_sync(kFull, rk, p);
+    const int pm_k = __shfl_sync(kFull, perm, k), pm_p = __shfl_sync(kFull, perm, p);
+    if (j == k) {
+      rk = rk_p;
+      perm = pm_p;
+    } else if (j == p) {
+      rk = rk_k;
+      perm = pm_k;
+    }
+    if (lane == 0 && pivot_too_small(__longlong_as_double((long long)best), rk_p)) flag(kStatusSingular);
+    // exchange rows k and p
+    const double mk = pick8(m, k & 7), mp = pick8(m, p & 7);
+    const double vk = __shfl_sync(kFull, mk, j + 16 * (k >> 3));
+    const double vp = __shfl_sync(kFull, mp, j + 16 * (p >> 3));
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const double x = (8 * h + r == p) ? vk : m[r];
+      m[r] = (8 * h + r == k) ? vp : x;
+    }
+    const double inv = 1.0 / __shfl_sync(kFull, vp, k);
+    const double pr = (j == k ? 1.0 : vp) * inv;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const double f = __shfl_sync(kFull, m[r], k + 16 * h);
+      const double v = fma(-f, pr, j == k ? 0.0 : m[r]);
+      m[r] = (8 * h + r == k) ? pr : v;
+    }
+  }
+  return perm;
+}
+
+// Offset of a shared-memory buffer from the CTA's dynamic shared memory.
+__device__ __forceinline__ int sm_off(const double* p) {
+  extern __shared__ __align__(16) double split_smem[];
+  return (int)(p - split_smem);
+}
+// Rows (kWld or 16 doubles apart) of a buffer as vectors, and its columns.
+__device__ __forceinline__ split::Mat16 rows_of(const double* p, int ld) { return {sm_off(p), ld, 1}; }
+__device__ __forceinline__ split::Mat16 cols_of(const double* p, int ld) { return {sm_off(p), 1, ld}; }
+
+// Minv (row stride kWld) <- W^-1 by the elimination in FP64.
+static __device__ __noinline__ void inverse_f64(const double* W, double* Minv) {
+  const int lane = threadIdx.x & 31, j = lane & 15, i0 = 8 * (lane >> 4);
+  double m[8];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) m[r] = W[(i0 + r) * kWld + j];
+  const int perm = invert16(lane, m, row_scale(lane, W));
+#pragma unroll
+  for (int r = 0; r < 8; ++r) Minv[(i0 + r) * kWld + perm] = m[r];
+  __syncwarp();
+}
+
+// Minv <- the FP32 inverse of W, by one warp; false: see invert16_f32.
+__device__ __forceinline__ bool inverse_f32(int lane, const double* W, double* Minv) {
+  const int j = lane & 15, i0 = 8 * (lane >> 4);
+  float m[8];
+  float s = 1.0f;
+#pragma unroll
+  for (int r = 0; r < 8; ++r) s = fmaxf(s, fabsf((float)W[j * kWld + i0 + r]));
+  s = fmaxf(s, __shfl_xor_sync(kFull, s, 16));
+#pragma unroll
+  for (int r = 0; r < 8; ++r) m[r] = (float)W[(i0 + r) * kWld + j];
+  int perm;
+  const bool ok = invert16_f32(lane, m, s, perm);
+#pragma unroll
+  for (int r = 0; r < 8; ++r) Minv[(i0 + r) * kWld + perm] = (double)m[r];
+  __syncwarp();
+  return ok;
+}
+
+// Newton steps on Minv (row stride kWld), which holds the FP32 inverse of W
+// (row stride kWld) when `fast` (the same in every thread); E (row stride ld)
+// is scratch.
+template <int NW>
+__device__ __forceinline__ void refine_inverse(const double* W, double* Minv, double* E, int ld, bool fast) {
+  constexpr int kExp1 = 1023;  // biased exponent of 1
+  // at most four steps: |W M - I| < 2^-28 (row sum) before the last one
+  int last = kExp1 - 1;
+  for (int it = 0; it < 4; ++it) {
+    if (!fast) {
+      if (NW == 1 || threadIdx.x < 32) inverse_f64(W, Minv);
+      split::sync16<NW>();
+    }
+    const int top = split::product16<NW>(rows_of(W, kWld), cols_of(Minv, kWld), rows_of(E, ld), -1, split::kSet);
+    // the residual must fall at least eightfold per step, from below 1/16
+    bool done = top <= kExp1 - 32, lost = top > last - 3 || top > kExp1 - 5;
+    if constexpr (NW > 1) {
+      done = __syncthreads_and(done) != 0;
+      lost = __syncthreads_or(lost) != 0;
+    }
+    done = done || !fast;
+    if (!done && (lost || it == 3)) {
+      fast = false;  // not converging: the FP64 inverse, then its one step
+      it = 2;
+      continue;
+    }
+    last = top;
+    split::product16<NW>(rows_of(Minv, kWld), cols_of(E, ld), rows_of(Minv, kWld), 0, split::kSubtract);
+    if (done) break;
+  }
+}
+
+// x = W^-1 r from M = W^-1, r and x in shared memory (r is overwritten), one
+// warp: x = M r and one step of refinement, so that W x - r is of the size an
+// elimination leaves (x = M r alone leaves up to cond(W) times that, which the
+// zeta and eta terms, made from J2 x - eta2 with its cancellation, would feel).
+__device__ __forceinline__ void solve_refined(int lane, const double* W, const double* Minv, double* r, double* x) {
+  const int i = lane & 15, h = lane >> 4;
+  const double x0 = matvec<double>(lane, [&](int a, int l) { return Minv[a * kWld + l]; }, [&](int l) { return r[l]; },
+                                   0.0);
+  if (h == 0) x[i] = x0;
+  __syncwarp();
+  const double d = matvec<double>(lane, [&](int a, int l) { return -W[a * kWld + l]; }, [&](int l) { return x[l]; },
+                                  r[i]);
+  __syncwarp();
+  if (h == 0) r[i] = d;
+  __syncwarp();
+  const double x1 = matvec<double>(lane, [&](int a, int l) { return Minv[a * kWld + l]; }, [&](int l) { return r[l]; },
+                                   x0);
+  __syncwarp();
+  if (h == 0) x[i] = x1;
+  __syncwarp();
+}
+
+// Scratch of combine_split(): four 16 x 17 buffers and vectors.
+constexpr int kSplitBuf = 16 * kWld;
+constexpr int kSplitScratch = 4 * kSplitBuf + 6 * 16;
+
+// e1 <- e1 (x) e2 in place, FP64 (both full records in shared memory), by one
+// warp or a CTA of two: the second warp takes products that do not wait for
+// the inverse or for the vectors, and eight columns of the others.
+template <int NW>
+__device__ inline void combine_split(double* e1, const double* e2, double* scr) {
+  using split::kSet;
+  using split::product16;
+  using split::sync16;
+  double* W = scr;               // W, then M C1, then A2 M C1 A2^T
+  double* Mi = W + kSplitBuf;    // M = W^-1
+  double* T1 = Mi + kSplitBuf;   // J2 A1, then K1^T J2 A1
+  double* K1 = T1 + kSplitBuf;   // the Newton residual, K1 = M A1, A2 M C1
+  double* z0 = K1 + kSplitBuf;
+  double* J2z = z0 + 16;
+  double* l0 = J2z + 16;
+  double* wv = l0 + 16;
+  double* rr = wv + 16;
+  int* fast = reinterpret_cast<int*>(rr + 16);
+  const double* A1 = e1 + kOffA;
+  const double* C1 = e1 + kOffC;
+  const double* b1 = e1 + kOffB;
+  const double* A2 = e2 + kOffA;
+  const double* C2 = e2 + kOffC;
+  const double* J2 = e2 + kOffJ;
+  const double* b2 = e2 + kOffB;
+  const double* eta2 = e2 + kOffEta;
+  const int tid = NW == 1 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
+  const int lane = tid & 31, i = lane & 15, h = lane >> 4;
+  const bool first = NW == 1 || tid < 32, second = NW == 1 || tid >= 32;
+  // W = I + C1 J2, T1 = J2 A1 (C1, J2 symmetric: their rows are their columns)
+  product16<NW>(rows_of(C1, 16), rows_of(J2, 16), rows_of(W, kWld), 1, kSet);
+  if (first) {
+    const bool ok = inverse_f32(lane, W, Mi);
+    if (lane == 0) *fast = ok ? 1 : 0;
+  }
+  if (second) {
+    product16<1>(rows_of(J2, 16), cols_of(A1, 16), rows_of(T1, kWld), 0, kSet);
+    const double rv = matvec<double>(lane, [&](int r, int l) { return C1[l * 16 + r]; },
+                                     [&](int l) { return eta2[l]; }, b1[i]);
+    const double w = matvec<double>(lane, [&](int r, int l) { return -J2[l * 16 + r]; }, [&](int l) { return b1[l]; },
+                                    eta2[i]);
+    if (h == 0) {
+      wv[i] = w;
+      rr[i] = rv;
+    }
+  }
+  sync16<NW>();
+  refine_inverse<NW>(W, Mi, K1, kWld, *fast != 0);
+  product16<NW>(rows_of(Mi, kWld), cols_of(A1, 16), rows_of(K1, kWld), 0, kSet);
+  double bo = 0.0, zs = 0.0, et = 0.0;
+  if (first) {
+    // z0 = M (b1 + C1 eta2), l0 = J2 z0 - eta2 ; zeta ; b = A2 z0 + b2
+    solve_refined(lane, W, Mi, rr, z0);
+    const double jz = matvec<double>(lane, [&](int r, int l) { return J2[l * 16 + r]; }, [&](int l) { return z0[l]; },
+                                     0.0);
+    if (h == 0) {
+      J2z[i] = jz;
+      l0[i] = jz - eta2[i];
+    }
+    bo = matvec<double>(lane, [&](int r, int l) { return A2[r * 16 + l]; }, [&](int l) { return z0[l]; }, b2[i]);
+    __syncwarp();
+    const double cl = matvec<double>(lane, [&](int r, int l) { return C1[l * 16 + r]; }, [&](int l) { return l0[l]; },
+                                     0.0);
+    const double zt = (h == 0) ? fma(0.5 * l0[i], cl, z0[i] * fma(0.5, J2z[i], -eta2[i])) : 0.0;
+    zs = warp_sum(zt);
+  }
+  if (second) {
+    // eta = K1^T wv + eta1 ; K1^T T1 ; A = A2 K1 (A1 was consumed by T1, K1)
+    et = matvec<double>(lane, [&](int r, int l) { return K1[l * kWld + r]; }, [&](int l) { return wv[l]; },
+                        e1[kOffEta + i]);
+    product16<1>(cols_of(K1, kWld), cols_of(T1, kWld), rows_of(T1, kWld), 0, kSet);
+    product16<1>(rows_of(A2, 16), cols_of(K1, kWld), rows_of(e1 + kOffA, 16), 0, kSet);
+  }
+  sync16<NW>();
+  if (first) {
+    if (h == 0) e1[kOffB + i] = bo;
+    if (lane == 0) e1[kOffZeta] = e1[kOffZeta] + e2[kOffZeta] + zs;
+  }
+  if (second && h == 0) e1[kOffEta + i] = et;
+  // C = A2 (M C1) A2^T + C2
+  product16<NW>(rows_of(Mi, kWld), rows_of(C1, 16), rows_of(W, kWld), 0, kSet);
+  product16<NW>(rows_of(A2, 16), cols_of(W, kWld), rows_of(K1, kWld), 0, kSet);
+  product16<NW>(rows_of(K1, kWld), rows_of(A2, 16), rows_of(W, kWld), 0, kSet);
+  // symmetric by taking the upper triangle
+  for (int e = tid; e < 256; e += 32 * NW) {
+    const int r = e >> 4, c = e & 15;
+    const int o = r < c ? r * kWld + c : c * kWld + r;
+    e1[kOffJ + e] += T1[o];
+    e1[kOffC + e] = C2[e] + W[o];
+  }
+  sync16<NW>();
+}
+
+// Scratch of combine_value_split(): three 16 x 17 buffers and vectors.
+constexpr int kVSplitScratch = 3 * kSplitBuf + 5 * 16;
+
+// combine_value() in FP64 with split products, by a CTA of two warps.
+__device__ inline void combine_value_split(const double* e, const double* V, double* out, double* Psi, double* alpha,
+                                           double* scr, double* zeta_inc) {
+  constexpr int NW = 2;
+  using split::kSet;
+  using split::product16;
+  double* W = scr;
+  double* T1 = W + kSplitBuf;  // S2 A, then Psi^T S2 A
+  double* Mi = T1 + kSplitBuf;
+  double* wv = Mi + kSplitBuf;
+  double* Sz = wv + 16;
+  double* l0 = Sz + 16;
+  double* rr = l0 + 16;
+  int* fast = reinterpret_cast<int*>(rr + 16);
+  const double* A = e + kOffA;
+  const double* C = e + kOffC;
+  const double* b = e + kOffB;
+  const double* S2 = V;
+  const double* v2 = V + 256;
+  const int tid = threadIdx.x, lane = tid & 31, i = lane & 15, h = lane >> 4;
+  product16<NW>(rows_of(C, 16), rows_of(S2, 16), rows_of(W, kWld), 1, kSet);
+  if (tid < 32) {
+    const bool ok = inverse_f32(lane, W, Mi);
+    if (lane == 0) *fast = ok ? 1 : 0;
+  } else {
+    product16<1>(rows_of(S2, 16), cols_of(A, 16), rows_of(T1, kWld), 0, kSet);
+    const double rv = matvec<double>(lane, [&](int r, int l) { return C[l * 16 + r]; }, [&](int l) { return v2[l]; },
+                                     b[i]);
+    const double w = matvec<double>(lane, [&](int r, int l) { return -S2[l * 16 + r]; }, [&](int l) { return b[l]; },
+                                    v2[i]);
+    if (h == 0) {
+      wv[i] = w;
+      rr[i] = rv;
+    }
+  }
+  __syncthreads();
+  refine_inverse<NW>(W, Mi, Psi, 16, *fast != 0);
+  product16<NW>(rows_of(Mi, kWld), cols_of(A, 16), rows_of(Psi, 16), 0, kSet);
+  if (tid < 32) {
+    // alpha ; Sz = S2 alpha, l0 = Sz - v2 ; zeta
+    solve_refined(lane, W, Mi, rr, alpha);
+    const double sz = matvec<double>(lane, [&](int r, int l) { return S2[l * 16 + r]; },
+                                     [&](int l) { return alpha[l]; }, 0.0);
+    if (h == 0) {
+      Sz[i] = sz;
+      l0[i] = sz - v2[i];
+    }
+    __syncwarp();
+    const double cl = matvec<double>(lane, [&](int r, int l) { return C[l * 16 + r]; }, [&](int l) { return l0[l]; },
+                                     0.0);
+    const double zt = (h == 0) ? fma(0.5 * l0[i], cl, alpha[i] * fma(0.5, Sz[i], -v2[i])) : 0.0;
+    const double z = warp_sum(zt);
+    if (lane == 0) {
+      const double inc = e[kOffZeta] + z;  // the element's own share; the carry's zeta added after
+      out[272] = inc + V[272];
+      *zeta_inc = inc;
+    }
+  } else {
+    // v = eta + Psi^T wv ; Psi^T T1
+    const double vo = matvec<double>(lane, [&](int r, int l) { return Psi[l * 16 + r]; },
+                                     [&](int l) { return wv[l]; }, e[kOffEta + i]);
+    if (h == 0) out[256 + i] = vo;
+    product16<1>(cols_of(Psi, 16), cols_of(T1, kWld), rows_of(T1, kWld), 0, kSet);
+  }
+  __syncthreads();
+  for (int q = tid; q < 256; q += 32 * NW) {
+    const int r = q >> 4, c = q & 15;
+    out[q] = e[kOffJ + q] + T1[r < c ? r * kWld + c : c * kWld + r];
+  }
+  __syncthreads();
+}
+
+// (P, p) <- (P Psi, P alpha + p), by a CTA of two warps.
+__device__ inline void compose_right_split(double* P, double* p, const double* Psi, const double* alpha) {
+  const int lane = threadIdx.x & 31;
+  double pa = 0.0;
+  if (threadIdx.x < 32)
+    pa = matvec<double>(lane, [&](int r, int l) { return P[r * 16 + l]; }, [&](int l) { return alpha[l]; },
+                        p[lane & 15]);
+  __syncthreads();
+  split::product16<2>(rows_of(P, 16), cols_of(Psi, 16), rows_of(P, 16), 0, split::kSet);
+  if (threadIdx.x < 16) p[lane] = pa;
+  __syncthreads();
 }
 
 }  // namespace w16
