@@ -38,6 +38,7 @@
 
 #include "lqt_device.cuh"
 #include "lqt_internal.h"
+#include "lqt_uniform.cuh"
 
 namespace lqt {
 
@@ -723,6 +724,7 @@ __global__ void __launch_bounds__(32, 15) rk4_adjoint_warp_kernel(RK4AdjArgs a) 
   double* rhob = qb + (2 * 8 + 1) * AN;  // [2K+1]
   for (int64_t jj = blockIdx.x; jj < a.T; jj += gridDim.x) {
     const int64_t j = a.j0 + jj;
+    if (uniform_near(a.cf.uni, a.t, j, K)) continue;  // in the shared element's sweep
     const double h = (a.t[j + 1] - a.t[j]) / K;
     const double* F = a.cf.F.ptr + sample_index(a.cf.F.mode, j, 0, K) * nn;
     const double* Lt = a.cf.Lt.ptr + sample_index(a.cf.Lt.mode, j, 0, K) * n * M;
@@ -912,6 +914,85 @@ __global__ void b_to_lu_kernel(int n, int m, int64_t cnt, const double* __restri
     }
 }
 
+// The same for one sample (constant L and U) by a CTA: the factorisation of U
+// with its right-hand side L^T in shared memory (pivots and SINGULAR test as in
+// solve_rt; one thread took 167 us at n = 8, m = 4).
+__global__ void __launch_bounds__(256) b_to_lu_const_kernel(int n, int m, const double* __restrict__ Bb,
+                                                            const double* __restrict__ L,
+                                                            const double* __restrict__ U, double* __restrict__ gL,
+                                                            double* __restrict__ gU) {
+  __shared__ double W[16 * 16], R[16 * AN], S[AN * AN], V[16 * AN];
+  __shared__ unsigned long long rk[16];
+  __shared__ int piv;
+  const int tid = threadIdx.x;
+  for (int e = tid; e < m * m; e += 256) W[e] = U[e];
+  for (int e = tid; e < m * n; e += 256) R[e] = L[(e % n) * m + e / n];
+  for (int e = tid; e < n * n; e += 256) S[e] = Bb[e] + Bb[(e % n) * n + e / n];
+  __syncthreads();
+  if (tid < m) {
+    rk[tid] = 0ull;
+    for (int j = 0; j < m; ++j) rk[tid] = umax64(rk[tid], mag_key(W[tid * m + j]));
+  }
+  __syncthreads();
+  for (int k = 0; k < m; ++k) {
+    if (tid == 0) {
+      int p = k;
+      for (int i = k + 1; i < m; ++i)
+        if (mag_key(W[i * m + k]) > mag_key(W[p * m + k])) p = i;
+      if (pivot_too_small(W[p * m + k], rk[p])) flag(kStatusSingular);
+      const unsigned long long t = rk[k];
+      rk[k] = rk[p];
+      rk[p] = t;
+      piv = p;
+    }
+    __syncthreads();
+    const int p = piv;
+    for (int c = tid; p != k && c < m + n; c += 256) {
+      double* x = c < m ? &W[k * m + c] : &R[k * n + c - m];
+      double* y = c < m ? &W[p * m + c] : &R[p * n + c - m];
+      const double t = *x;
+      *x = *y;
+      *y = t;
+    }
+    __syncthreads();
+    // row k scaled, the other rows reduced (Gauss-Jordan on the right-hand side)
+    const double inv = 1.0 / W[k * m + k];
+    const int cols = m - k - 1 + n;
+    double f[2], v[2];
+    for (int s = 0; s < 2; ++s) {
+      const int e = tid + 256 * s, i = e / cols, c = e - i * cols;
+      if (e < m * cols) {
+        f[s] = W[i * m + k] * inv;
+        v[s] = c < m - k - 1 ? W[k * m + k + 1 + c] : R[k * n + c - (m - k - 1)];
+      }
+    }
+    __syncthreads();
+    for (int s = 0; s < 2; ++s) {
+      const int e = tid + 256 * s, i = e / cols, c = e - i * cols;
+      if (e < m * cols) {
+        double* x = c < m - k - 1 ? &W[i * m + k + 1 + c] : &R[i * n + c - (m - k - 1)];
+        *x = i == k ? v[s] * inv : fma(-f[s], v[s], *x);
+      }
+    }
+    __syncthreads();
+  }
+  // R = U^-1 L^T ; Lbar = (Bbar + Bbar^T) R^T ; Ubar = -R sym(Bbar) R^T
+  for (int e = tid; e < n * m; e += 256) {
+    const int i = e / m, c = e % m;
+    double s = 0.0;
+    for (int l = 0; l < n; ++l) s = fma(S[i * n + l], R[c * n + l], s);
+    gL[e] = s;
+    V[c * n + i] = 0.5 * s;
+  }
+  __syncthreads();
+  for (int e = tid; e < m * m; e += 256) {
+    const int i = e / m, c = e % m;
+    double s = 0.0;
+    for (int l = 0; l < n; ++l) s = fma(R[i * n + l], V[c * n + l], s);
+    gU[e] = -s;
+  }
+}
+
 // ---------------------------------------------------------------------------
 // host driver
 // ---------------------------------------------------------------------------
@@ -961,7 +1042,7 @@ static void cong_scan(int n, int64_t T, const double* maps0, const double* D, do
 }
 
 struct BackwardPlan {
-  size_t coef, elems, maps, rmaps, ystates, affine, D, emap, Sigma, cong, ebar, ys, pF, pB, pX, pr, gB, gLt, gUt,
+  size_t coef, elems, maps, rmaps, ystates, affine, D, emap, Sigma, cong, ebar, ys, pF, pB, pX, pr, upart, gB, gLt, gUt,
       end;
 };
 
@@ -999,9 +1080,12 @@ static BackwardPlan backward_plan(const lqt_problem& p, const Layout& L, size_t 
   }
   b.ebar = off; off = al(off + T1 * fs * 8);
   b.ys = off; off = al(off + (size_t)adjoint_segment(p.T) * K * 4 * fs * 8);
-  b.pF = off; off = al(off + T * n * n * 8);
-  b.pB = off; off = al(off + T * n * n * 8);
-  b.pX = off; off = al(off + T * n * n * 8);
+  // (three rows more for the shared element's totals, lqt_uniform_adjoint.cu)
+  b.pF = off; off = al(off + (T + 3) * n * n * 8);
+  b.pB = off; off = al(off + (T + 3) * n * n * 8);
+  b.pX = off; off = al(off + (T + 3) * n * n * 8);
+  b.upart = off;
+  if (L.uniform) off = al(off + (size_t)uniform_adjoint_parts(p.T) * 13 * n * n * 8);
   b.pr = off; off = al(off + T * (2 * K + 1) * n * 8);
   const size_t nLt = (size_t)sample_count(L.mode_Lt, p.T, p.K);
   b.gB = off; off = al(off + nLt * n * n * 8);
@@ -1033,14 +1117,18 @@ cudaError_t run_backward(const lqt_problem& p, const Layout& L, size_t elem_byte
   // are recomputed there, segment by segment
   const bool one_segment = T <= adjoint_segment(T) && T <= kAdjSegment;
   if (one_segment) {
-    cf.uni = nullptr;  // every sub-interval's RK4 stages are recorded
+    if (cf.uni) {
+      e = launch_uniform_master(p, cf, st);
+      if (e == cudaSuccess) e = launch_uniform_expand(p, cf, el, st);
+      if (e != cudaSuccess) return e;
+    }
+    // (the sub-intervals the shared element does not serve)
     e = launch_build_stages_range(p, L, cf, 0, T, (double*)(ws + b.ys), st, el);
     if (e == cudaSuccess) e = launch_terminal_element(p, el, st);
   } else {
     e = launch_build(p, L, cf, el, st);
   }
   if (e != cudaSuccess) return e;
-  cf.uni = nullptr;
   double* maps = (double*)(ws + b.maps);
   e = launch_maps_from_values(p, el, S, v, maps, st);
   if (e != cudaSuccess) return e;
@@ -1102,6 +1190,15 @@ cudaError_t run_backward(const lqt_problem& p, const Layout& L, size_t elem_byte
     }
     ra.T = T;
   }
+  if (cf.uni) {
+    UniAdjArgs ua{};
+    ua.n = n; ua.K = K; ua.T = T; ua.t = p.t; ua.cf = cf; ua.X = p.X.ptr; ua.r = p.r.ptr; ua.r_mode = p.r.mode;
+    ua.ebar = ea.ebar_out; ua.part = (double*)(ws + b.upart); ua.parts = uniform_adjoint_parts(T);
+    ua.pF = ra.pF; ua.pB = ra.pB; ua.pX = ra.pX; ua.pr = ra.pr;
+    e = launch_uniform_adjoint(ua, st);
+    if (e != cudaSuccess) return e;
+  }
+  const int64_t rows = cf.uni ? T + 3 : T;  // rows of pF, pB, pX
   // 6. reductions
   auto reduce = [&](const double* part, int64_t rows, int size, int32_t mode, double* out) {
     if (!out) return;
@@ -1112,8 +1209,8 @@ cudaError_t run_backward(const lqt_problem& p, const Layout& L, size_t elem_byte
     }
     count_launch();
   };
-  reduce(ra.pF, T, n * n, p.F.mode, gF);
-  reduce(ra.pX, T, n * n, p.X.mode, gX);
+  reduce(ra.pF, rows, n * n, p.F.mode, gF);
+  reduce(ra.pX, rows, n * n, p.X.mode, gX);
   if (gr && p.r.ptr) {
     if (p.r.mode == kConst) {
       reduce(ra.pr, T * (2 * K + 1), n, kConst, gr);
@@ -1126,10 +1223,13 @@ cudaError_t run_backward(const lqt_problem& p, const Layout& L, size_t elem_byte
   if (gL || gU) {
     const int64_t nLt = sample_count(L.mode_Lt, T, K);
     double* gB = (double*)(ws + b.gB);
-    reduce(ra.pB, T, n * n, L.mode_Lt, gB);
+    reduce(ra.pB, rows, n * n, L.mode_Lt, gB);
     double* gLt = (double*)(ws + b.gLt);
     double* gUt = (double*)(ws + b.gUt);
-    b_to_lu_kernel<<<nb(nLt, 64), 64, 0, st>>>(n, m, nLt, gB, p.L.ptr, p.L.mode, p.U.ptr, p.U.mode, K, gLt, gUt);
+    if (nLt == 1)
+      b_to_lu_const_kernel<<<1, 256, 0, st>>>(n, m, gB, p.L.ptr, p.U.ptr, gLt, gUt);
+    else
+      b_to_lu_kernel<<<nb(nLt, 64), 64, 0, st>>>(n, m, nLt, gB, p.L.ptr, p.L.mode, p.U.ptr, p.U.mode, K, gLt, gUt);
     count_launch();
     reduce(gLt, nLt, n * m, p.L.mode == L.mode_Lt ? kPerInterval : kConst, gL);
     reduce(gUt, nLt, m * m, p.U.mode == L.mode_Lt ? kPerInterval : kConst, gU);

@@ -449,45 +449,63 @@ cudaError_t launch_prepare_coefs(const lqt_problem& p, const Layout& lay, char* 
 //   dJ/ds    = -Q - J F - F^T J + J B J     = -Q - JF - (JF)^T + P P^T
 //   dzeta/ds = -rho/2 + eta^T B eta / 2 + eta^T c = -rho/2 + |w|^2/2 + eta^T c
 // with AL = A Lt, P = J Lt, w = Lt^T eta, q = H^T X r, rho = r^T X r.
+//
+// nzF, nzL: bit l N + j (l M + a) is set where F_lj (Lt_la) may be nonzero.
+// With constant F and L the bits are the same in every thread of a warp, and a
+// product by an exact zero is skipped by a branch instead of taking its 64
+// cycles of the FP64 pipe: models made of integrator chains have few nonzeros
+// (the point mass: 2 of 16 in F, 2 of 8 in L; its right-hand side then takes
+// 146 FP64 instructions of 300).  Dense or sampled F, L: every bit set.
 template <int N, int M>
 __device__ __forceinline__ void element_rhs(const Elem<N>& y, const double* __restrict__ F,
                                             const double* __restrict__ c, const double* __restrict__ Lt,
                                             const double* __restrict__ Q, const double* __restrict__ qr,
-                                            Elem<N>& k) {
+                                            Elem<N>& k, unsigned long long nzF, unsigned long long nzL) {
   double AL[N * M], P[N * M], w[M];
 #pragma unroll
-  for (int i = 0; i < N; ++i)
+  for (int e = 0; e < N * M; ++e) AL[e] = P[e] = 0.0;
 #pragma unroll
-    for (int a = 0; a < M; ++a) {
-      double s1 = 0.0, s2 = 0.0;
+  for (int a = 0; a < M; ++a) w[a] = 0.0;
 #pragma unroll
-      for (int l = 0; l < N; ++l) {
+  for (int l = 0; l < N; ++l)
+#pragma unroll
+    for (int a = 0; a < M; ++a)
+      for (unsigned on = taken_if(nzL >> (l * M + a) & 1ull); on != 0u; on >>= 1) {
         const double lt = Lt[l * M + a];
-        s1 = fma(y.A[i * N + l], lt, s1);
-        s2 = fma(y.J[sidx<N>(i, l)], lt, s2);
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+          AL[i * M + a] = fma(y.A[i * N + l], lt, AL[i * M + a]);
+          P[i * M + a] = fma(y.J[sidx<N>(i, l)], lt, P[i * M + a]);
+        }
+        w[a] = fma(lt, y.eta[l], w[a]);
       }
-      AL[i * M + a] = s1;
-      P[i * M + a] = s2;
-    }
+  // dA = AL P^T - A F, JF = J F, deta = -q - F^T eta ...
+  double JF[N * N];
 #pragma unroll
-  for (int a = 0; a < M; ++a) {
-    double s = 0.0;
-#pragma unroll
-    for (int l = 0; l < N; ++l) s = fma(Lt[l * M + a], y.eta[l], s);
-    w[a] = s;
-  }
-  // dA = AL P^T - A F
-#pragma unroll
-  for (int i = 0; i < N; ++i)
+  for (int i = 0; i < N; ++i) {
+    k.eta[i] = -qr[i];
 #pragma unroll
     for (int j = 0; j < N; ++j) {
       double s = 0.0;
 #pragma unroll
       for (int a = 0; a < M; ++a) s = fma(AL[i * M + a], P[j * M + a], s);
-#pragma unroll
-      for (int l = 0; l < N; ++l) s = fma(-y.A[i * N + l], F[l * N + j], s);
       k.A[i * N + j] = s;
+      JF[i * N + j] = 0.0;
     }
+  }
+#pragma unroll
+  for (int l = 0; l < N; ++l)
+#pragma unroll
+    for (int j = 0; j < N; ++j)
+      for (unsigned on = taken_if(nzF >> (l * N + j) & 1ull); on != 0u; on >>= 1) {
+        const double f = F[l * N + j];
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+          k.A[i * N + j] = fma(-y.A[i * N + l], f, k.A[i * N + j]);
+          JF[i * N + j] = fma(y.J[sidx<N>(i, l)], f, JF[i * N + j]);
+        }
+        k.eta[j] = fma(-f, y.eta[l], k.eta[j]);
+      }
   // db = -AL w - A c
 #pragma unroll
   for (int i = 0; i < N; ++i) {
@@ -510,12 +528,10 @@ __device__ __forceinline__ void element_rhs(const Elem<N>& y, const double* __re
       for (int a = 0; a < M; ++a) s = fma(-AL[i * M + a], AL[j * M + a], s);
       k.C[sidx<N>(i, j)] = s;
     }
-  // deta = -q - F^T eta + J c + P w
+  // deta ... + J c + P w
 #pragma unroll
   for (int i = 0; i < N; ++i) {
-    double s = -qr[i];
-#pragma unroll
-    for (int l = 0; l < N; ++l) s = fma(-F[l * N + i], y.eta[l], s);
+    double s = k.eta[i];
     if (c) {
 #pragma unroll
       for (int l = 0; l < N; ++l) s = fma(y.J[sidx<N>(i, l)], c[l], s);
@@ -525,16 +541,6 @@ __device__ __forceinline__ void element_rhs(const Elem<N>& y, const double* __re
     k.eta[i] = s;
   }
   // dJ = -Q - JF - (JF)^T + P P^T
-  double JF[N * N];
-#pragma unroll
-  for (int i = 0; i < N; ++i)
-#pragma unroll
-    for (int j = 0; j < N; ++j) {
-      double s = 0.0;
-#pragma unroll
-      for (int l = 0; l < N; ++l) s = fma(y.J[sidx<N>(i, l)], F[l * N + j], s);
-      JF[i * N + j] = s;
-    }
 #pragma unroll
   for (int i = 0; i < N; ++i)
 #pragma unroll
@@ -555,6 +561,30 @@ __device__ __forceinline__ void element_rhs(const Elem<N>& y, const double* __re
   k.zeta = z;
 }
 
+// The right-hand side at the boundary A = I, J = 0, eta = 0, where every
+// sub-interval starts.
+template <int N, int M>
+__device__ __forceinline__ void element_rhs_start(const double* __restrict__ F, const double* __restrict__ c,
+                                                  const double* __restrict__ Lt, const double* __restrict__ Q,
+                                                  const double* __restrict__ qr, Elem<N>& k) {
+#pragma unroll
+  for (int e = 0; e < N * N; ++e) k.A[e] = 0.0 - F[e];
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    k.b[i] = c ? 0.0 - c[i] : 0.0;
+    k.eta[i] = -qr[i];
+#pragma unroll
+    for (int j = i; j < N; ++j) {
+      double s = 0.0;
+#pragma unroll
+      for (int a = 0; a < M; ++a) s = fma(-Lt[i * M + a], Lt[j * M + a], s);
+      k.C[sidx<N>(i, j)] = s;
+      k.J[sidx<N>(i, j)] = -Q[i * N + j];
+    }
+  }
+  k.zeta = -0.5 * qr[N];
+}
+
 // y <- base + s * k over every field.
 template <int N>
 __device__ __forceinline__ void axpy_to(Elem<N>& y, const Elem<N>& base, double s, const Elem<N>& k) {
@@ -571,6 +601,18 @@ __device__ __forceinline__ void axpy_to(Elem<N>& y, const Elem<N>& base, double 
     y.J[i] = fma(s, k.J[i], base.J[i]);
   }
   y.zeta = fma(s, k.zeta, base.zeta);
+}
+
+// The same over A, eta and J, which drive the element flow: b, C and zeta
+// appear on no right-hand side, so a stage input needs none of them.
+template <int N>
+__device__ __forceinline__ void axpy_flow(Elem<N>& y, const Elem<N>& base, double s, const Elem<N>& k) {
+#pragma unroll
+  for (int i = 0; i < N * N; ++i) y.A[i] = fma(s, k.A[i], base.A[i]);
+#pragma unroll
+  for (int i = 0; i < N; ++i) y.eta[i] = fma(s, k.eta[i], base.eta[i]);
+#pragma unroll
+  for (int i = 0; i < Dim<N>::NS; ++i) y.J[i] = fma(s, k.J[i], base.J[i]);
 }
 
 struct BuildArgs {
@@ -632,6 +674,8 @@ __device__ __forceinline__ void build_one(const Coefs& cf, const double* t, int6
     y.J[i] = 0.0;
   }
   y.zeta = 0.0;
+  if constexpr (kStages) yt = y;  // the stored b, C, zeta of a stage input are zero
+  const unsigned long long nzF = nonzero_bits<N * N>(cf.F), nzL = nonzero_bits<N * M>(cf.Lt);
   for (int32_t i = K - 1; i >= 0; --i) {
     // stage times (in half steps from t_j): 2i+2, 2i+1, 2i+1, 2i
     const int32_t ps[3] = {2 * i + 2, 2 * i + 1, 2 * i};
@@ -650,19 +694,22 @@ __device__ __forceinline__ void build_one(const Coefs& cf, const double* t, int6
     }
     double* st = kStages ? stages + (int64_t)i * 4 * FS : nullptr;
     if constexpr (kStages) store_full<N>(y, st);
-    element_rhs<N, M>(y, F[0], c[0], Lt[0], Q[0], qr[0], k);
+    if (i == K - 1)
+      element_rhs_start<N, M>(F[0], c[0], Lt[0], Q[0], qr[0], k);
+    else
+      element_rhs<N, M>(y, F[0], c[0], Lt[0], Q[0], qr[0], k, nzF, nzL);
     axpy_to(yn, y, -h / 6.0, k);
-    axpy_to(yt, y, -0.5 * h, k);
+    axpy_flow(yt, y, -0.5 * h, k);
     if constexpr (kStages) store_full<N>(yt, st + FS);
-    element_rhs<N, M>(yt, F[1], c[1], Lt[1], Q[1], qr[1], k);
+    element_rhs<N, M>(yt, F[1], c[1], Lt[1], Q[1], qr[1], k, nzF, nzL);
     axpy_to(yn, yn, -h / 3.0, k);
-    axpy_to(yt, y, -0.5 * h, k);
+    axpy_flow(yt, y, -0.5 * h, k);
     if constexpr (kStages) store_full<N>(yt, st + 2 * FS);
-    element_rhs<N, M>(yt, F[1], c[1], Lt[1], Q[1], qr[1], k);
+    element_rhs<N, M>(yt, F[1], c[1], Lt[1], Q[1], qr[1], k, nzF, nzL);
     axpy_to(yn, yn, -h / 3.0, k);
-    axpy_to(yt, y, -h, k);
+    axpy_flow(yt, y, -h, k);
     if constexpr (kStages) store_full<N>(yt, st + 3 * FS);
-    element_rhs<N, M>(yt, F[2], c[2], Lt[2], Q[2], qr[2], k);
+    element_rhs<N, M>(yt, F[2], c[2], Lt[2], Q[2], qr[2], k, nzF, nzL);
     axpy_to(y, yn, -h / 6.0, k);
   }
 }
@@ -683,7 +730,7 @@ __global__ void __launch_bounds__(128) build_kernel(BuildArgs a) {
 template <int N, int M>
 __global__ void __launch_bounds__(128) build_stages_kernel(BuildArgs a, int64_t j0, double* stages) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= a.T) return;
+  if (i >= a.T || uniform_near(a.cf.uni, a.t, j0 + i, a.K)) return;
   constexpr int FS = 3 * N * N + 2 * N + 1;
   Elem<N> y;
   build_one<N, M, true>(a.cf, a.t, j0 + i, a.K, y, stages + i * (int64_t)a.K * 4 * FS);

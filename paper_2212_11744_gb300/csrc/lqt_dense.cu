@@ -142,6 +142,7 @@ __global__ void __launch_bounds__(128) densify_kernel(DenseArgs a) {
   constexpr int NS = Dim<N>::NS;
   const int32_t K = a.K;
   const Coefs& cf = a.cf;
+  const unsigned long long nzF = nonzero_bits<N * N>(cf.F), nzL = nonzero_bits<N * M>(cf.Lt);
   for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < a.T; j += (int64_t)gridDim.x * blockDim.x) {
     const double h = (a.t[j + 1] - a.t[j]) / K;
     const int64_t g0 = j * K;
@@ -161,17 +162,17 @@ __global__ void __launch_bounds__(128) densify_kernel(DenseArgs a) {
         Q[q] = cf.Q.ptr + sample_index(cf.Q.mode, j, ps[q], K) * N * N;
         qr[q] = cf.qr.ptr + sample_index(cf.qr.mode, j, ps[q], K) * (N + 1);
       }
-      riccati_rhs<N, M>(y, F[0], c[0], Lt[0], Q[0], qr[0], k);
+      riccati_rhs<N, M>(y, F[0], c[0], Lt[0], Q[0], qr[0], k, nzF, nzL);
       D[i + 1] = k;
       ric_axpy(yn, y, -h / 6.0, k);
       ric_axpy(yt, y, -0.5 * h, k);
-      riccati_rhs<N, M>(yt, F[1], c[1], Lt[1], Q[1], qr[1], k);
+      riccati_rhs<N, M>(yt, F[1], c[1], Lt[1], Q[1], qr[1], k, nzF, nzL);
       ric_axpy(yn, yn, -h / 3.0, k);
       ric_axpy(yt, y, -0.5 * h, k);
-      riccati_rhs<N, M>(yt, F[1], c[1], Lt[1], Q[1], qr[1], k);
+      riccati_rhs<N, M>(yt, F[1], c[1], Lt[1], Q[1], qr[1], k, nzF, nzL);
       ric_axpy(yn, yn, -h / 3.0, k);
       ric_axpy(yt, y, -h, k);
-      riccati_rhs<N, M>(yt, F[2], c[2], Lt[2], Q[2], qr[2], k);
+      riccati_rhs<N, M>(yt, F[2], c[2], Lt[2], Q[2], qr[2], k, nzF, nzL);
       ric_axpy(y, yn, -h / 6.0, k);
       if (i > 0) ok = store_values<N>(y, a.Sd + (g0 + i) * N * N, a.vd + (g0 + i) * N, a.zd + g0 + i) && ok;
     }
@@ -182,7 +183,7 @@ __global__ void __launch_bounds__(128) densify_kernel(DenseArgs a) {
       const double* Lt = cf.Lt.ptr + sample_index(cf.Lt.mode, j, 0, K) * N * M;
       const double* Q = cf.Q.ptr + sample_index(cf.Q.mode, j, 0, K) * N * N;
       const double* qr = cf.qr.ptr + sample_index(cf.qr.mode, j, 0, K) * (N + 1);
-      riccati_rhs<N, M>(y, F, c, Lt, Q, qr, D[0]);
+      riccati_rhs<N, M>(y, F, c, Lt, Q, qr, D[0], nzF, nzL);
     }
     // boundary point t_j: the given solution
     double x[N];
@@ -217,25 +218,25 @@ __global__ void __launch_bounds__(128) densify_kernel(DenseArgs a) {
         Lt[q] = cf.Lt.ptr + sample_index(cf.Lt.mode, j, ps[q], K) * N * M;
       }
       double kx[N], ax[N], xt[N];
-      closed_loop_rhs<N, M>(y0.S, y0.v, x, F[0], c[0], Lt[0], kx);
+      closed_loop_rhs<N, M>(y0.S, y0.v, x, F[0], c[0], Lt[0], kx, nzF, nzL);
 #pragma unroll
       for (int q = 0; q < N; ++q) {
         ax[q] = fma(h / 6.0, kx[q], x[q]);
         xt[q] = fma(0.5 * h, kx[q], x[q]);
       }
-      closed_loop_rhs<N, M>(ym.S, ym.v, xt, F[1], c[1], Lt[1], kx);
+      closed_loop_rhs<N, M>(ym.S, ym.v, xt, F[1], c[1], Lt[1], kx, nzF, nzL);
 #pragma unroll
       for (int q = 0; q < N; ++q) {
         ax[q] = fma(h / 3.0, kx[q], ax[q]);
         xt[q] = fma(0.5 * h, kx[q], x[q]);
       }
-      closed_loop_rhs<N, M>(ym.S, ym.v, xt, F[1], c[1], Lt[1], kx);
+      closed_loop_rhs<N, M>(ym.S, ym.v, xt, F[1], c[1], Lt[1], kx, nzF, nzL);
 #pragma unroll
       for (int q = 0; q < N; ++q) {
         ax[q] = fma(h / 3.0, kx[q], ax[q]);
         xt[q] = fma(h, kx[q], x[q]);
       }
-      closed_loop_rhs<N, M>(y1.S, y1.v, xt, F[2], c[2], Lt[2], kx);
+      closed_loop_rhs<N, M>(y1.S, y1.v, xt, F[2], c[2], Lt[2], kx, nzF, nzL);
 #pragma unroll
       for (int q = 0; q < N; ++q) {
         x[q] = fma(h / 6.0, kx[q], ax[q]);

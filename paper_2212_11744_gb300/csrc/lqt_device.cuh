@@ -46,6 +46,27 @@ struct Val {
   double zeta;
 };
 
+// Bit e set where entry e of a constant matrix is not zero; all bits for a
+// sampled one.
+template <int CNT>
+__device__ __forceinline__ unsigned long long nonzero_bits(const Coef& c) {
+  if (c.mode != kConst || CNT > 64) return ~0ull;
+  unsigned long long b = 0;
+  for (int e = 0; e < CNT; ++e)
+    b |= ((unsigned long long)__double_as_longlong(c.ptr[e]) << 1) != 0ull ? 1ull << e : 0ull;
+  return b;
+}
+
+// 1 or 0, hidden from the optimiser: `for (unsigned on = taken_if(bit); on; on =
+// 0)` runs its body behind a branch.  An `if` around a few multiply-adds is
+// compiled to predicated instructions instead, and an FP64 instruction whose
+// predicate is false in every lane still takes its 64 cycles.
+__device__ __forceinline__ unsigned taken_if(bool bit) {
+  unsigned v = bit ? 1u : 0u;
+  asm volatile("" : "+r"(v));
+  return v;
+}
+
 // Packed element size in doubles (A, b, C packed, eta, J packed, zeta).
 template <int N>
 __host__ __device__ constexpr int packed_elem_doubles() {

@@ -115,6 +115,22 @@ int64_t uniform_table_doubles(int n, int M);
 size_t uniform_table_bytes(int n, int M);
 cudaError_t launch_uniform_master(const lqt_problem& p, const Coefs& cf, cudaStream_t st);
 cudaError_t launch_uniform_expand(const lqt_problem& p, const Coefs& cf, const ElemPtrs& out, cudaStream_t st);
+// Reverse mode of that build (lqt_uniform_adjoint.cu).
+struct UniAdjArgs {
+  int32_t n, K;
+  int64_t T;
+  const double* t;
+  Coefs cf;             // cf.uni: the table
+  const double *X, *r;  // constant X; r constant or per interval, or null
+  int32_t r_mode;
+  const double* ebar;   // element adjoints [T][3 n^2 + 2 n + 1]
+  double* part;         // [parts][13 n^2]
+  int32_t parts;        // uniform_adjoint_parts(T)
+  double *pF, *pB, *pX;  // [T + 3][n^2]: rows T .. T + 2 receive the totals
+  double* pr;            // [T][2 K + 1][n]
+};
+int uniform_adjoint_parts(int64_t T);
+cudaError_t launch_uniform_adjoint(const UniAdjArgs& a, cudaStream_t st);
 cudaError_t launch_terminal_element(const lqt_problem& p, const ElemPtrs& out, cudaStream_t st);
 cudaError_t launch_build(const lqt_problem& p, const Layout& lay, const Coefs& cf, const ElemPtrs& out,
                          cudaStream_t s, double* team_scratch = nullptr);
@@ -158,6 +174,15 @@ void team_upper_reduce(const double* src, int64_t cnt, double* agg, cudaStream_t
 template <int N, typename GT>
 void team_upper_down(const double* src, int64_t cnt, const double* above, int64_t cnt_above, double* vals,
                      cudaStream_t st);
+// One step of the suffix scan over cnt element records (n = 4, 8), and the whole
+// prefix scan over cnt affine maps applied to x_in (starts [cnt + 1][n]; bufA,
+// bufB: cnt maps each): every step covers all records, so the scan has half the
+// dependent launches of an up- and a down-sweep.
+template <int N>
+void team_suffix_step(const double* src, int64_t cnt, int64_t d, double* dst, double* vals, cudaStream_t st);
+template <int N>
+void team_prefix_maps(const double* maps, int64_t cnt, const double* x_in, double* bufA, double* bufB, double* starts,
+                      cudaStream_t st);
 template <int N>
 void team_maps_reduce(const double* maps, int64_t cnt, int G, double* comp, cudaStream_t st);
 template <int N>

@@ -24,37 +24,50 @@ __host__ __device__ constexpr int ric_doubles() {
 // dS/dt = -(SF)^T - SF - Q + (S Lt)(S Lt)^T
 // dv/dt = -q + S c - F^T v + (S Lt)(Lt^T v)
 // dz/dt = -rho/2 + |Lt^T v|^2 / 2 + v^T c
+// nzF, nzL: the entries of F and Lt that may be nonzero (nonzero_bits); the
+// others are skipped.
 template <int N, int M>
 __device__ __forceinline__ void riccati_rhs(const RicState<N>& y, const double* __restrict__ F,
                                             const double* __restrict__ c, const double* __restrict__ Lt,
                                             const double* __restrict__ Q, const double* __restrict__ qr,
-                                            RicState<N>& k) {
-  double SL[N * M], w[M], SF[N * N];
+                                            RicState<N>& k, unsigned long long nzF = ~0ull,
+                                            unsigned long long nzL = ~0ull) {
+  double SL[N * M], w[M], SF[N * N], Fv[N];
 #pragma unroll
-  for (int i = 0; i < N; ++i)
+  for (int e = 0; e < N * M; ++e) SL[e] = 0.0;
 #pragma unroll
-    for (int a = 0; a < M; ++a) {
-      double s = 0.0;
+  for (int a = 0; a < M; ++a) w[a] = 0.0;
 #pragma unroll
-      for (int l = 0; l < N; ++l) s = fma(y.S[sidx<N>(i, l)], Lt[l * M + a], s);
-      SL[i * M + a] = s;
+  for (int l = 0; l < N; ++l)
+#pragma unroll
+    for (int a = 0; a < M; ++a)
+      for (unsigned on = taken_if(nzL >> (l * M + a) & 1ull); on != 0u; on >>= 1) {
+        const double lt = Lt[l * M + a];
+#pragma unroll
+        for (int i = 0; i < N; ++i) SL[i * M + a] = fma(y.S[sidx<N>(i, l)], lt, SL[i * M + a]);
+        w[a] = fma(lt, y.v[l], w[a]);
+      }
+#pragma unroll
+  for (int e = 0; e < N * N; ++e) SF[e] = 0.0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    double s = -qr[i];
+    if (c) {
+#pragma unroll
+      for (int l = 0; l < N; ++l) s = fma(y.S[sidx<N>(i, l)], c[l], s);
     }
-#pragma unroll
-  for (int a = 0; a < M; ++a) {
-    double s = 0.0;
-#pragma unroll
-    for (int l = 0; l < N; ++l) s = fma(Lt[l * M + a], y.v[l], s);
-    w[a] = s;
+    Fv[i] = s;
   }
 #pragma unroll
-  for (int i = 0; i < N; ++i)
+  for (int l = 0; l < N; ++l)
 #pragma unroll
-    for (int j = 0; j < N; ++j) {
-      double s = 0.0;
+    for (int j = 0; j < N; ++j)
+      for (unsigned on = taken_if(nzF >> (l * N + j) & 1ull); on != 0u; on >>= 1) {
+        const double f = F[l * N + j];
 #pragma unroll
-      for (int l = 0; l < N; ++l) s = fma(y.S[sidx<N>(i, l)], F[l * N + j], s);
-      SF[i * N + j] = s;
-    }
+        for (int i = 0; i < N; ++i) SF[i * N + j] = fma(y.S[sidx<N>(i, l)], f, SF[i * N + j]);
+        Fv[j] = fma(-f, y.v[l], Fv[j]);
+      }
 #pragma unroll
   for (int i = 0; i < N; ++i)
 #pragma unroll
@@ -69,13 +82,7 @@ __device__ __forceinline__ void riccati_rhs(const RicState<N>& y, const double* 
   for (int a = 0; a < M; ++a) z = fma(0.5 * w[a], w[a], z);
 #pragma unroll
   for (int i = 0; i < N; ++i) {
-    double s = -qr[i];
-    if (c) {
-#pragma unroll
-      for (int l = 0; l < N; ++l) s = fma(y.S[sidx<N>(i, l)], c[l], s);
-    }
-#pragma unroll
-    for (int l = 0; l < N; ++l) s = fma(-F[l * N + i], y.v[l], s);
+    double s = Fv[i];
 #pragma unroll
     for (int a = 0; a < M; ++a) s = fma(SL[i * M + a], w[a], s);
     k.v[i] = s;
@@ -89,7 +96,8 @@ template <int N, int M>
 __device__ __forceinline__ void closed_loop_rhs(const double* __restrict__ S, const double* __restrict__ v,
                                                 const double* __restrict__ x, const double* __restrict__ F,
                                                 const double* __restrict__ c, const double* __restrict__ Lt,
-                                                double* __restrict__ dx) {
+                                                double* __restrict__ dx, unsigned long long nzF = ~0ull,
+                                                unsigned long long nzL = ~0ull) {
   double e[N], w[M];
 #pragma unroll
   for (int i = 0; i < N; ++i) {
@@ -102,16 +110,19 @@ __device__ __forceinline__ void closed_loop_rhs(const double* __restrict__ S, co
   for (int a = 0; a < M; ++a) {
     double s = 0.0;
 #pragma unroll
-    for (int l = 0; l < N; ++l) s = fma(Lt[l * M + a], e[l], s);
+    for (int l = 0; l < N; ++l)
+      for (unsigned on = taken_if(nzL >> (l * M + a) & 1ull); on != 0u; on >>= 1) s = fma(Lt[l * M + a], e[l], s);
     w[a] = s;
   }
 #pragma unroll
   for (int i = 0; i < N; ++i) {
     double s = c ? c[i] : 0.0;
 #pragma unroll
-    for (int l = 0; l < N; ++l) s = fma(F[i * N + l], x[l], s);
+    for (int l = 0; l < N; ++l)
+      for (unsigned on = taken_if(nzF >> (i * N + l) & 1ull); on != 0u; on >>= 1) s = fma(F[i * N + l], x[l], s);
 #pragma unroll
-    for (int a = 0; a < M; ++a) s = fma(-Lt[i * M + a], w[a], s);
+    for (int a = 0; a < M; ++a)
+      for (unsigned on = taken_if(nzL >> (i * M + a) & 1ull); on != 0u; on >>= 1) s = fma(-Lt[i * M + a], w[a], s);
     dx[i] = s;
   }
 }

@@ -212,6 +212,34 @@ __global__ void __launch_bounds__(128) down_vals_upper_kernel(SrcFull<N> src, in
   }
 }
 
+// One step of the suffix scan over cnt records, one thread per record (n <= 3;
+// n = 4, 8: a warp, suffix_w8_kernel): dst_k = src_k (x) src_{k + d}, or src_k
+// where k + d is past the end; with `vals` (the last step) the value records.
+template <int N>
+__global__ void __launch_bounds__(32) suffix_step_kernel(const double* __restrict__ src, int64_t cnt, int64_t d,
+                                                         double* __restrict__ dst, double* __restrict__ vals) {
+  const int64_t k = (int64_t)blockIdx.x * 32 + threadIdx.x;
+  if (k >= cnt) return;
+  constexpr int FE = full_elem_doubles<N>();
+  Elem<N> a, e;
+  load_full<N>(src + k * FE, a);
+  if (k + d < cnt) {
+    load_full<N>(src + (k + d) * FE, e);
+    combine<N, double>(a, e, a);
+  }
+  if (vals) {
+    Val<N> v;
+#pragma unroll
+    for (int i = 0; i < Dim<N>::NS; ++i) v.S[i] = a.J[i];
+#pragma unroll
+    for (int i = 0; i < N; ++i) v.v[i] = a.eta[i];
+    v.zeta = a.zeta;
+    store_val_full<N>(vals + k * full_val_doubles<N>(), v);
+  } else {
+    store_full<N>(dst + k * FE, a);
+  }
+}
+
 // ---------------------------------------------------------------------------
 // affine-map (trajectory) scan kernels
 // ---------------------------------------------------------------------------
@@ -455,14 +483,31 @@ struct ScanPlan {
   int tlev;
   int64_t tcnt[64];                 // number of maps at trajectory level l (l >= 1)
   size_t off_tmap[64], off_tstart[64];
+  // the topmost value level is scanned in log2(cnt) steps over all its records
+  // instead of by levels above it (two buffers of records), and the topmost
+  // map level likewise
+  bool flat, tflat;
+  size_t off_flat[2], off_tflat[2];
   size_t bytes;
 };
 
+// Largest level that is scanned flat: there every step's combinations (all
+// records at once) still fit the sub-partitions about once over, so a step
+// takes the latency of one combination, and log2(cnt) steps replace log2(cnt)
+// levels up and as many, dearer ones, down.  Measured at n = 4, T = 10007 (2502
+// records): 110 + 188 us for the levels; n = 2, T = 1024: 65 + 93 us.
 template <int N>
-static ScanPlan make_plan(int64_t T, bool with_traj) {
+constexpr int64_t flat_below() { return N >= 8 ? 620 : N >= 4 ? 700 : 8192; }
+constexpr int64_t kFlatMaps = 1300;
+
+// The mixed path keeps the level structure (its results depend on the grouping
+// to FP32 rounding), and a scan of the values alone the size of its workspace.
+template <int N>
+static ScanPlan make_plan(int64_t T, bool with_traj, bool mixed = false) {
   ScanPlan pl;
   pl.G0 = level0_group(T);
   pl.T = T;
+  pl.flat = pl.tflat = false;
   size_t off = 0;
   const size_t PE = sizeof(double) * full_elem_doubles<N>();
   const size_t PV = sizeof(double) * full_val_doubles<N>();
@@ -480,6 +525,14 @@ static ScanPlan make_plan(int64_t T, bool with_traj) {
     ++pl.nlev;
     c = nc;
     G = kUpperGroup;
+    if (with_traj && !mixed && nc > kUpperGroup && nc <= flat_below<N>()) {
+      pl.flat = true;
+      for (size_t& o : pl.off_flat) {
+        o = off;
+        off = align_up(off + nc * PE);
+      }
+      break;
+    }
   }
   pl.off_maps = off;
   pl.tlev = 0;
@@ -495,6 +548,14 @@ static ScanPlan make_plan(int64_t T, bool with_traj) {
       off = align_up(off + (mc + 1) * sizeof(double) * N);
       ++pl.tlev;
       if (mc <= kUpperGroup) break;
+      if (!mixed && mc <= kFlatMaps) {
+        pl.tflat = true;
+        for (size_t& o : pl.off_tflat) {
+          o = off;
+          off = align_up(off + mc * PM);
+        }
+        break;
+      }
       mc = ceil_div(mc, kUpperGroup);
     }
   }
@@ -538,8 +599,26 @@ static void value_scan(const ScanPlan& pl, const ElemPtrs& el, const DownOut& ou
     }
     c = pl.cnt[l];
   }
+  // the topmost level's suffix values in steps over all its records
+  if (pl.flat) {
+    const int l = pl.nlev - 1;
+    const double* src = (const double*)(ws + pl.off_agg[l]);
+    double* vals = (double*)(ws + pl.off_val[l]);
+    int b = 0;
+    for (int64_t d = 1; d < pl.cnt[l]; d *= 2, b ^= 1) {
+      double* dst = (double*)(ws + pl.off_flat[b]);
+      double* out = 2 * d >= pl.cnt[l] ? vals : nullptr;
+      if constexpr (N == 4 || N == 8) {
+        team_suffix_step<N>(src, pl.cnt[l], d, dst, out, st);
+      } else {
+        suffix_step_kernel<N><<<(unsigned)ceil_div(pl.cnt[l], 32), 32, 0, st>>>(src, pl.cnt[l], d, dst, out);
+        count_launch();
+      }
+      src = dst;
+    }
+  }
   // down the levels: top level first (one group, zero carry)
-  for (int l = pl.nlev; l >= 1; --l) {
+  for (int l = pl.flat ? pl.nlev - 1 : pl.nlev; l >= 1; --l) {
     const double* above = (l < pl.nlev) ? (const double*)(ws + pl.off_val[l]) : nullptr;
     const int64_t cabove = (l < pl.nlev) ? pl.cnt[l] : 0;
     const int64_t cl = pl.cnt[l - 1];
@@ -578,8 +657,13 @@ static void traj_scan(const ScanPlan& pl, const double* x0, const double* S, con
       count_launch();
     }
   }
+  if (pl.tflat) {
+    const int l = pl.tlev - 1;
+    team_prefix_maps<N>((const double*)(ws + pl.off_tmap[l]), pl.tcnt[l], x0, (double*)(ws + pl.off_tflat[0]),
+                        (double*)(ws + pl.off_tflat[1]), (double*)(ws + pl.off_tstart[l]), st);
+  }
   // starts down the levels
-  for (int l = pl.tlev - 1; l >= 0; --l) {
+  for (int l = pl.tflat ? pl.tlev - 2 : pl.tlev - 1; l >= 0; --l) {
     const double* above = (l + 1 < pl.tlev) ? (const double*)(ws + pl.off_tstart[l + 1]) : nullptr;
     const int G = (l + 1 < pl.tlev) ? kUpperGroup : (int)pl.tcnt[l];
     const int64_t groups = ceil_div(pl.tcnt[l], G);
@@ -606,7 +690,7 @@ template <int N>
 static cudaError_t run_n(const lqt_problem& p, const Coefs& cf, const ElemPtrs& el, double* S, double* v,
                          double* zeta, const double* x0, double* x, double* u, double* cost, bool do_value,
                          bool do_traj, char* ws, cudaStream_t st) {
-  const ScanPlan pl = make_plan<N>(p.T, do_traj);
+  const ScanPlan pl = make_plan<N>(p.T, do_traj, t_mixed);
   double* maps0 = (double*)(ws + pl.off_maps);
   double* comp1 = pl.tlev > 0 ? (double*)(ws + pl.off_tmap[0]) : nullptr;
   if (do_value) {
@@ -1030,13 +1114,20 @@ cudaError_t run_method2(const lqt_problem& p, const Coefs& cf, const ElemPtrs& f
   }
 }
 
+// lqt_solve and lqt_solve_mixed share one size.
+template <int N>
+static size_t plan_bytes(int64_t T, bool with_traj) {
+  const size_t a = make_plan<N>(T, with_traj).bytes, b = make_plan<N>(T, with_traj, true).bytes;
+  return a > b ? a : b;
+}
+
 size_t scan_workspace_bytes(int32_t n, int64_t T, bool with_traj) {
   switch (n) {
-    case 1: return make_plan<1>(T, with_traj).bytes;
-    case 2: return make_plan<2>(T, with_traj).bytes;
-    case 3: return make_plan<3>(T, with_traj).bytes;
-    case 4: return make_plan<4>(T, with_traj).bytes;
-    case 8: return make_plan<8>(T, with_traj).bytes;
+    case 1: return plan_bytes<1>(T, with_traj);
+    case 2: return plan_bytes<2>(T, with_traj);
+    case 3: return plan_bytes<3>(T, with_traj);
+    case 4: return plan_bytes<4>(T, with_traj);
+    case 8: return plan_bytes<8>(T, with_traj);
     case 16:
     case 64: return team_scan_workspace_bytes(n, T, with_traj);
     default: return 0;

@@ -93,6 +93,7 @@ constexpr int max_slot_doubles() {
   if (reduce_slot_doubles<N>() > a) a = reduce_slot_doubles<N>();
   if (down_slot_doubles<N>() > a) a = down_slot_doubles<N>();
   if (maps_slot_doubles<N>() > a) a = maps_slot_doubles<N>();
+  if (N == 64 && 2 * Rec<N>::SIZE + s64::kSlotDoubles > a) a = 2 * Rec<N>::SIZE + s64::kSlotDoubles;
   return a;
 }
 
@@ -515,6 +516,11 @@ __device__ __forceinline__ bool finite_bits(double x) {
   return (__double_as_longlong(x) & 0x7ff0000000000000ll) != 0x7ff0000000000000ll;
 }
 
+// Doubles of a CTA's slot: the two running records (or two value records and
+// the chunk composite) and the combination's two global buffers.
+constexpr int kS64SlotDoubles = 2 * Rec<64>::SIZE + s64::kSlotDoubles;
+static_assert(kS64SlotDoubles >= 2 * team::val_doubles<64>() + 64 * 64 + 64 + s64::kSlotDoubles, "down-sweep slot");
+
 // n = 64 in FP64: one CTA per combination on split products; the running
 // records live in the CTA's workspace slot (L2).
 __global__ void __launch_bounds__(s64::kThreads, 1) reduce_s64_kernel(TeamScanArgs a) {
@@ -525,7 +531,8 @@ __global__ void __launch_bounds__(s64::kThreads, 1) reduce_s64_kernel(TeamScanAr
   const int tid = threadIdx.x;
   if (tid == 0) zero = 0.0;
   __syncthreads();
-  double* base = slot_base<N>(a.gscratch, reduce_slot_doubles<N>());
+  double* base = slot_base<N>(a.gscratch, kS64SlotDoubles);
+  const s64::Slot sl{base + 2 * Rec<N>::SIZE, base + 2 * Rec<N>::SIZE + s64::kBuf};
   const int64_t groups = tdiv(a.cnt, a.G);
   for (int64_t g = blockIdx.x; g < groups; g += gridDim.x) {
     const int64_t first = g * a.G;
@@ -533,7 +540,7 @@ __global__ void __launch_bounds__(s64::kThreads, 1) reduce_s64_kernel(TeamScanAr
     Rec<N> acc = Rec<N>::packed(base), nxt = Rec<N>::packed(base + Rec<N>::SIZE);
     team::copy_rec<N, NT>(tid, acc, level_elem<N>(a, last, &zero));
     for (int64_t k = last - 1; k >= first; --k) {
-      s64::combine(sm, level_elem<N>(a, k, &zero), acc, nxt);
+      s64::combine(sm, sl, level_elem<N>(a, k, &zero), acc, nxt);
       const Rec<N> t = acc;
       acc = nxt;
       nxt = t;
@@ -551,10 +558,11 @@ __global__ void __launch_bounds__(s64::kThreads, 1) down_s64_kernel(TeamScanArgs
   const int tid = threadIdx.x;
   if (tid == 0) zero = 0.0;
   __syncthreads();
-  double* c0 = slot_base<N>(a.gscratch, down_slot_doubles<N>());
+  double* c0 = slot_base<N>(a.gscratch, kS64SlotDoubles);
   double* c1 = c0 + VS;
   double* P = c1 + VS;
   double* pv = P + N * N;
+  const s64::Slot sl{pv + N, pv + N + s64::kBuf};
   const int64_t groups = tdiv(a.cnt, a.G);
   for (int64_t g = blockIdx.x; g < groups; g += gridDim.x) {
     const int64_t first = g * a.G;
@@ -567,7 +575,7 @@ __global__ void __launch_bounds__(s64::kThreads, 1) down_s64_kernel(TeamScanArgs
       for (int e = tid; e < PM; e += NT) P[e] = (e < N * N && e % (N + 1) == 0) ? 1.0 : 0.0;  // P, then pv
     __syncthreads();
     for (int64_t k = last; k >= first; --k) {
-      s64::combine_value(sm, level_elem<N>(a, k, &zero), carry, nv, &zinc);
+      s64::combine_value(sm, sl, level_elem<N>(a, k, &zero), carry, nv, &zinc);
       if (Level0) {
         bool ok = true;
         for (int e = tid; e < VS; e += NT) {
@@ -580,8 +588,8 @@ __global__ void __launch_bounds__(s64::kThreads, 1) down_s64_kernel(TeamScanArgs
         if (!ok) flag(kStatusNonFinite);
         if (a.maps != nullptr && k < a.T) {
           for (int e = tid; e < PM; e += NT)
-            a.maps[k * PM + e] = e < N * N ? sm.K1[(e >> 6) * s64::kLd + (e & 63)] : sm.vec[4][e - N * N];
-          s64::compose_right(sm, P, pv);
+            a.maps[k * PM + e] = e < N * N ? sl.K1[(e >> 6) * s64::kLd + (e & 63)] : sm.vec[4][e - N * N];
+          s64::compose_right(sm, sl, P, pv);
         }
       } else {
         for (int e = tid; e < VS; e += NT) a.vals[k * VS + e] = nv[e];
@@ -1134,6 +1142,113 @@ __global__ void __launch_bounds__(32) down_w8_kernel(const double* __restrict__ 
   }
 }
 
+// One step of the suffix scan over cnt records: dst_k = src_k (x) src_{k + d}, or
+// src_k where k + d is past the end (already the whole suffix).  With `vals`
+// (the last step) the results' J, eta, zeta, the suffix values, are written
+// there as value records instead.
+template <int N>
+__global__ void __launch_bounds__(32) suffix_w8_kernel(const double* __restrict__ src, int64_t cnt, int64_t d,
+                                                       double* __restrict__ dst, double* __restrict__ vals) {
+  using L = w8::Lay<N>;
+  __shared__ double e1[L::REC], e2[L::REC], out[L::REC], scr[L::SCRATCH];
+  const int lane = threadIdx.x;
+  for (int64_t k = blockIdx.x; k < cnt; k += gridDim.x) {
+    const bool two = k + d < cnt;
+    for (int e = lane; e < L::REC; e += 32) {
+      e1[e] = src[k * L::REC + e];
+      if (two) e2[e] = src[(k + d) * L::REC + e];
+    }
+    __syncwarp();
+    if (two) w8::combine<N, double>(lane, e1, e2, out, scr);
+    const double* r = two ? out : e1;
+    if (vals) {
+      for (int e = lane; e < L::VAL; e += 32)
+        vals[k * L::VAL + e] = e < N * N ? r[L::J + e] : e < N * N + N ? r[L::ETA + e - N * N] : r[L::ZETA];
+    } else {
+      for (int e = lane; e < L::REC; e += 32) dst[k * L::REC + e] = r[e];
+    }
+    __syncwarp();
+  }
+}
+
+template <int N>
+void team_suffix_step(const double* src, int64_t cnt, int64_t d, double* dst, double* vals, cudaStream_t st) {
+  if constexpr (N == 4 || N == 8) {
+    suffix_w8_kernel<N><<<(unsigned)cnt, 32, 0, st>>>(src, cnt, d, dst, vals);
+    count_launch();
+  }
+}
+
+// One radix-4 step of the prefix scan over cnt affine maps: dst_k = src_k o
+// src_{k - d} o src_{k - 2d} o src_{k - 3d} (those that exist; the rightmost is
+// applied first).  With `starts` (the last step) the states starts_{k + 1} =
+// dst_k(x_in) and starts_0 = x_in are written instead of the maps.
+template <int N>
+__global__ void __launch_bounds__(32) prefix_maps_kernel(const double* __restrict__ src, int64_t cnt, int64_t d,
+                                                         double* __restrict__ dst, const double* __restrict__ x_in,
+                                                         double* __restrict__ starts) {
+  constexpr int PM = N * N + N;
+  __shared__ double P[2][PM];
+  const int lane = threadIdx.x;
+  for (int64_t k = blockIdx.x; k < cnt; k += gridDim.x) {
+    double* cur = P[0];
+    double* nxt = P[1];
+    for (int e = lane; e < PM; e += 32) cur[e] = src[k * PM + e];
+    __syncwarp();
+    for (int s = 1; s < 4 && k - s * d >= 0; ++s) {
+      // (cur) o (m): Psi = Pc Pm, alpha = Pc a_m + a_c
+      const double* m = src + (k - s * d) * PM;
+      for (int e = lane; e < PM; e += 32) {
+        double v;
+        if (e < N * N) {
+          const int i = e / N, j = e % N;
+          v = 0.0;
+#pragma unroll
+          for (int l = 0; l < N; ++l) v = fma(cur[i * N + l], m[l * N + j], v);
+        } else {
+          const int i = e - N * N;
+          v = cur[e];
+#pragma unroll
+          for (int l = 0; l < N; ++l) v = fma(cur[i * N + l], m[N * N + l], v);
+        }
+        nxt[e] = v;
+      }
+      __syncwarp();
+      double* t = cur;
+      cur = nxt;
+      nxt = t;
+    }
+    if (starts) {
+      if (lane < N) {
+        double v = cur[N * N + lane];
+#pragma unroll
+        for (int l = 0; l < N; ++l) v = fma(cur[lane * N + l], x_in[l], v);
+        starts[(k + 1) * N + lane] = v;
+        if (k == 0) starts[lane] = x_in[lane];
+      }
+    } else {
+      for (int e = lane; e < PM; e += 32) dst[k * PM + e] = cur[e];
+    }
+    __syncwarp();
+  }
+}
+
+template <int N>
+void team_prefix_maps(const double* maps, int64_t cnt, const double* x_in, double* bufA, double* bufB, double* starts,
+                      cudaStream_t st) {
+  const double* src = maps;
+  double* dst = bufA;
+  int64_t d = 1;
+  for (;; d *= 4) {
+    const bool last = d * 4 >= cnt;
+    prefix_maps_kernel<N><<<(unsigned)cnt, 32, 0, st>>>(src, cnt, d, dst, x_in, last ? starts : nullptr);
+    count_launch();
+    if (last) break;
+    src = dst;
+    dst = dst == bufA ? bufB : bufA;
+  }
+}
+
 template <int N, typename GT>
 void team_upper_reduce(const double* src, int64_t cnt, double* agg, cudaStream_t st) {
   static_assert(Rec<N>::SIZE == full_elem_doubles<N>(), "record layouts differ");
@@ -1579,6 +1694,9 @@ template void launch_inv_master_team<64, 16>(int32_t, int32_t, const BatchProb*,
                                              double*, int64_t, cudaStream_t);
 
 #define LQT_TEAM_UPPER(N)                                                                                 \
+  template void team_suffix_step<N>(const double*, int64_t, int64_t, double*, double*, cudaStream_t);    \
+  template void team_prefix_maps<N>(const double*, int64_t, const double*, double*, double*, double*,    \
+                                    cudaStream_t);                                                       \
   template void team_upper_reduce<N, double>(const double*, int64_t, double*, cudaStream_t);             \
   template void team_upper_reduce<N, float>(const double*, int64_t, double*, cudaStream_t);              \
   template void team_upper_down<N, double>(const double*, int64_t, const double*, int64_t, double*,      \

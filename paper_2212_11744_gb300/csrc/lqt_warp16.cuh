@@ -693,6 +693,16 @@ __device__ __forceinline__ void solve_refined(int lane, const double* W, const d
   __syncwarp();
 }
 
+// Entry of zeta's saddle value z'Jz/2 - z'eta + l'(b - z) - l'Cl/2 at z0 = (I +
+// C J)^-1 (b + C eta), l0 = J z0 - eta (Sec. IV-A, the minimiser and multiplier
+// at x = 0).  At the exact saddle b - z0 = C l0 and this is l0'Cl0/2 + z0'Jz0/2 -
+// z0'eta; in this form an error of z0 or l0 enters to second order only, so
+// that zeta does not feel the conditioning of I + C J (at cond 1e8, n = 64, the
+// other form was 2e-6 off after 130 combinations).
+__device__ __forceinline__ double saddle_term(double z, double Jz, double eta, double l, double b, double Cl) {
+  return fma(z, fma(0.5, Jz, -eta), l * ((b - z) - 0.5 * Cl));
+}
+
 // Scratch of combine_split(): four 16 x 17 buffers and vectors.
 constexpr int kSplitBuf = 16 * kWld;
 constexpr int kSplitScratch = 4 * kSplitBuf + 6 * 16;
@@ -760,7 +770,7 @@ __device__ inline void combine_split(double* e1, const double* e2, double* scr) 
     __syncwarp();
     const double cl = matvec<double>(lane, [&](int r, int l) { return C1[l * 16 + r]; }, [&](int l) { return l0[l]; },
                                      0.0);
-    const double zt = (h == 0) ? fma(0.5 * l0[i], cl, z0[i] * fma(0.5, J2z[i], -eta2[i])) : 0.0;
+    const double zt = (h == 0) ? saddle_term(z0[i], J2z[i], eta2[i], l0[i], b1[i], cl) : 0.0;
     zs = warp_sum(zt);
   }
   if (second) {
@@ -843,7 +853,7 @@ __device__ inline void combine_value_split(const double* e, const double* V, dou
     __syncwarp();
     const double cl = matvec<double>(lane, [&](int r, int l) { return C[l * 16 + r]; }, [&](int l) { return l0[l]; },
                                      0.0);
-    const double zt = (h == 0) ? fma(0.5 * l0[i], cl, alpha[i] * fma(0.5, Sz[i], -v2[i])) : 0.0;
+    const double zt = (h == 0) ? saddle_term(alpha[i], Sz[i], v2[i], l0[i], b[i], cl) : 0.0;
     const double z = warp_sum(zt);
     if (lane == 0) {
       const double inc = e[kOffZeta] + z;  // the element's own share; the carry's zeta added after

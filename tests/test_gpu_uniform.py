@@ -123,3 +123,34 @@ def test_batch_members_with_other_grids(n):
         ref, got = oracle.solve(p), bt.problem_slice(out, b)
         for k in ("S", "v", "zeta", "x", "u"):
             assert rel(to_np(got[k]), ref[k]) <= TOL, (b, k)
+
+
+@pytest.mark.parametrize("grid,r,K", [("equal", "interval", 4), ("offsets", "interval", 2), ("thirds", "interval", 1),
+                                      ("offsets", "const", 8), ("uneven", "interval", 2)])
+def test_gradients_match_oracle(grid, r, K):
+    """The reverse sweep of the shared element (csrc/lqt_uniform_adjoint.cu)
+    beside the sweeps of the sub-intervals it does not serve."""
+    from tests.test_gpu_adjoint import TOL as GTOL, gpu_grads, oracle_grads, rel as grel, weights
+    p = make(8, 4, 1027 if K == 4 else 1056, K, grid, r)
+    w = weights(p, 5)
+    got, ref = gpu_grads(p, *w), oracle_grads(p, *w)
+    for k in ref:
+        assert grel(got[k].reshape(ref[k].shape), ref[k]) <= GTOL, k
+
+
+@pytest.mark.parametrize("n", [2, 4])
+def test_gradients_beyond_one_segment(n):
+    """T above the reverse sweep's segment: constant F (the shared element)
+    against the same F given per sub-interval (the general sweeps)."""
+    from tests.test_gpu_adjoint import TOL as GTOL, gpu_grads, rel as grel
+    T = 33001
+    p = make(n, 1, T, 2, "offsets", "interval")
+    rng = np.random.default_rng(n)
+    w = (rng.standard_normal((T + 1, n, n)), rng.standard_normal((T + 1, n)), rng.standard_normal(T + 1),
+         rng.standard_normal((T + 1, n)), 1.3)
+    a = gpu_grads(p, *w)
+    p.F = W.Coef(np.repeat(p.F.values, T, axis=0), W.PER_INTERVAL)
+    b = gpu_grads(p, *w)
+    b["F"] = b["F"].sum(axis=0, keepdims=True)
+    for k in a:
+        assert grel(a[k], b[k]) <= GTOL, k
