@@ -16,9 +16,8 @@
 //            updates w_k <- P_l (x) w_k, all such k and all grid points in one
 //            launch.  After the last bit w_k = V(., t_k).
 //
-// Both products are one kernel: a 16 x 16 tile of outputs per CTA, one output
-// per thread, the reduction index in steps of 64 staged in shared memory.  The
-// minimum is defined on FP64 sums, ascending k, strict improvement only (the
+// Both products are one kernel: a tile of outputs per CTA, several per thread, the
+// reduction index staged in shared memory.  The minimum is defined on FP64 sums, ascending k, strict improvement only (the
 // lowest index wins a tie).  GB300 retires FP64 adds at 1/64 of its FP32
 // rate, so every candidate is first screened in FP32 (a bracket around its
 // sum) and only the few whose bracket reaches the smallest upper bound are
@@ -56,8 +55,11 @@ GridArgs grid_args(const lqt_grid_problem& p) {
   return GridArgs{p.G, p.x_min, p.dx, p.d0, p.d1, p.d2, p.q, p.rho, p.qf, p.tau, p.substeps, p.T, p.interp};
 }
 
-constexpr int kGT = 16;  // output tile edge
-constexpr int kGK = 64;  // reduction step staged in shared memory (a grid of <= 64 points: one tile)
+// A CTA of 256 threads forms a tile of 16 P x 16 Q outputs, P x Q per thread; the
+// reduction index is staged in shared memory in float, at most kKC at a time (a
+// grid of <= 224 points: once).
+constexpr int kThreads = 256;
+constexpr int kKC = 224;
 
 __device__ __forceinline__ double grid_x(const GridArgs& a, int i) { return __dadd_rn(a.x_min, __dmul_rn((double)i, a.dx)); }
 
@@ -161,8 +163,12 @@ struct Operands {
 // FP64 sum g_k + f_k equals the FP64 minimum has lo_k <= U; every k with
 // lo_k > U has a larger FP64 sum.  So the exact minimum, with the lowest-index
 // rule, is taken over the survivors lo_k <= U alone, in ascending k, in FP64.
+// Where no operand of the tile is negative, t_k is s_k itself, so that U = s_min
+// + c s_min and lo_k <= U is a bound on s_k: a candidate then costs one
+// addition and one minimum, and one addition and one comparison in the second
+// pass (a bound rounded up keeps a few candidates more, never fewer).
 // Operands of magnitude >= 2^100 (or not finite) fall outside the screen's
-// float range: a CTA that meets one takes the FP64 path for all its outputs.
+// float range: a CTA that meets one evaluates every candidate in FP64.
 constexpr float kScreenC = 9.5367431640625e-07f;  // 2^-20
 constexpr float kScreenD = 7.888609052210118e-31f;  // 2^-100
 constexpr float kScreenPad = 1.329227995784916e+36f;  // 2^120: k beyond the grid
@@ -183,17 +189,6 @@ __device__ __forceinline__ float screen_float(double x) {
   return __uint_as_float(fb);
 }
 
-union GridSmem {
-  struct {
-    double A[kGT][kGK + 1];
-    double B[kGK][kGT + 1];
-  } d;  // FP64 path
-  struct {
-    float A[kGT][kGK + 2];
-    float Bt[kGT][kGK + 2];  // B transposed: one row of k per output column
-  } f;  // screen; rows of 66 floats keep float2 reads aligned and conflict-free
-};
-
 __device__ __forceinline__ float screen_hi(float a, float b) {
   return __fmaf_rn(kScreenC, __fadd_rn(fabsf(a), fabsf(b)), __fadd_rn(a, b));
 }
@@ -201,183 +196,218 @@ __device__ __forceinline__ float screen_lo(float a, float b) {
   return __fmaf_rn(-kScreenC, __fadd_rn(fabsf(a), fabsf(b)), __fadd_rn(a, b));
 }
 
-// Float tiles of A (rows i0.., reduction k0..) and B (reduction k0..,
-// columns c0..); k beyond the grid holds kScreenPad.  Returns whether an
-// operand lies outside the screen's range.
-template <bool kValues>
-__device__ __forceinline__ bool stage_float(const Operands<kValues>& op, GridSmem& sm, int t, int i0, int64_t c0,
-                                            int64_t ncols, int k0) {
-  const int G = op.a.G;
-  bool bad = false;
-  for (int e = t; e < kGT * kGK; e += kGT * kGT) {
-    const int r = e / kGK, kk = e % kGK;
-    const int gi = i0 + r, gk = k0 + kk;
+// Row stride (floats) of the staged tiles for kc values of k: a multiple of 4
+// that is 4 modulo 32, so that 16-byte reads of eight consecutive rows fall on
+// different banks.
+__host__ __device__ __forceinline__ int screen_stride(int kc) { return ((kc + 27) / 32) * 32 + 4; }
+
+// Float tiles of the A rows i0 .. and the B columns c0 .., k0 <= k < k0 + kc; k
+// beyond the grid holds kScreenPad.  Returns bit 0: an operand outside the
+// screen's range, bit 1: a negative operand.
+template <int TR, int TC, bool kValues>
+__device__ __forceinline__ int stage_float(const Operands<kValues>& op, float* As, float* Bs, int S, int t, int i0,
+                                           int64_t c0, int64_t ncols, int k0, int kc) {
+  const int G = op.a.G, warp = t >> 5, lane = t & 31;
+  int bad = 0;
+  auto put = [&](float* dst, bool live, int gk, double x) {
     float v = kScreenPad;
     if (gk < G) {
       v = 0.0f;
-      if (gi < G) {
-        const double x = op.av(gi, gk);
-        bad |= !screen_range(x);
+      if (live) {
+        bad |= (screen_range(x) ? 0 : 1) | (x < 0.0 ? 2 : 0);
         v = screen_float(x);
       }
     }
-    sm.f.A[r][kk] = v;
-  }
-  for (int e = t; e < kGT * kGK; e += kGT * kGT) {
-    int kk, cc;
-    if (kValues) {
-      cc = e / kGK; kk = e % kGK;
-    } else {
-      kk = e / kGT; cc = e % kGT;
+    *dst = v;
+  };
+  for (int r = warp; r < TR; r += kThreads / 32)
+    for (int kk = lane; kk < kc; kk += 32) {
+      const bool live = i0 + r < G && k0 + kk < G;
+      put(As + r * S + kk, live, k0 + kk, live ? op.av(i0 + r, k0 + kk) : 0.0);
     }
-    const int gk = k0 + kk;
-    const int64_t gc = c0 + cc;
-    float v = kScreenPad;
-    if (gk < G) {
-      v = 0.0f;
-      if (gc < ncols) {
-        const double x = op.bv(op.bcol(gc), gk);
-        bad |= !screen_range(x);
-        v = screen_float(x);
+  if (kValues) {
+    for (int r = warp; r < TC; r += kThreads / 32) {
+      const bool col = c0 + r < ncols;
+      const double* b = col ? op.bcol(c0 + r) : nullptr;
+      for (int kk = lane; kk < kc; kk += 32) {
+        const bool live = col && k0 + kk < G;
+        put(Bs + r * S + kk, live, k0 + kk, live ? b[k0 + kk] : 0.0);
       }
     }
-    sm.f.Bt[cc][kk] = v;
+  } else {
+    for (int e = t; e < TC * kc; e += kThreads) {
+      const int kk = e / TC, r = e % TC;
+      const bool live = c0 + r < ncols && k0 + kk < G;
+      put(Bs + r * S + kk, live, k0 + kk, live ? op.Bm[(int64_t)(k0 + kk) * G + c0 + r] : 0.0);
+    }
   }
   return bad;
 }
 
-// The FP64 evaluation of every candidate (CTAs whose operands leave the
-// screen's range): double tiles, ascending k, strict improvement.
-template <bool kValues>
-__device__ __forceinline__ void fp64_scan(const Operands<kValues>& op, GridSmem& sm, int t, int i0, int64_t c0,
-                                          int64_t ncols, int r_loc, int c_loc, double& best, int& bk) {
-  const int G = op.a.G;
-  long long bestk = LLONG_MAX;
-  for (int k0 = 0; k0 < G; k0 += kGK) {
-    for (int e = t; e < kGT * kGK; e += kGT * kGT) {
-      const int r = e / kGK, kk = e % kGK;
-      const int gi = i0 + r, gk = k0 + kk;
-      sm.d.A[r][kk] = (gi < G && gk < G) ? op.av(gi, gk) : 0.0;
-    }
-    for (int e = t; e < kGT * kGK; e += kGT * kGT) {
-      int kk, cc;
-      if (kValues) {
-        cc = e / kGK; kk = e % kGK;
-      } else {
-        kk = e / kGT; cc = e % kGT;
-      }
-      const int gk = k0 + kk;
-      const int64_t gc = c0 + cc;
-      sm.d.B[kk][cc] = (gk < G && gc < ncols) ? op.bv(op.bcol(gc), gk) : 0.0;
-    }
-    __syncthreads();
-    const int kend = G - k0 < kGK ? G - k0 : kGK;
-    for (int kk = 0; kk < kend; ++kk) {
-      const double v = __dadd_rn(sm.d.A[r_loc][kk], sm.d.B[kk][c_loc]);
-      const long long key = order_key(v);
-      if (key < bestk) {
-        bestk = key;
-        best = v;
-        bk = k0 + kk;
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// One output (i, c) per thread, a 16 x 16 tile per CTA: the FP32 screen over
-// all k (two passes: the bound U, then the survivors), the FP64 minimum over
-// the survivors, App. E's refinement, the store.  Rows run over i (grid y),
-// columns over j or c (grid x); in the values mode consecutive threads walk i
-// so that the w_out stores are coalesced.
-template <bool kValues>
-__global__ void __launch_bounds__(kGT* kGT, 4)
+// A tile of 16 P x 16 Q outputs (i, c) per CTA, P x Q per thread (rows t % 16 +
+// 16 p, columns t / 16 + 16 q: a warp's 16-byte reads of the staged rows are free
+// of conflicts, and in the values mode 16 consecutive lanes store 16
+// consecutive i): the FP32 screen over all k (two passes: the bound U, then the
+// survivors), the FP64 minimum over the survivors, App. E's refinement, the
+// store.  Bound by the FP32 and ALU instructions of the two passes and, per
+// output, by some 30 FP64 instructions of the refinement (its three divisions)
+// at 64 cycles each.  One output per thread, with staging again in the second
+// pass, took 4.43 ms for the block and the values at G = 201, T = 10^4; this
+// 3.09 ms (13 levels of about 5000 columns at 0.2 ms each).
+template <int P, int Q, bool kValues>
+__global__ void __launch_bounds__(kThreads, 2)
     grid_minplus_kernel(GridArgs a, const double* __restrict__ A, const double* Bm, double* Om, double* X0,
                         double* X1, int l, int64_t ncols, const double2* __restrict__ tab) {
-  __shared__ GridSmem sm;
+  constexpr int TR = 16 * P, TC = 16 * Q;
+  extern __shared__ __align__(16) float grid_smem[];
   const Operands<kValues> op{a, A, Bm, Om, X0, X1, l};
-  const int G = a.G;
-  const int t = threadIdx.x;
-  const int r_loc = kValues ? t % kGT : t / kGT;  // output row inside the tile
-  const int c_loc = kValues ? t / kGT : t % kGT;  // output column inside the tile
-  const int i0 = blockIdx.y * kGT;
-  const int64_t c0 = (int64_t)blockIdx.x * kGT;
-  const int i = i0 + r_loc;
-  const int64_t c = c0 + c_loc;
-  const bool valid = i < G && c < ncols;
+  const int G = a.G, t = threadIdx.x, ti = t & 15, tc = t >> 4;
+  const int i0 = blockIdx.y * TR;
+  const int64_t c0 = (int64_t)blockIdx.x * TC;
+  const int kc = G < kKC ? ((G + 3) & ~3) : kKC;  // staged values of k (padded)
+  const int S = screen_stride(kc);
+  float* As = grid_smem;
+  float* Bs = As + TR * S;
 
-  double best = 0.0;
-  int bk = 0;
-  // pass 1: U = min_k hi_k
-  bool bad = false;
-  float U = __int_as_float(0x7f800000);  // +inf
-  for (int k0 = 0; k0 < G; k0 += kGK) {
-    bad |= stage_float(op, sm, t, i0, c0, ncols, k0);
+  int bad = 0;
+  float U[P][Q];
+#pragma unroll
+  for (int p = 0; p < P; ++p)
+#pragma unroll
+    for (int q = 0; q < Q; ++q) U[p][q] = __int_as_float(0x7f800000);  // +inf
+  // pass 1, as if nothing were negative: the smallest sum
+  for (int k0 = 0; k0 < G; k0 += kc) {
+    if (k0) __syncthreads();
+    bad |= stage_float<TR, TC>(op, As, Bs, S, t, i0, c0, ncols, k0, kc);
     __syncthreads();
-    const int kend = G - k0 < kGK ? G - k0 : kGK;
-    float U1 = U;  // two chains
-    for (int kk = 0; kk < kend; kk += 2) {  // an odd kend reads one padded k
-      const float2 a2 = *reinterpret_cast<const float2*>(&sm.f.A[r_loc][kk]);
-      const float2 b2 = *reinterpret_cast<const float2*>(&sm.f.Bt[c_loc][kk]);
-      U = fminf(U, screen_hi(a2.x, b2.x));
-      U1 = fminf(U1, screen_hi(a2.y, b2.y));
+    for (int kk = 0; kk < kc; kk += 4) {
+      float4 x[P], y[Q];
+#pragma unroll
+      for (int p = 0; p < P; ++p) x[p] = *reinterpret_cast<const float4*>(As + (ti + 16 * p) * S + kk);
+#pragma unroll
+      for (int q = 0; q < Q; ++q) y[q] = *reinterpret_cast<const float4*>(Bs + (tc + 16 * q) * S + kk);
+#pragma unroll
+      for (int p = 0; p < P; ++p)
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+          const float m0 = fminf(__fadd_rn(x[p].x, y[q].x), __fadd_rn(x[p].y, y[q].y));
+          const float m1 = fminf(__fadd_rn(x[p].z, y[q].z), __fadd_rn(x[p].w, y[q].w));
+          U[p][q] = fminf(U[p][q], fminf(m0, m1));
+        }
     }
-    U = fminf(U, U1);
-    __syncthreads();
   }
-  if (__syncthreads_or(bad)) {
-    fp64_scan(op, sm, t, i0, c0, ncols, r_loc, c_loc, best, bk);
-  } else {
-    // pass 2: survivors lo_k <= U + d, ascending, up to kMaxSurvivors packed
-    // as 16-bit indices (G <= 16384)
-    const float Ub = __fadd_ru(U, kScreenD);
-    unsigned long long pk = 0;
-    int ns = 0;
-    for (int k0 = 0; k0 < G; k0 += kGK) {
-      if (G > kGK) {  // one tile: pass 1's staging is still in place
-        stage_float(op, sm, t, i0, c0, ncols, k0);
+  const bool range = __syncthreads_or(bad & 1) != 0, neg = __syncthreads_or(bad & 2) != 0;
+  unsigned long long pk[P][Q];  // survivors' indices, 16 bits each (G <= 16384)
+  int ns[P][Q];
+#pragma unroll
+  for (int p = 0; p < P; ++p)
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      pk[p][q] = 0;
+      ns[p][q] = range ? kMaxSurvivors + 1 : 0;
+    }
+  auto push = [&](int p, int q, int k) {
+    if (ns[p][q] < kMaxSurvivors) pk[p][q] |= (unsigned long long)k << (16 * ns[p][q]);
+    ++ns[p][q];
+  };
+  if (!range && !neg) {
+    // s_k - c s_k <= s_min + c s_min + d holds for no s_k above this bound
+    float thr[P][Q];
+#pragma unroll
+    for (int p = 0; p < P; ++p)
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const float ub = __fadd_ru(__fmaf_rn(kScreenC, U[p][q], U[p][q]), kScreenD);
+        thr[p][q] = __fmaf_ru(2.0f * kScreenC, ub, ub);
+      }
+    for (int k0 = 0; k0 < G; k0 += kc) {
+      if (G > kc) {  // one stage: pass 1's is still in place
+        __syncthreads();
+        stage_float<TR, TC>(op, As, Bs, S, t, i0, c0, ncols, k0, kc);
         __syncthreads();
       }
-      const int kend = G - k0 < kGK ? G - k0 : kGK;
-      for (int kk = 0; kk < kend; kk += 2) {
-        const float2 a2 = *reinterpret_cast<const float2*>(&sm.f.A[r_loc][kk]);
-        const float2 b2 = *reinterpret_cast<const float2*>(&sm.f.Bt[c_loc][kk]);
-        if (screen_lo(a2.x, b2.x) <= Ub) {
-          if (ns < kMaxSurvivors) pk |= (unsigned long long)(k0 + kk) << (16 * ns);
-          ++ns;
-        }
-        if (screen_lo(a2.y, b2.y) <= Ub) {  // a padded k never passes
-          if (ns < kMaxSurvivors) pk |= (unsigned long long)(k0 + kk + 1) << (16 * ns);
-          ++ns;
-        }
+      for (int kk = 0; kk < kc; kk += 4) {
+        float4 x[P], y[Q];
+#pragma unroll
+        for (int p = 0; p < P; ++p) x[p] = *reinterpret_cast<const float4*>(As + (ti + 16 * p) * S + kk);
+#pragma unroll
+        for (int q = 0; q < Q; ++q) y[q] = *reinterpret_cast<const float4*>(Bs + (tc + 16 * q) * S + kk);
+#pragma unroll
+        for (int p = 0; p < P; ++p)
+#pragma unroll
+          for (int q = 0; q < Q; ++q) {
+            const float s0 = __fadd_rn(x[p].x, y[q].x), s1 = __fadd_rn(x[p].y, y[q].y);
+            const float s2 = __fadd_rn(x[p].z, y[q].z), s3 = __fadd_rn(x[p].w, y[q].w);
+            if (fminf(fminf(s0, s1), fminf(s2, s3)) <= thr[p][q]) {
+              if (s0 <= thr[p][q]) push(p, q, k0 + kk);
+              if (s1 <= thr[p][q]) push(p, q, k0 + kk + 1);
+              if (s2 <= thr[p][q]) push(p, q, k0 + kk + 2);
+              if (s3 <= thr[p][q]) push(p, q, k0 + kk + 3);
+            }
+          }
       }
-      __syncthreads();
     }
-    if (!valid) return;
-    const double* col = op.bcol(c);
-    long long bestk = LLONG_MAX;
-    const int cnt = ns <= kMaxSurvivors ? ns : G;  // too many survivors: every k
-    for (int r = 0; r < cnt; ++r) {
-      const int k = ns <= kMaxSurvivors ? (int)((pk >> (16 * r)) & 0xffff) : r;
-      const double v = __dadd_rn(op.av(i, k), op.bv(col, k));
-      const long long key = order_key(v);
-      if (key < bestk) {
-        bestk = key;
-        best = v;
-        bk = k;
+  } else if (!range) {
+    // negative operands: the brackets with their own t_k
+#pragma unroll
+    for (int p = 0; p < P; ++p)
+#pragma unroll
+      for (int q = 0; q < Q; ++q) U[p][q] = __int_as_float(0x7f800000);
+    for (int pass = 0; pass < 2; ++pass) {
+      for (int k0 = 0; k0 < G; k0 += kc) {
+        if (G > kc) {
+          __syncthreads();
+          stage_float<TR, TC>(op, As, Bs, S, t, i0, c0, ncols, k0, kc);
+          __syncthreads();
+        }
+        const int kend = G - k0 < kc ? G - k0 : kc;
+        for (int kk = 0; kk < kend; ++kk)
+#pragma unroll
+          for (int p = 0; p < P; ++p)
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+              const float x = As[(ti + 16 * p) * S + kk], y = Bs[(tc + 16 * q) * S + kk];
+              if (pass == 0)
+                U[p][q] = fminf(U[p][q], screen_hi(x, y));
+              else if (screen_lo(x, y) <= __fadd_ru(U[p][q], kScreenD))
+                push(p, q, k0 + kk);
+            }
       }
     }
   }
-  if (!valid) return;
-  const double* col = op.bcol(c);
-  double res = best;
-  if (a.interp && bk > 0 && bk < G - 1) {
-    const double2 gc = tab ? tab[(int64_t)i * G + bk] : curvature(a, op.av(i, bk - 1), op.av(i, bk), op.av(i, bk + 1));
-    res = refine_with(best, gc, curvature(a, op.bv(col, bk - 1), op.bv(col, bk), op.bv(col, bk + 1)));
-  }
-  if (kValues) value_column(a, l, c, X0, X1).out[i] = res;
-  else Om[(int64_t)i * G + c] = res;
-  if (!isfinite(res)) flag(kStatusNonFinite);
+#pragma unroll
+  for (int p = 0; p < P; ++p)
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const int i = i0 + ti + 16 * p;
+      const int64_t c = c0 + tc + 16 * q;
+      if (i >= G || c >= ncols) continue;
+      const double* col = op.bcol(c);
+      double best = 0.0;
+      int bk = 0;
+      long long bestk = LLONG_MAX;
+      const bool listed = ns[p][q] <= kMaxSurvivors;
+      const int cnt = listed ? ns[p][q] : G;  // too many survivors: every k
+      for (int r = 0; r < cnt; ++r) {
+        const int k = listed ? (int)((pk[p][q] >> (16 * r)) & 0xffff) : r;
+        const double v = __dadd_rn(op.av(i, k), op.bv(col, k));
+        const long long key = order_key(v);
+        if (key < bestk) {
+          bestk = key;
+          best = v;
+          bk = k;
+        }
+      }
+      double res = best;
+      if (a.interp && bk > 0 && bk < G - 1) {
+        const double2 gc =
+            tab ? tab[(int64_t)i * G + bk] : curvature(a, op.av(i, bk - 1), op.av(i, bk), op.av(i, bk + 1));
+        res = refine_with(best, gc, curvature(a, op.bv(col, bk - 1), op.bv(col, bk), op.bv(col, bk + 1)));
+      }
+      if (kValues) value_column(a, l, c, X0, X1).out[i] = res;
+      else Om[(int64_t)i * G + c] = res;
+      if (!isfinite(res)) flag(kStatusNonFinite);
+    }
 }
 
 // Row k of the values starts as phi(x_i) = qf x_i^2 / 2 in the buffer it
@@ -408,11 +438,33 @@ int64_t set_count(int64_t T, int l) {
   return full * half + (rem > half ? rem - half : 0);
 }
 
-cudaError_t launch_combine(const GridArgs& a, const double* A, const double* B, double* out, cudaStream_t st) {
-  const dim3 grid(cdiv_u(a.G, kGT), cdiv_u(a.G, kGT));
-  grid_minplus_kernel<false><<<grid, kGT * kGT, 0, st>>>(a, A, B, out, nullptr, nullptr, 0, a.G, nullptr);
+template <int P, int Q, bool kValues>
+cudaError_t launch_tiles(const GridArgs& a, const double* A, const double* B, double* out, double* X0, double* X1,
+                         int l, int64_t ncols, const double2* tab, cudaStream_t st) {
+  const int kc = a.G < kKC ? ((a.G + 3) & ~3) : kKC;
+  const size_t smem = (size_t)(16 * P + 16 * Q) * screen_stride(kc) * sizeof(float);  // at most 88 KB
+  const auto kernel = grid_minplus_kernel<P, Q, kValues>;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const dim3 grid(cdiv_u(ncols, 16 * Q), cdiv_u(a.G, 16 * P));
+  kernel<<<grid, kThreads, smem, st>>>(a, A, B, out, X0, X1, l, ncols, tab);
   count_launch();
   return cudaGetLastError();
+}
+
+// 32 x 64 tiles where they fill the SMs (two CTAs on each of 152), 16 x 16
+// otherwise: a product of two 201 x 201 matrices has 28 of the large tiles and
+// 169 of the small ones.
+template <bool kValues>
+cudaError_t launch_minplus(const GridArgs& a, const double* A, const double* B, double* out, double* X0, double* X1,
+                           int l, int64_t ncols, const double2* tab, cudaStream_t st) {
+  const int64_t large = (int64_t)cdiv_u(ncols, 64) * cdiv_u(a.G, 32);
+  return large >= 2 * 152 ? launch_tiles<2, 4, kValues>(a, A, B, out, X0, X1, l, ncols, tab, st)
+                          : launch_tiles<1, 1, kValues>(a, A, B, out, X0, X1, l, ncols, tab, st);
+}
+
+cudaError_t launch_combine(const GridArgs& a, const double* A, const double* B, double* out, cudaStream_t st) {
+  return launch_minplus<false>(a, A, B, out, nullptr, nullptr, 0, a.G, nullptr, st);
 }
 
 }  // namespace
@@ -470,10 +522,8 @@ cudaError_t run_grid_values(const lqt_grid_problem& p, const double* Vblock, dou
   count_launch();
   for (int l = 0; l < L; ++l) {
     const int64_t nc = set_count(p.T, l);
-    const dim3 grid(cdiv_u(nc, kGT), cdiv_u(p.G, kGT));
-    grid_minplus_kernel<true><<<grid, kGT * kGT, 0, st>>>(a, pw + l * GG, nullptr, nullptr, V, X1, l, nc,
-                                                          p.interp ? tab + l * GG : nullptr);
-    count_launch();
+    e = launch_minplus<true>(a, pw + l * GG, nullptr, nullptr, V, X1, l, nc, p.interp ? tab + l * GG : nullptr, st);
+    if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();
 }
