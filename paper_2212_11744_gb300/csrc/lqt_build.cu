@@ -456,11 +456,26 @@ cudaError_t launch_prepare_coefs(const lqt_problem& p, const Layout& lay, char* 
 // cycles of the FP64 pipe: models made of integrator chains have few nonzeros
 // (the point mass: 2 of 16 in F, 2 of 8 in L; its right-hand side then takes
 // 146 FP64 instructions of 300).  Dense or sampled F, L: every bit set.
-template <int N, int M>
+//
+// ROLE: the fields this thread integrates, kCostSide (eta, J, zeta), kFlowSide
+// (A, b, C) or both.  The cost side is closed in itself and hands P and w on
+// with `give`; the flow side alone takes them with `take`.
+constexpr int kCostSide = 1, kFlowSide = 2, kBothSides = 3;
+
+struct NoExchange {
+  template <int N, int M>
+  __device__ __forceinline__ void give(const double*, const double*) {}
+  template <int N, int M>
+  __device__ __forceinline__ void take(double*, double*) {}
+};
+
+template <int N, int M, int ROLE = kBothSides, class X = NoExchange>
 __device__ __forceinline__ void element_rhs(const Elem<N>& y, const double* __restrict__ F,
                                             const double* __restrict__ c, const double* __restrict__ Lt,
                                             const double* __restrict__ Q, const double* __restrict__ qr,
-                                            Elem<N>& k, unsigned long long nzF, unsigned long long nzL) {
+                                            Elem<N>& k, unsigned long long nzF, unsigned long long nzL,
+                                            X xch = X()) {
+  constexpr bool kFlow = (ROLE & kFlowSide) != 0, kCost = (ROLE & kCostSide) != 0;
   double AL[N * M], P[N * M], w[M];
 #pragma unroll
   for (int e = 0; e < N * M; ++e) AL[e] = P[e] = 0.0;
@@ -474,22 +489,26 @@ __device__ __forceinline__ void element_rhs(const Elem<N>& y, const double* __re
         const double lt = Lt[l * M + a];
 #pragma unroll
         for (int i = 0; i < N; ++i) {
-          AL[i * M + a] = fma(y.A[i * N + l], lt, AL[i * M + a]);
-          P[i * M + a] = fma(y.J[sidx<N>(i, l)], lt, P[i * M + a]);
+          if constexpr (kFlow) AL[i * M + a] = fma(y.A[i * N + l], lt, AL[i * M + a]);
+          if constexpr (kCost) P[i * M + a] = fma(y.J[sidx<N>(i, l)], lt, P[i * M + a]);
         }
-        w[a] = fma(lt, y.eta[l], w[a]);
+        if constexpr (kCost) w[a] = fma(lt, y.eta[l], w[a]);
       }
+  if constexpr (ROLE == kCostSide) xch.template give<N, M>(P, w);
+  if constexpr (ROLE == kFlowSide) xch.template take<N, M>(P, w);
   // dA = AL P^T - A F, JF = J F, deta = -q - F^T eta ...
   double JF[N * N];
 #pragma unroll
   for (int i = 0; i < N; ++i) {
-    k.eta[i] = -qr[i];
+    if constexpr (kCost) k.eta[i] = -qr[i];
 #pragma unroll
     for (int j = 0; j < N; ++j) {
-      double s = 0.0;
+      if constexpr (kFlow) {
+        double s = 0.0;
 #pragma unroll
-      for (int a = 0; a < M; ++a) s = fma(AL[i * M + a], P[j * M + a], s);
-      k.A[i * N + j] = s;
+        for (int a = 0; a < M; ++a) s = fma(AL[i * M + a], P[j * M + a], s);
+        k.A[i * N + j] = s;
+      }
       JF[i * N + j] = 0.0;
     }
   }
@@ -501,118 +520,136 @@ __device__ __forceinline__ void element_rhs(const Elem<N>& y, const double* __re
         const double f = F[l * N + j];
 #pragma unroll
         for (int i = 0; i < N; ++i) {
-          k.A[i * N + j] = fma(-y.A[i * N + l], f, k.A[i * N + j]);
-          JF[i * N + j] = fma(y.J[sidx<N>(i, l)], f, JF[i * N + j]);
+          if constexpr (kFlow) k.A[i * N + j] = fma(-y.A[i * N + l], f, k.A[i * N + j]);
+          if constexpr (kCost) JF[i * N + j] = fma(y.J[sidx<N>(i, l)], f, JF[i * N + j]);
         }
-        k.eta[j] = fma(-f, y.eta[l], k.eta[j]);
+        if constexpr (kCost) k.eta[j] = fma(-f, y.eta[l], k.eta[j]);
       }
-  // db = -AL w - A c
+  if constexpr (kFlow) {
+    // db = -AL w - A c
 #pragma unroll
-  for (int i = 0; i < N; ++i) {
-    double s = 0.0;
-#pragma unroll
-    for (int a = 0; a < M; ++a) s = fma(-AL[i * M + a], w[a], s);
-    if (c) {
-#pragma unroll
-      for (int l = 0; l < N; ++l) s = fma(-y.A[i * N + l], c[l], s);
-    }
-    k.b[i] = s;
-  }
-  // dC = -AL AL^T
-#pragma unroll
-  for (int i = 0; i < N; ++i)
-#pragma unroll
-    for (int j = i; j < N; ++j) {
+    for (int i = 0; i < N; ++i) {
       double s = 0.0;
 #pragma unroll
-      for (int a = 0; a < M; ++a) s = fma(-AL[i * M + a], AL[j * M + a], s);
-      k.C[sidx<N>(i, j)] = s;
-    }
-  // deta ... + J c + P w
+      for (int a = 0; a < M; ++a) s = fma(-AL[i * M + a], w[a], s);
+      if (c) {
 #pragma unroll
-  for (int i = 0; i < N; ++i) {
-    double s = k.eta[i];
+        for (int l = 0; l < N; ++l) s = fma(-y.A[i * N + l], c[l], s);
+      }
+      k.b[i] = s;
+    }
+    // dC = -AL AL^T
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+      for (int j = i; j < N; ++j) {
+        double s = 0.0;
+#pragma unroll
+        for (int a = 0; a < M; ++a) s = fma(-AL[i * M + a], AL[j * M + a], s);
+        k.C[sidx<N>(i, j)] = s;
+      }
+  }
+  if constexpr (kCost) {
+    // deta ... + J c + P w
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      double s = k.eta[i];
+      if (c) {
+#pragma unroll
+        for (int l = 0; l < N; ++l) s = fma(y.J[sidx<N>(i, l)], c[l], s);
+      }
+#pragma unroll
+      for (int a = 0; a < M; ++a) s = fma(P[i * M + a], w[a], s);
+      k.eta[i] = s;
+    }
+    // dJ = -Q - JF - (JF)^T + P P^T
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+      for (int j = i; j < N; ++j) {
+        double s = -Q[i * N + j] - JF[i * N + j] - JF[j * N + i];
+#pragma unroll
+        for (int a = 0; a < M; ++a) s = fma(P[i * M + a], P[j * M + a], s);
+        k.J[sidx<N>(i, j)] = s;
+      }
+    // dzeta
+    double z = -0.5 * qr[N];
+#pragma unroll
+    for (int a = 0; a < M; ++a) z = fma(0.5 * w[a], w[a], z);
     if (c) {
 #pragma unroll
-      for (int l = 0; l < N; ++l) s = fma(y.J[sidx<N>(i, l)], c[l], s);
+      for (int l = 0; l < N; ++l) z = fma(y.eta[l], c[l], z);
     }
-#pragma unroll
-    for (int a = 0; a < M; ++a) s = fma(P[i * M + a], w[a], s);
-    k.eta[i] = s;
+    k.zeta = z;
   }
-  // dJ = -Q - JF - (JF)^T + P P^T
-#pragma unroll
-  for (int i = 0; i < N; ++i)
-#pragma unroll
-    for (int j = i; j < N; ++j) {
-      double s = -Q[i * N + j] - JF[i * N + j] - JF[j * N + i];
-#pragma unroll
-      for (int a = 0; a < M; ++a) s = fma(P[i * M + a], P[j * M + a], s);
-      k.J[sidx<N>(i, j)] = s;
-    }
-  // dzeta
-  double z = -0.5 * qr[N];
-#pragma unroll
-  for (int a = 0; a < M; ++a) z = fma(0.5 * w[a], w[a], z);
-  if (c) {
-#pragma unroll
-    for (int l = 0; l < N; ++l) z = fma(y.eta[l], c[l], z);
-  }
-  k.zeta = z;
 }
 
 // The right-hand side at the boundary A = I, J = 0, eta = 0, where every
 // sub-interval starts.
-template <int N, int M>
+template <int N, int M, int ROLE = kBothSides>
 __device__ __forceinline__ void element_rhs_start(const double* __restrict__ F, const double* __restrict__ c,
                                                   const double* __restrict__ Lt, const double* __restrict__ Q,
                                                   const double* __restrict__ qr, Elem<N>& k) {
+  if constexpr ((ROLE & kFlowSide) != 0) {
 #pragma unroll
-  for (int e = 0; e < N * N; ++e) k.A[e] = 0.0 - F[e];
+    for (int e = 0; e < N * N; ++e) k.A[e] = 0.0 - F[e];
 #pragma unroll
-  for (int i = 0; i < N; ++i) {
-    k.b[i] = c ? 0.0 - c[i] : 0.0;
-    k.eta[i] = -qr[i];
+    for (int i = 0; i < N; ++i) {
+      k.b[i] = c ? 0.0 - c[i] : 0.0;
 #pragma unroll
-    for (int j = i; j < N; ++j) {
-      double s = 0.0;
+      for (int j = i; j < N; ++j) {
+        double s = 0.0;
 #pragma unroll
-      for (int a = 0; a < M; ++a) s = fma(-Lt[i * M + a], Lt[j * M + a], s);
-      k.C[sidx<N>(i, j)] = s;
-      k.J[sidx<N>(i, j)] = -Q[i * N + j];
+        for (int a = 0; a < M; ++a) s = fma(-Lt[i * M + a], Lt[j * M + a], s);
+        k.C[sidx<N>(i, j)] = s;
+      }
     }
   }
-  k.zeta = -0.5 * qr[N];
+  if constexpr ((ROLE & kCostSide) != 0) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      k.eta[i] = -qr[i];
+#pragma unroll
+      for (int j = i; j < N; ++j) k.J[sidx<N>(i, j)] = -Q[i * N + j];
+    }
+    k.zeta = -0.5 * qr[N];
+  }
 }
 
-// y <- base + s * k over every field.
-template <int N>
+// y <- base + s * k over every field of ROLE.
+template <int N, int ROLE = kBothSides>
 __device__ __forceinline__ void axpy_to(Elem<N>& y, const Elem<N>& base, double s, const Elem<N>& k) {
+  if constexpr ((ROLE & kFlowSide) != 0) {
 #pragma unroll
-  for (int i = 0; i < N * N; ++i) y.A[i] = fma(s, k.A[i], base.A[i]);
+    for (int i = 0; i < N * N; ++i) y.A[i] = fma(s, k.A[i], base.A[i]);
 #pragma unroll
-  for (int i = 0; i < N; ++i) {
-    y.b[i] = fma(s, k.b[i], base.b[i]);
-    y.eta[i] = fma(s, k.eta[i], base.eta[i]);
+    for (int i = 0; i < N; ++i) y.b[i] = fma(s, k.b[i], base.b[i]);
+#pragma unroll
+    for (int i = 0; i < Dim<N>::NS; ++i) y.C[i] = fma(s, k.C[i], base.C[i]);
   }
+  if constexpr ((ROLE & kCostSide) != 0) {
 #pragma unroll
-  for (int i = 0; i < Dim<N>::NS; ++i) {
-    y.C[i] = fma(s, k.C[i], base.C[i]);
-    y.J[i] = fma(s, k.J[i], base.J[i]);
+    for (int i = 0; i < N; ++i) y.eta[i] = fma(s, k.eta[i], base.eta[i]);
+#pragma unroll
+    for (int i = 0; i < Dim<N>::NS; ++i) y.J[i] = fma(s, k.J[i], base.J[i]);
+    y.zeta = fma(s, k.zeta, base.zeta);
   }
-  y.zeta = fma(s, k.zeta, base.zeta);
 }
 
 // The same over A, eta and J, which drive the element flow: b, C and zeta
 // appear on no right-hand side, so a stage input needs none of them.
-template <int N>
+template <int N, int ROLE = kBothSides>
 __device__ __forceinline__ void axpy_flow(Elem<N>& y, const Elem<N>& base, double s, const Elem<N>& k) {
+  if constexpr ((ROLE & kFlowSide) != 0) {
 #pragma unroll
-  for (int i = 0; i < N * N; ++i) y.A[i] = fma(s, k.A[i], base.A[i]);
+    for (int i = 0; i < N * N; ++i) y.A[i] = fma(s, k.A[i], base.A[i]);
+  }
+  if constexpr ((ROLE & kCostSide) != 0) {
 #pragma unroll
-  for (int i = 0; i < N; ++i) y.eta[i] = fma(s, k.eta[i], base.eta[i]);
+    for (int i = 0; i < N; ++i) y.eta[i] = fma(s, k.eta[i], base.eta[i]);
 #pragma unroll
-  for (int i = 0; i < Dim<N>::NS; ++i) y.J[i] = fma(s, k.J[i], base.J[i]);
+    for (int i = 0; i < Dim<N>::NS; ++i) y.J[i] = fma(s, k.J[i], base.J[i]);
+  }
 }
 
 struct BuildArgs {
@@ -655,9 +692,9 @@ __device__ __forceinline__ void store_full(const Elem<N>& y, double* dst) {
 // down to s = t_j (Sec. IV-B, eq. abcej_boundary).  With kStages the four
 // stage inputs of every step go to stages[i][0..3] (full layout), for the
 // discrete adjoint's reverse sweep.
-template <int N, int M, bool kStages = false>
+template <int N, int M, bool kStages = false, int ROLE = kBothSides, class X = NoExchange>
 __device__ __forceinline__ void build_one(const Coefs& cf, const double* t, int64_t j, int32_t K, Elem<N>& y,
-                                          double* stages = nullptr) {
+                                          double* stages = nullptr, X xch = X()) {
   constexpr int FS = 3 * N * N + 2 * N + 1;
   const double h = (t[j + 1] - t[j]) / K;
   Elem<N> yn, yt, k;
@@ -695,22 +732,22 @@ __device__ __forceinline__ void build_one(const Coefs& cf, const double* t, int6
     double* st = kStages ? stages + (int64_t)i * 4 * FS : nullptr;
     if constexpr (kStages) store_full<N>(y, st);
     if (i == K - 1)
-      element_rhs_start<N, M>(F[0], c[0], Lt[0], Q[0], qr[0], k);
+      element_rhs_start<N, M, ROLE>(F[0], c[0], Lt[0], Q[0], qr[0], k);
     else
-      element_rhs<N, M>(y, F[0], c[0], Lt[0], Q[0], qr[0], k, nzF, nzL);
-    axpy_to(yn, y, -h / 6.0, k);
-    axpy_flow(yt, y, -0.5 * h, k);
+      element_rhs<N, M, ROLE>(y, F[0], c[0], Lt[0], Q[0], qr[0], k, nzF, nzL, xch);
+    axpy_to<N, ROLE>(yn, y, -h / 6.0, k);
+    axpy_flow<N, ROLE>(yt, y, -0.5 * h, k);
     if constexpr (kStages) store_full<N>(yt, st + FS);
-    element_rhs<N, M>(yt, F[1], c[1], Lt[1], Q[1], qr[1], k, nzF, nzL);
-    axpy_to(yn, yn, -h / 3.0, k);
-    axpy_flow(yt, y, -0.5 * h, k);
+    element_rhs<N, M, ROLE>(yt, F[1], c[1], Lt[1], Q[1], qr[1], k, nzF, nzL, xch);
+    axpy_to<N, ROLE>(yn, yn, -h / 3.0, k);
+    axpy_flow<N, ROLE>(yt, y, -0.5 * h, k);
     if constexpr (kStages) store_full<N>(yt, st + 2 * FS);
-    element_rhs<N, M>(yt, F[1], c[1], Lt[1], Q[1], qr[1], k, nzF, nzL);
-    axpy_to(yn, yn, -h / 3.0, k);
-    axpy_flow(yt, y, -h, k);
+    element_rhs<N, M, ROLE>(yt, F[1], c[1], Lt[1], Q[1], qr[1], k, nzF, nzL, xch);
+    axpy_to<N, ROLE>(yn, yn, -h / 3.0, k);
+    axpy_flow<N, ROLE>(yt, y, -h, k);
     if constexpr (kStages) store_full<N>(yt, st + 3 * FS);
-    element_rhs<N, M>(yt, F[2], c[2], Lt[2], Q[2], qr[2], k, nzF, nzL);
-    axpy_to(y, yn, -h / 6.0, k);
+    element_rhs<N, M, ROLE>(yt, F[2], c[2], Lt[2], Q[2], qr[2], k, nzF, nzL, xch);
+    axpy_to<N, ROLE>(y, yn, -h / 6.0, k);
   }
 }
 
@@ -721,6 +758,68 @@ __global__ void __launch_bounds__(128) build_kernel(BuildArgs a) {
   Elem<N> y;
   build_one<N, M>(a.cf, a.t, j, a.K, y);
   store_public<N>(a.out, j, y);
+}
+
+// The cost side's P = J Lt and w = Lt^T eta of one right-hand side, from the
+// first warp of a 64-thread CTA to the second through one of two buffers in
+// shared memory.  One barrier per right-hand side: a buffer is written again
+// two right-hand sides later, after the barrier of the one between, which the
+// reader reaches only when it has read.
+struct PairExchange {
+  double* buf;    // two buffers of (N M + M) x 32
+  unsigned* odd;  // this thread's count of exchanges, low bit
+  // the two warps meet from different code, so by a named barrier
+  __device__ __forceinline__ void meet() { asm volatile("barrier.sync 1, 64;" ::: "memory"); }
+  template <int N, int M>
+  __device__ __forceinline__ double* slot() {
+    double* p = buf + (*odd & 1u) * ((N * M + M) * 32) + (threadIdx.x & 31);
+    *odd ^= 1u;
+    return p;
+  }
+  template <int N, int M>
+  __device__ __forceinline__ void give(const double* P, const double* w) {
+    double* p = slot<N, M>();
+#pragma unroll
+    for (int e = 0; e < N * M; ++e) p[e * 32] = P[e];
+#pragma unroll
+    for (int a = 0; a < M; ++a) p[(N * M + a) * 32] = w[a];
+    meet();
+  }
+  template <int N, int M>
+  __device__ __forceinline__ void take(double* P, double* w) {
+    meet();
+    const double* p = slot<N, M>();
+#pragma unroll
+    for (int e = 0; e < N * M; ++e) P[e] = p[e * 32];
+#pragma unroll
+    for (int a = 0; a < M; ++a) w[a] = p[(N * M + a) * 32];
+  }
+};
+
+// Two warps per 32 sub-intervals: the first integrates eta, J, zeta, the second
+// A, b, C (about half of the FP64 instructions each), exchanging P and w once
+// per right-hand side.  The results are the same bits as build_kernel's.  A
+// warp alone on its sub-partition waits for its own FP64 results between
+// issues; two warps, and half of the chain, hide that.  Lanes without a
+// sub-interval of their own integrate the last one and store nothing, so that
+// every thread meets every barrier.
+template <int N, int M>
+__global__ void __launch_bounds__(64) build_pair_kernel(BuildArgs a) {
+  __shared__ double buf[2 * (N * M + M) * 32];
+  int64_t j = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);
+  const bool live = j < a.T && !uniform_near(a.cf.uni, a.t, j, a.K);
+  if (!__syncthreads_or(live)) return;
+  if (j >= a.T) j = a.T - 1;
+  unsigned odd = 0;
+  const PairExchange xch{buf, &odd};
+  Elem<N> y;
+  if (threadIdx.x < 32) {
+    build_one<N, M, false, kCostSide>(a.cf, a.t, j, a.K, y, nullptr, xch);
+    if (live) store_public_cost<N>(a.out, j, y);
+  } else {
+    build_one<N, M, false, kFlowSide>(a.cf, a.t, j, a.K, y, nullptr, xch);
+    if (live) store_public_flow<N>(a.out, j, y);
+  }
 }
 
 // The same for sub-intervals j0 .. j0 + T - 1 (a.T counts the range), writing
@@ -931,15 +1030,31 @@ cudaError_t batch_build(const BatchDev& bd, const ElemPtrs& el, char* team_scrat
   return cudaGetLastError();
 }
 
+// Two warps per 32 sub-intervals up to this T for n = 2..4, one thread each
+// beyond, where the sub-partitions have several warps either way.  Whole element
+// builds on an uneven grid, one thread -> two warps: n = 4, m = 2, K = 10: 681
+// -> 521 us at T = 10007, 2385 -> 2089 at 60000, 6451 -> 6089 at 200000, 15154
+// -> 15362 at 500000; n = 3, m = 2, K = 4: 187 -> 122 at 2048, 576 -> 518 at
+// 60000; n = 2, m = 1, K = 10: 167 -> 125 at 2048, 519 -> 502 at 60000, 1331 ->
+// 1344 at 200000.  n = 1 has too little to share (60 -> 64 at 10007).
+constexpr int64_t kPairMaxT = 1 << 17;
+
 template <int N, int M>
 static void launch_build_nm(const BuildArgs& a, cudaStream_t st, double* stages, int64_t j0) {
   const int threads = 128;
   const int64_t blocks = (a.T + threads - 1) / threads;
-  if (stages)
-    build_stages_kernel<N, M><<<(unsigned)blocks, threads, 0, st>>>(a, j0, stages);
-  else
-    build_kernel<N, M><<<(unsigned)blocks, threads, 0, st>>>(a);
   count_launch();
+  if (stages) {
+    build_stages_kernel<N, M><<<(unsigned)blocks, threads, 0, st>>>(a, j0, stages);
+    return;
+  }
+  if constexpr (N >= 2 && N <= 4) {
+    if (a.T <= kPairMaxT) {
+      build_pair_kernel<N, M><<<(unsigned)((a.T + 31) / 32), 64, 0, st>>>(a);
+      return;
+    }
+  }
+  build_kernel<N, M><<<(unsigned)blocks, threads, 0, st>>>(a);
 }
 
 template <int N>

@@ -147,27 +147,37 @@ __device__ __forceinline__ void load_public(const ElemPtrs& el, int64_t k, Elem<
 }
 
 template <int N>
-__device__ __forceinline__ void store_public(const ElemPtrs& el, int64_t k, const Elem<N>& e) {
+__device__ __forceinline__ void store_public_flow(const ElemPtrs& el, int64_t k, const Elem<N>& e) {
   double* A = el.A + k * N * N;
   double* b = el.b + k * N;
   double* C = el.C + k * N * N;
-  double* eta = el.eta + k * N;
-  double* J = el.J + k * N * N;
 #pragma unroll
   for (int i = 0; i < N * N; ++i) A[i] = e.A[i];
 #pragma unroll
-  for (int i = 0; i < N; ++i) {
-    b[i] = e.b[i];
-    eta[i] = e.eta[i];
-  }
+  for (int i = 0; i < N; ++i) b[i] = e.b[i];
 #pragma unroll
   for (int i = 0; i < N; ++i)
 #pragma unroll
-    for (int j = 0; j < N; ++j) {
-      C[i * N + j] = e.C[sidx<N>(i, j)];
-      J[i * N + j] = e.J[sidx<N>(i, j)];
-    }
+    for (int j = 0; j < N; ++j) C[i * N + j] = e.C[sidx<N>(i, j)];
+}
+
+template <int N>
+__device__ __forceinline__ void store_public_cost(const ElemPtrs& el, int64_t k, const Elem<N>& e) {
+  double* eta = el.eta + k * N;
+  double* J = el.J + k * N * N;
+#pragma unroll
+  for (int i = 0; i < N; ++i) eta[i] = e.eta[i];
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+#pragma unroll
+    for (int j = 0; j < N; ++j) J[i * N + j] = e.J[sidx<N>(i, j)];
   if (el.zeta) el.zeta[k] = e.zeta;
+}
+
+template <int N>
+__device__ __forceinline__ void store_public(const ElemPtrs& el, int64_t k, const Elem<N>& e) {
+  store_public_flow<N>(el, k, e);
+  store_public_cost<N>(el, k, e);
 }
 
 // Full-matrix record layouts shared with the team kernels (lqt_team.cuh):
