@@ -253,9 +253,9 @@ __device__ __forceinline__ int stage_float(const Operands<kValues>& op, float* A
 // output, by some 30 FP64 instructions of the refinement (its three divisions)
 // at 64 cycles each.  One output per thread, with staging again in the second
 // pass, took 4.43 ms for the block and the values at G = 201, T = 10^4; this
-// 3.09 ms (13 levels of about 5000 columns at 0.2 ms each).
+// 2.82 ms; 2 x 4 outputs and two CTAs on an SM 3.09.
 template <int P, int Q, bool kValues>
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(kThreads, P * Q <= 4 ? 3 : 2)
     grid_minplus_kernel(GridArgs a, const double* __restrict__ A, const double* Bm, double* Om, double* X0,
                         double* X1, int l, int64_t ncols, const double2* __restrict__ tab) {
   constexpr int TR = 16 * P, TC = 16 * Q;
@@ -442,7 +442,7 @@ template <int P, int Q, bool kValues>
 cudaError_t launch_tiles(const GridArgs& a, const double* A, const double* B, double* out, double* X0, double* X1,
                          int l, int64_t ncols, const double2* tab, cudaStream_t st) {
   const int kc = a.G < kKC ? ((a.G + 3) & ~3) : kKC;
-  const size_t smem = (size_t)(16 * P + 16 * Q) * screen_stride(kc) * sizeof(float);  // at most 88 KB
+  const size_t smem = (size_t)(16 * P + 16 * Q) * screen_stride(kc) * sizeof(float);  // at most 58 KB
   const auto kernel = grid_minplus_kernel<P, Q, kValues>;
   const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -452,14 +452,15 @@ cudaError_t launch_tiles(const GridArgs& a, const double* A, const double* B, do
   return cudaGetLastError();
 }
 
-// 32 x 64 tiles where they fill the SMs (two CTAs on each of 152), 16 x 16
-// otherwise: a product of two 201 x 201 matrices has 28 of the large tiles and
-// 169 of the small ones.
+// 32 x 32 tiles where they fill the SMs (three CTAs on each of 152, so that one
+// CTA's FP64 refinement runs beside another's screen), 16 x 16 otherwise: a
+// product of two 201 x 201 matrices has 49 of the large tiles and 169 of the
+// small ones.
 template <bool kValues>
 cudaError_t launch_minplus(const GridArgs& a, const double* A, const double* B, double* out, double* X0, double* X1,
                            int l, int64_t ncols, const double2* tab, cudaStream_t st) {
-  const int64_t large = (int64_t)cdiv_u(ncols, 64) * cdiv_u(a.G, 32);
-  return large >= 2 * 152 ? launch_tiles<2, 4, kValues>(a, A, B, out, X0, X1, l, ncols, tab, st)
+  const int64_t large = (int64_t)cdiv_u(ncols, 32) * cdiv_u(a.G, 32);
+  return large >= 3 * 152 ? launch_tiles<2, 2, kValues>(a, A, B, out, X0, X1, l, ncols, tab, st)
                           : launch_tiles<1, 1, kValues>(a, A, B, out, X0, X1, l, ncols, tab, st);
 }
 

@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("G,T", [
-    (31, 20001), (33, 19999), (65, 14001),  # 1, 2, 3 rows of 32 x 64 tiles, ragged columns
+    (31, 20001), (33, 19999), (65, 14001),  # 1, 2, 3 rows of large tiles, ragged columns
     (224, 5600), (225, 4900), (300, 4000),  # one stage, one stage and 1, one stage and 76
 ])
 @pytest.mark.parametrize("qf", [4.0, -1.0])
@@ -29,7 +29,7 @@ def test_values_in_large_tiles(G, T, qf):
     same(got, oracle.grid_values(g, Vb), "values")
 
 
-@pytest.mark.parametrize("G", [15, 17, 223, 226, 449, 1100])  # 1100: 35 x 18 large tiles
+@pytest.mark.parametrize("G", [15, 17, 223, 226, 449, 1100])  # 1100: 35 x 35 large tiles
 @pytest.mark.parametrize("kind", ["positive", "signs", "range", "zeros"])
 def test_combine_at_tile_edges(G, kind):
     import paper_2212_11744_gb300 as lqt
