@@ -76,6 +76,9 @@ static Layout make_layout(const lqt_problem& p) {
   L.uniform = uniform_eligible(p);
   L.off_uni = off;
   if (L.uniform) off += uniform_table_bytes(p.n, L.M);
+  L.off_repeat = off;
+  L.repeat_bytes = team_repeat_bytes(p, L.M, L.uniform);
+  off = align_up(off + L.repeat_bytes);
   L.coef_bytes = off;
   return L;
 }

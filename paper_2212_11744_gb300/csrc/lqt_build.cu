@@ -427,6 +427,7 @@ Coefs coefs_view(const lqt_problem& p, const Layout& lay, double* Lt, double* Q,
   cf.Ku_per_boundary = ku_const ? 0 : 1;
   cf.M = lay.M;
   cf.uni = nullptr;
+  cf.repeat = nullptr;
   return cf;
 }
 
@@ -434,6 +435,7 @@ cudaError_t launch_prepare_coefs(const lqt_problem& p, const Layout& lay, char* 
   const cudaError_t e = launch_prepare_into(p, lay, (double*)(ws + lay.off_Lt), (double*)(ws + lay.off_Q),
                                             (double*)(ws + lay.off_qr), (double*)(ws + lay.off_Ku), cf, st);
   if (lay.uniform) cf.uni = (const double*)(ws + lay.off_uni);
+  if (lay.repeat_bytes) cf.repeat = ws + lay.off_repeat;
   return e;
 }
 

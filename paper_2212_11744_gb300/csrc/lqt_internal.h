@@ -64,6 +64,8 @@ struct Coefs {
   // table of the constant-coefficient build (lqt_uniform.cu); NULL: the
   // general build makes every element
   const double* uni;
+  // workspace of the build by repeated lengths (lqt_team.cu), n = 64; NULL: none
+  char* repeat;
 };
 
 struct ElemPtrs {
@@ -78,6 +80,7 @@ struct Layout {
   // byte offsets inside the workspace
   size_t off_Lt, off_Q, off_qr, off_Ku, off_uni;
   bool uniform;  // the constant-coefficient build applies (lqt_uniform.cu)
+  size_t off_repeat, repeat_bytes;  // the build by repeated lengths (0 bytes: does not apply)
   size_t coef_bytes;  // end of the coefficient region
 };
 
@@ -111,6 +114,7 @@ cudaError_t launch_build_stages_range(const lqt_problem& p, const Layout& lay, c
 // the table (cf.uni) from the grid's mean step, then the elements of the
 // sub-intervals that have it; the general build makes the others.
 bool uniform_eligible(const lqt_problem& p);
+size_t team_repeat_bytes(const lqt_problem& p, int32_t M, bool eligible);
 int64_t uniform_table_doubles(int n, int M);
 size_t uniform_table_bytes(int n, int M);
 cudaError_t launch_uniform_master(const lqt_problem& p, const Coefs& cf, cudaStream_t st);

@@ -144,11 +144,11 @@ __device__ void store_stage(int lane, double* dst, Rec<N> src, bool full) {
 // Element j of a problem (coefficients cf, grid t) into the packed record at
 // yb; the other buffers are scratch.  With `stages`, the four stage inputs of
 // RK4 step i go to stages + (i 4 + s) (3N^2 + 2N + 1), s = 0..3, in the full
-// layout.
+// layout.  With `ap`, the products AL and P of stage s go to ap + (i 4 + s) 2 N M.
 template <int N, int M>
 __device__ void team_build_one(int lane, const Coefs& cf, const double* t, int64_t j, int32_t K, double* yb,
-                               double* ynb, double* ytb, double* kb, double* AL, double* P, double* w,
-                               double* stages = nullptr) {
+                               double* ynb, double* ytb, double* kb, double* AL, double* w,
+                               double* stages = nullptr, double* ap = nullptr) {
   constexpr int TEAM = TeamCfg<N>::TEAM;
   constexpr int FS = Rec<N>::SIZE;
   const Rec<N> y = Rec<N>::packed(yb), yn = Rec<N>::flow(ynb), yt = Rec<N>::flow(ytb), k = Rec<N>::flow(kb);
@@ -166,22 +166,23 @@ __device__ void team_build_one(int lane, const Coefs& cf, const double* t, int64
       Q[q] = cf.Q.ptr + sample_index(cf.Q.mode, j, ps[q], K) * N * N;
       qr[q] = cf.qr.ptr + sample_index(cf.qr.mode, j, ps[q], K) * (N + 1);
     }
+    auto al = [&](int s) { return ap ? ap + ((int64_t)i * 4 + s) * (2 * N * M) : AL; };
     // (A, eta, J) by classical RK4 through yn and yt; b, C, zeta accumulated
     // into y by the right-hand side
     if (st) store_stage<N, TEAM>(lane, st, y, true);
-    team::rhs<N, M, TEAM>(lane, y, k, F[0], c[0], Lt[0], Q[0], qr[0], AL, P, w, -h / 6.0, y);
+    team::rhs<N, M, TEAM>(lane, y, k, F[0], c[0], Lt[0], Q[0], qr[0], al(0), al(0) + N * M, w, -h / 6.0, y);
     team::axpy_flow<N, TEAM>(lane, yn, y, -h / 6.0, k);
     team::axpy_flow<N, TEAM>(lane, yt, y, -0.5 * h, k);
     if (st) store_stage<N, TEAM>(lane, st + FS, yt, false);
-    team::rhs<N, M, TEAM>(lane, yt, k, F[1], c[1], Lt[1], Q[1], qr[1], AL, P, w, -h / 3.0, y);
+    team::rhs<N, M, TEAM>(lane, yt, k, F[1], c[1], Lt[1], Q[1], qr[1], al(1), al(1) + N * M, w, -h / 3.0, y);
     team::axpy_flow<N, TEAM>(lane, yn, yn, -h / 3.0, k);
     team::axpy_flow<N, TEAM>(lane, yt, y, -0.5 * h, k);
     if (st) store_stage<N, TEAM>(lane, st + 2 * FS, yt, false);
-    team::rhs<N, M, TEAM>(lane, yt, k, F[1], c[1], Lt[1], Q[1], qr[1], AL, P, w, -h / 3.0, y);
+    team::rhs<N, M, TEAM>(lane, yt, k, F[1], c[1], Lt[1], Q[1], qr[1], al(2), al(2) + N * M, w, -h / 3.0, y);
     team::axpy_flow<N, TEAM>(lane, yn, yn, -h / 3.0, k);
     team::axpy_flow<N, TEAM>(lane, yt, y, -h, k);
     if (st) store_stage<N, TEAM>(lane, st + 3 * FS, yt, false);
-    team::rhs<N, M, TEAM>(lane, yt, k, F[2], c[2], Lt[2], Q[2], qr[2], AL, P, w, -h / 6.0, y);
+    team::rhs<N, M, TEAM>(lane, yt, k, F[2], c[2], Lt[2], Q[2], qr[2], al(3), al(3) + N * M, w, -h / 6.0, y);
     team::axpy_flow<N, TEAM>(lane, y, yn, -h / 6.0, k);
   }
 }
@@ -197,11 +198,10 @@ __global__ void __launch_bounds__(TeamCfg<N>::TEAM, TeamCfg<N>::BUILD_MIN) build
   double* ytb = ynb + Rec<N>::FLOW;
   double* kb = ytb + Rec<N>::FLOW;
   double* AL = kb + Rec<N>::FLOW;
-  double* P = AL + N * M;
-  double* w = P + N * M;
+  double* w = AL + 2 * N * M;
   for (int64_t j = blockIdx.x; j < a.T; j += gridDim.x) {
     if (uniform_near(a.cf.uni, a.t, j, a.K)) continue;  // written by the constant-coefficient build
-    team_build_one<N, M>(lane, a.cf, a.t, j, a.K, yb, ynb, ytb, kb, AL, P, w);
+    team_build_one<N, M>(lane, a.cf, a.t, j, a.K, yb, ynb, ytb, kb, AL, w);
     double zz = 0.0;
     Rec<N> dst = Rec<N>::pub(a.out, j, &zz);
     team::copy_rec<N, TEAM>(lane, dst, Rec<N>::packed(yb));
@@ -226,16 +226,174 @@ __global__ void __launch_bounds__(TeamCfg<N>::TEAM) build_team_range_kernel(Team
   double* ytb = ynb + Rec<N>::FLOW;
   double* kb = ytb + Rec<N>::FLOW;
   double* AL = kb + Rec<N>::FLOW;
-  double* P = AL + N * M;
-  double* w = P + N * M;
+  double* w = AL + 2 * N * M;
   for (int64_t jj = blockIdx.x; jj < a.T; jj += gridDim.x) {
     if (uniform_near(a.cf.uni, a.t, j0 + jj, a.K)) continue;
-    team_build_one<N, M>(lane, a.cf, a.t, j0 + jj, a.K, yb, ynb, ytb, kb, AL, P, w,
+    team_build_one<N, M>(lane, a.cf, a.t, j0 + jj, a.K, yb, ynb, ytb, kb, AL, w,
                          stages ? stages + jj * (int64_t)a.K * 4 * Rec<N>::SIZE : nullptr);
     if (a.out.A) {
       double zz = 0.0;
       team::copy_rec<N, TEAM>(lane, Rec<N>::pub(a.out, j0 + jj, &zz), Rec<N>::packed(yb));
     }
+  }
+}
+
+// Constant F, L, U, X without drift: A, C and J of a sub-interval depend on its
+// length alone, so sub-intervals of one length, to the last bit, have them alike
+// to the last bit (a grid of equal steps has some twenty lengths by the rounding
+// of its boundaries).  The first of each length integrates all fields and keeps
+// its stages' AL and P; every other one copies A, C, J and integrates b, eta and
+// zeta, 1/30 of the operations, by the same expressions in the same order: all
+// elements are the bits of build_team_kernel's, which the mixed-precision solve
+// needs.  Bound by one element's integration by one CTA (1.9 ms at K = 2).  The
+// mixed solve at n = 64, T = 1000, K = 2: 29.4 ms element by element (13.1 of
+// them the build), 18.4 so.
+constexpr int64_t kRepeatMaxT = 4096;  // the search compares every pair
+constexpr int32_t kRepeatMaxK = 8;
+constexpr int kRepeatSlots = 152;  // lengths that keep AL and P; others: element by element
+
+struct Repeats {
+  int32_t *first;  // the first sub-interval of the same length
+  int32_t *slot;   // its AL, P slot; -1: none
+  int32_t *list;   // the sub-intervals that integrate all fields
+  int32_t *count;
+  double* ap;      // kRepeatSlots x 4 K x 2 N M
+};
+
+static size_t repeat_ints(int64_t T) { return ((size_t)(3 * T + 1) * sizeof(int32_t) + 255) / 256 * 256; }
+
+// Workspace of the search and the kept products; 0: not applicable.
+size_t team_repeat_bytes(const lqt_problem& p, int32_t M, bool eligible) {
+  if (!eligible || p.n != 64 || p.T > kRepeatMaxT || p.K > kRepeatMaxK) return 0;
+  const size_t slots = (size_t)std::min<int64_t>(p.T, kRepeatSlots);
+  return repeat_ints(p.T) + slots * 4 * (size_t)p.K * 2 * p.n * M * sizeof(double);
+}
+
+static Repeats carve_repeats(char* base, int64_t T) {
+  int32_t* q = (int32_t*)base;
+  return Repeats{q, q + T, q + 2 * T, q + 3 * T, (double*)(base + repeat_ints(T))};
+}
+
+__global__ void __launch_bounds__(128) repeat_find_kernel(int64_t T, const double* t, Repeats r) {
+  __shared__ long long len[kRepeatMaxT];
+  const int64_t j = (int64_t)blockIdx.x * 128 + threadIdx.x;
+  const int64_t end = (int64_t)(blockIdx.x + 1) * 128 < T ? (int64_t)(blockIdx.x + 1) * 128 : T;
+  for (int64_t q = threadIdx.x; q < end; q += 128) len[q] = __double_as_longlong(t[q + 1] - t[q]);
+  __syncthreads();
+  if (j >= T) return;
+  const long long mine = len[j];
+  int32_t f = 0;
+  while (len[f] != mine) ++f;  // at the latest at j
+  r.first[j] = f;
+}
+
+// Slots in the order of first occurrence, then the list; one CTA of 1024, each
+// thread a run of at most kRepeatMaxT / 1024 sub-intervals.
+__global__ void __launch_bounds__(1024) repeat_list_kernel(int32_t T, Repeats r) {
+  __shared__ int32_t sums[1024];
+  const int tid = threadIdx.x, run = (T + 1023) / 1024;
+  const int j0 = tid * run, j1 = min(j0 + run, T);
+  for (int pass = 0; pass < 2; ++pass) {
+    auto counts = [&](int j) { return r.first[j] == j || (pass == 1 && r.slot[r.first[j]] < 0); };
+    int32_t c = 0;
+    for (int j = j0; j < j1; ++j) c += counts(j) ? 1 : 0;
+    sums[tid] = c;
+    __syncthreads();
+    for (int d = 1; d < 1024; d *= 2) {
+      const int32_t v = tid >= d ? sums[tid - d] : 0;
+      __syncthreads();
+      sums[tid] += v;
+      __syncthreads();
+    }
+    int32_t at = sums[tid] - c;
+    for (int j = j0; j < j1; ++j) {
+      const bool on = counts(j);
+      if (pass == 0) r.slot[j] = on && at < kRepeatSlots ? at : -1;
+      else if (on) r.list[at] = j;
+      at += on ? 1 : 0;
+    }
+    if (pass == 1 && tid == 1023) *r.count = sums[1023];
+    __syncthreads();
+  }
+}
+
+template <int N, int M>
+__global__ void __launch_bounds__(TeamCfg<N>::TEAM, TeamCfg<N>::BUILD_MIN)
+    build_team_list_kernel(TeamBuildArgs a, Repeats r) {
+  constexpr int TEAM = TeamCfg<N>::TEAM;
+  const int lane = threadIdx.x;
+  double* yb = slot_base<N>(a.gscratch, build_slot_doubles<N, M>());
+  double* ynb = yb + Rec<N>::SIZE;
+  double* ytb = ynb + Rec<N>::FLOW;
+  double* kb = ytb + Rec<N>::FLOW;
+  double* AL = kb + Rec<N>::FLOW;
+  double* w = AL + 2 * N * M;
+  const int count = *r.count;
+  for (int i = blockIdx.x; i < count; i += gridDim.x) {
+    const int64_t j = r.list[i];
+    const int s = r.slot[j];
+    team_build_one<N, M>(lane, a.cf, a.t, j, a.K, yb, ynb, ytb, kb, AL, w, nullptr,
+                         s >= 0 ? r.ap + (int64_t)s * a.K * 4 * (2 * N * M) : nullptr);
+    double zz = 0.0;
+    team::copy_rec<N, TEAM>(lane, Rec<N>::pub(a.out, j, &zz), Rec<N>::packed(yb));
+  }
+}
+
+template <int N, int M>
+__global__ void __launch_bounds__(TeamCfg<N>::TEAM) repeat_vectors_kernel(TeamBuildArgs a, Repeats r) {
+  constexpr int TEAM = TeamCfg<N>::TEAM;
+  __shared__ double w[M], b[N], zeta, y[N], yn[N], yt[N], k[N];
+  const int lane = threadIdx.x;
+  const double *F = a.cf.F.ptr, *Lt = a.cf.Lt.ptr;
+  for (int64_t j = blockIdx.x; j < a.T; j += gridDim.x) {
+    const int64_t f = r.first[j];
+    const int s = r.slot[f];
+    if (f == j || s < 0) continue;
+    for (int e = lane; e < N * N; e += TEAM) {
+      a.out.A[j * N * N + e] = a.out.A[f * N * N + e];
+      a.out.C[j * N * N + e] = a.out.C[f * N * N + e];
+      a.out.J[j * N * N + e] = a.out.J[f * N * N + e];
+    }
+    for (int e = lane; e < N; e += TEAM) b[e] = y[e] = 0.0;
+    if (lane == 0) zeta = 0.0;
+    const double* qr = a.cf.qr.ptr + sample_index(a.cf.qr.mode, j, 0, a.K) * (N + 1);
+    const double h = (a.t[j + 1] - a.t[j]) / a.K;
+    team::sync<TEAM>();
+    for (int32_t i = a.K - 1; i >= 0; --i) {
+      const double* ap = r.ap + ((int64_t)s * a.K + i) * 4 * (2 * N * M);
+      auto stage = [&](const double* eta, double sq) {
+        team::rhs_w<N, M, TEAM>(lane, Lt, eta, w);
+        team::sync<TEAM>();
+        team::rhs_b_eta<N, M, TEAM>(lane, nullptr, nullptr, eta, F, nullptr, ap, ap + N * M, w, qr, sq, b, k);
+        team::rhs_zeta<N, M, TEAM>(lane, eta, nullptr, w, qr, sq, &zeta);
+        ap += 2 * N * M;
+        team::sync<TEAM>();
+      };
+      auto axpy = [&](double* out, const double* base, double c) {
+        for (int e = lane; e < N; e += TEAM) out[e] = fma(c, k[e], base[e]);
+      };
+      stage(y, -h / 6.0);
+      axpy(yn, y, -h / 6.0);
+      axpy(yt, y, -0.5 * h);
+      team::sync<TEAM>();
+      stage(yt, -h / 3.0);
+      axpy(yn, yn, -h / 3.0);
+      axpy(yt, y, -0.5 * h);
+      team::sync<TEAM>();
+      stage(yt, -h / 3.0);
+      axpy(yn, yn, -h / 3.0);
+      axpy(yt, y, -h);
+      team::sync<TEAM>();
+      stage(yt, -h / 6.0);
+      axpy(y, yn, -h / 6.0);
+      team::sync<TEAM>();
+    }
+    for (int e = lane; e < N; e += TEAM) {
+      a.out.b[j * N + e] = b[e];
+      a.out.eta[j * N + e] = y[e];
+    }
+    if (lane == 0 && a.out.zeta) a.out.zeta[j] = zeta;
+    team::sync<TEAM>();
   }
 }
 
@@ -252,15 +410,14 @@ __global__ void __launch_bounds__(TeamCfg<N>::TEAM, TeamCfg<N>::BUILD_MIN)
   double* ytb = ynb + Rec<N>::FLOW;
   double* kb = ytb + Rec<N>::FLOW;
   double* AL = kb + Rec<N>::FLOW;
-  double* P = AL + N * M;
-  double* w = P + N * M;
+  double* w = AL + 2 * N * M;
   for (int64_t g = blockIdx.x; g < bd.total; g += gridDim.x) {
     const int32_t b = batch_find(bd.off, bd.B, g);
     const BatchProb& pb = bd.probs[b];
     const int64_t j = g - pb.off;
     if (j < pb.T) {
       if (uniform_near(pb.cf.uni, pb.t, j, bd.K)) continue;
-      team_build_one<N, M>(lane, pb.cf, pb.t, j, bd.K, yb, ynb, ytb, kb, AL, P, w);
+      team_build_one<N, M>(lane, pb.cf, pb.t, j, bd.K, yb, ynb, ytb, kb, AL, w);
     } else {
       const Rec<N> y = Rec<N>::packed(yb);
       for (int e = lane; e < Rec<N>::SIZE; e += TEAM) yb[e] = 0.0;
@@ -1014,6 +1171,17 @@ template <int N, int M>
 static cudaError_t team_build_nm(const lqt_problem& p, const Coefs& cf, const ElemPtrs& out, double* gscratch,
                                  cudaStream_t st) {
   TeamBuildArgs a{p.T, p.K, p.t, cf, out, gscratch};
+  if constexpr (N == 64) {
+    if (cf.repeat && !cf.uni) {
+      const Repeats r = carve_repeats(cf.repeat, p.T);
+      repeat_find_kernel<<<(unsigned)((p.T + 127) / 128), 128, 0, st>>>(p.T, p.t, r);
+      repeat_list_kernel<<<1, 1024, 0, st>>>((int32_t)p.T, r);
+      team_launch<N>(build_team_list_kernel<N, M>, p.T, build_slot_doubles<N, M>(), a, st, TeamCfg<N>::BUILD_SLOTS, r);
+      repeat_vectors_kernel<N, M><<<(unsigned)std::min<int64_t>(p.T, 152 * 4), TeamCfg<N>::TEAM, 0, st>>>(a, r);
+      count_launch(3);
+      return cudaGetLastError();
+    }
+  }
   team_launch<N>(build_team_kernel<N, M>, p.T, build_slot_doubles<N, M>(), a, st, TeamCfg<N>::BUILD_SLOTS);
   return cudaGetLastError();
 }

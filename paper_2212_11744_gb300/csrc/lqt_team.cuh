@@ -172,6 +172,63 @@ __host__ __device__ constexpr int split_lanes(int outputs, int team) {
   return s;
 }
 
+// The vector parts of the right-hand side below.  w = Lt^T eta:
+template <int N, int M, int TEAM>
+__device__ __forceinline__ void rhs_w(int lane, const double* __restrict__ Lt, const double* eta, double* w) {
+  constexpr int S = split_lanes(M, TEAM);
+  const int o = lane / S, sub = lane % S;
+  double s = 0.0;
+  if (o < M)
+    for (int l = sub; l < N; l += S) s = fma(Lt[l * M + o], eta[l], s);
+  s = group_sum<S>(s);
+  if (sub == 0 && o < M) w[o] = s;
+}
+
+// db = -AL w - A c, accumulated times sq; deta = -q - F^T eta + J c + P w.  A and
+// J are read only where there is a drift.
+template <int N, int M, int TEAM>
+__device__ __forceinline__ void rhs_b_eta(int lane, const double* A, const double* J, const double* eta,
+                                          const double* __restrict__ F, const double* __restrict__ c,
+                                          const double* AL, const double* P, const double* w,
+                                          const double* __restrict__ qr, double sq, double* bacc, double* keta) {
+  constexpr int S = split_lanes(N, TEAM);
+  const int o = lane / S, sub = lane % S;
+  double s = 0.0, se = 0.0;
+  if (o < N) {
+    if (sub == 0) se = -qr[o];
+    for (int a = sub; a < M; a += S) {
+      s = fma(-AL[o * M + a], w[a], s);
+      se = fma(P[o * M + a], w[a], se);
+    }
+    for (int l = sub; l < N; l += S) se = fma(-F[l * N + o], eta[l], se);
+    if (c)
+      for (int l = sub; l < N; l += S) {
+        s = fma(-A[o * N + l], c[l], s);
+        se = fma(J[o * N + l], c[l], se);
+      }
+  }
+  s = group_sum<S>(s);
+  se = group_sum<S>(se);
+  if (sub == 0 && o < N) {
+    bacc[o] = fma(sq, s, bacc[o]);
+    keta[o] = se;
+  }
+}
+
+// dzeta = -rho/2 + |w|^2/2 + eta^T c, over the first warp, accumulated times sq.
+template <int N, int M, int TEAM>
+__device__ __forceinline__ void rhs_zeta(int lane, const double* eta, const double* __restrict__ c, const double* w,
+                                         const double* __restrict__ qr, double sq, double* zacc) {
+  if (lane < 32) {
+    double z = 0.0;
+    for (int a = lane; a < M; a += 32) z = fma(0.5 * w[a], w[a], z);
+    if (c)
+      for (int l = lane; l < N; l += 32) z = fma(eta[l], c[l], z);
+    z = group_sum<32>(z);
+    if (lane == 0) *zacc = fma(sq, z - 0.5 * qr[N], *zacc);
+  }
+}
+
 // k = f(y) for the flow fields (A, eta, J); the quadrature fields' rates
 // (db, dC, dzeta: nothing reads b, C or zeta) are added, times the RK4 weight
 // sq, straight into qacc's b, C, zeta, in the order the four-stage sum takes
@@ -222,15 +279,7 @@ __device__ void rhs(int lane, Rec<N> y, Rec<N> k, const double* __restrict__ F, 
     P[e] = s2;
   }
   }
-  {  // w = Lt^T eta
-    constexpr int S = split_lanes(M, TEAM);
-    const int o = lane / S, sub = lane % S;
-    double s = 0.0;
-    if (o < M)
-      for (int l = sub; l < N; l += S) s = fma(Lt[l * M + o], eta[l], s);
-    s = group_sum<S>(s);
-    if (sub == 0 && o < M) w[o] = s;
-  }
+  rhs_w<N, M, TEAM>(lane, Lt, eta, w);
   sync<TEAM>();
   constexpr int NS = N * (N + 1) / 2;
   // dA = AL P^T - A F
@@ -251,30 +300,7 @@ __device__ void rhs(int lane, Rec<N> y, Rec<N> k, const double* __restrict__ F, 
       k.A()[t] = s;
     }
   }
-  {  // db = -AL w - A c ; deta = -q - F^T eta + J c + P w
-    constexpr int S = split_lanes(N, TEAM);
-    const int o = lane / S, sub = lane % S;
-    double s = 0.0, se = 0.0;
-    if (o < N) {
-      if (sub == 0) se = -qr[o];
-      for (int a = sub; a < M; a += S) {
-        s = fma(-AL[o * M + a], w[a], s);
-        se = fma(P[o * M + a], w[a], se);
-      }
-      for (int l = sub; l < N; l += S) se = fma(-F[l * N + o], eta[l], se);
-      if (c)
-        for (int l = sub; l < N; l += S) {
-          s = fma(-A[o * N + l], c[l], s);
-          se = fma(J[o * N + l], c[l], se);
-        }
-    }
-    s = group_sum<S>(s);
-    se = group_sum<S>(se);
-    if (sub == 0 && o < N) {
-      qacc.b()[o] = fma(sq, s, qacc.b()[o]);
-      k.eta()[o] = se;
-    }
-  }
+  rhs_b_eta<N, M, TEAM>(lane, A, J, eta, F, c, AL, P, w, qr, sq, qacc.b(), k.eta());
   // dC = -AL AL^T ; dJ = -Q - JF - (JF)^T + P P^T  (upper triangles, mirrored):
   // whole passes one entry per thread, the remainder spread over lane groups
   if constexpr (TEAM > 32) {
@@ -341,14 +367,7 @@ __device__ void rhs(int lane, Rec<N> y, Rec<N> k, const double* __restrict__ F, 
     }
   }
   }
-  if (lane < 32) {  // dzeta = -rho/2 + |w|^2/2 + eta^T c, over the first warp
-    double z = 0.0;
-    for (int a = lane; a < M; a += 32) z = fma(0.5 * w[a], w[a], z);
-    if (c)
-      for (int l = lane; l < N; l += 32) z = fma(eta[l], c[l], z);
-    z = group_sum<32>(z);
-    if (lane == 0) *qacc.zeta() = fma(sq, z - 0.5 * qr[N], *qacc.zeta());
-  }
+  rhs_zeta<N, M, TEAM>(lane, eta, c, w, qr, sq, qacc.zeta());
   sync<TEAM>();
 }
 
