@@ -45,7 +45,7 @@
  *    original W: its condition number is then beyond ~1e12 and FP64 no longer
  *    carries the digits of a 1e-9 result.  A non-positive Cholesky pivot of
  *    U counts too.
- *  - Supported state dimensions n: 1, 2, 3, 4, 8 (one thread per element),
+ *  - Supported state dimensions n: 1, 2, 3, 4, 8 (one or two threads per element),
  *    16 and 64 (a warp / a CTA per element).  Other n return
  *    LQT_EUNSUPPORTED.  m <= 16, nr <= 64.
  */

@@ -30,7 +30,9 @@
 //     recomputed and stored, giving Fbar, Bbar (B = L U^-1 L^T), Qbar, qbar, rhobar, then
 //     Xbar, rbar (Q = X, q = X r, rho = r'Xr for H = I) and, after the
 //     reduction over sub-intervals, Lbar = (Bbar + Bbar^T) L U^-1 and
-//     Ubar = -U^-1 L^T Bbar L U^-1.
+//     Ubar = -U^-1 L^T Bbar L U^-1.  Sub-intervals that the constant-coefficient
+//     build serves share one sweep over their summed element adjoints
+//     (lqt_uniform_adjoint.cu).
 //
 // Kernels here use runtime-n loops over small local arrays (n <= 8): the
 // backward is not the benchmarked path and this keeps compile time small.

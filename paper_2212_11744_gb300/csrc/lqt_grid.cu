@@ -209,6 +209,9 @@ __device__ __forceinline__ int stage_float(const Operands<kValues>& op, float* A
                                            int64_t c0, int64_t ncols, int k0, int kc) {
   const int G = op.a.G, warp = t >> 5, lane = t & 31;
   int bad = 0;
+  // U loads in flight at a time: one by one, their latency was a fifth of a
+  // small product's time (G = 201: 27 us a product, 22 so)
+  constexpr int U = 7;
   auto put = [&](float* dst, bool live, int gk, double x) {
     float v = kScreenPad;
     if (gk < G) {
@@ -220,25 +223,44 @@ __device__ __forceinline__ int stage_float(const Operands<kValues>& op, float* A
     }
     *dst = v;
   };
-  for (int r = warp; r < TR; r += kThreads / 32)
-    for (int kk = lane; kk < kc; kk += 32) {
-      const bool live = i0 + r < G && k0 + kk < G;
-      put(As + r * S + kk, live, k0 + kk, live ? op.av(i0 + r, k0 + kk) : 0.0);
+  auto put_row = [&](float* dst, const double* src, bool live) {  // src: k0 onwards
+    for (int kb = lane; kb < kc; kb += 32 * U) {
+      double x[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int kk = kb + 32 * u;
+        x[u] = live && kk < kc && k0 + kk < G ? src[kk] : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int kk = kb + 32 * u;
+        if (kk < kc) put(dst + kk, live, k0 + kk, x[u]);
+      }
     }
+  };
+  for (int r = warp; r < TR; r += kThreads / 32)
+    put_row(As + r * S, op.A + (int64_t)(i0 + r) * G + k0, i0 + r < G);
   if (kValues) {
     for (int r = warp; r < TC; r += kThreads / 32) {
       const bool col = c0 + r < ncols;
-      const double* b = col ? op.bcol(c0 + r) : nullptr;
-      for (int kk = lane; kk < kc; kk += 32) {
-        const bool live = col && k0 + kk < G;
-        put(Bs + r * S + kk, live, k0 + kk, live ? b[k0 + kk] : 0.0);
-      }
+      put_row(Bs + r * S, col ? op.bcol(c0 + r) + k0 : nullptr, col);
     }
   } else {
-    for (int e = t; e < TC * kc; e += kThreads) {
-      const int kk = e / TC, r = e % TC;
-      const bool live = c0 + r < ncols && k0 + kk < G;
-      put(Bs + r * S + kk, live, k0 + kk, live ? op.Bm[(int64_t)(k0 + kk) * G + c0 + r] : 0.0);
+    const int r = t % TC;
+    const bool col = c0 + r < ncols;
+    constexpr int step = kThreads / TC;
+    for (int kb = t / TC; kb < kc; kb += step * U) {
+      double x[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int kk = kb + step * u;
+        x[u] = col && kk < kc && k0 + kk < G ? op.Bm[(int64_t)(k0 + kk) * G + c0 + r] : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int kk = kb + step * u;
+        if (kk < kc) put(Bs + r * S + kk, col, k0 + kk, x[u]);
+      }
     }
   }
   return bad;
@@ -253,7 +275,7 @@ __device__ __forceinline__ int stage_float(const Operands<kValues>& op, float* A
 // output, by some 30 FP64 instructions of the refinement (its three divisions)
 // at 64 cycles each.  One output per thread, with staging again in the second
 // pass, took 4.43 ms for the block and the values at G = 201, T = 10^4; this
-// 2.82 ms; 2 x 4 outputs and two CTAs on an SM 3.09.
+// 2.59 ms (2 x 4 outputs and two CTAs on an SM, loads one by one: 3.09).
 template <int P, int Q, bool kValues>
 __global__ void __launch_bounds__(kThreads, P * Q <= 4 ? 3 : 2)
     grid_minplus_kernel(GridArgs a, const double* __restrict__ A, const double* Bm, double* Om, double* X0,
