@@ -1039,10 +1039,13 @@ cudaError_t batch_build(const BatchDev& bd, const ElemPtrs& el, char* team_scrat
 // -> 15362 at 500000; n = 3, m = 2, K = 4: 187 -> 122 at 2048, 576 -> 518 at
 // 60000; n = 2, m = 1, K = 10: 167 -> 125 at 2048, 519 -> 502 at 60000, 1331 ->
 // 1344 at 200000.  n = 1 has too little to share (60 -> 64 at 10007).
+// The windows of a host call (equal runs of a long horizon, one after the other
+// behind their copies) stay with one thread: n = 4, T = 2^17, K = 4 took 2890 us
+// with pairs, 2855 without.
 constexpr int64_t kPairMaxT = 1 << 17;
 
 template <int N, int M>
-static void launch_build_nm(const BuildArgs& a, cudaStream_t st, double* stages, int64_t j0) {
+static void launch_build_nm(const BuildArgs& a, cudaStream_t st, double* stages, int64_t j0, bool window) {
   const int threads = 128;
   const int64_t blocks = (a.T + threads - 1) / threads;
   count_launch();
@@ -1051,7 +1054,7 @@ static void launch_build_nm(const BuildArgs& a, cudaStream_t st, double* stages,
     return;
   }
   if constexpr (N >= 2 && N <= 4) {
-    if (a.T <= kPairMaxT) {
+    if (a.T <= kPairMaxT && !window) {
       build_pair_kernel<N, M><<<(unsigned)((a.T + 31) / 32), 64, 0, st>>>(a);
       return;
     }
@@ -1061,12 +1064,12 @@ static void launch_build_nm(const BuildArgs& a, cudaStream_t st, double* stages,
 
 template <int N>
 static cudaError_t launch_build_n(const BuildArgs& a, int M, cudaStream_t st, double* stages = nullptr,
-                                  int64_t j0 = 0) {
+                                  int64_t j0 = 0, bool window = false) {
   switch (M) {
-    case 1: launch_build_nm<N, 1>(a, st, stages, j0); break;
-    case 2: if constexpr (N >= 2) { launch_build_nm<N, 2>(a, st, stages, j0); break; } else return cudaErrorInvalidValue;
-    case 4: if constexpr (N >= 3) { launch_build_nm<N, 4>(a, st, stages, j0); break; } else return cudaErrorInvalidValue;
-    case 8: if constexpr (N >= 8) { launch_build_nm<N, 8>(a, st, stages, j0); break; } else return cudaErrorInvalidValue;
+    case 1: launch_build_nm<N, 1>(a, st, stages, j0, window); break;
+    case 2: if constexpr (N >= 2) { launch_build_nm<N, 2>(a, st, stages, j0, window); break; } else return cudaErrorInvalidValue;
+    case 4: if constexpr (N >= 3) { launch_build_nm<N, 4>(a, st, stages, j0, window); break; } else return cudaErrorInvalidValue;
+    case 8: if constexpr (N >= 8) { launch_build_nm<N, 8>(a, st, stages, j0, window); break; } else return cudaErrorInvalidValue;
     default: return cudaErrorInvalidValue;
   }
   return cudaSuccess;
@@ -1101,11 +1104,11 @@ cudaError_t launch_build_range(const lqt_problem& p, const Layout& lay, const Co
     if (e != cudaSuccess) return e;
   }
   switch (p.n) {
-    case 1: return launch_build_n<1>(a, lay.M, st);
-    case 2: return launch_build_n<2>(a, lay.M, st);
-    case 3: return launch_build_n<3>(a, lay.M, st);
-    case 4: return launch_build_n<4>(a, lay.M, st);
-    case 8: return launch_build_n<8>(a, lay.M, st);
+    case 1: return launch_build_n<1>(a, lay.M, st, nullptr, 0, true);
+    case 2: return launch_build_n<2>(a, lay.M, st, nullptr, 0, true);
+    case 3: return launch_build_n<3>(a, lay.M, st, nullptr, 0, true);
+    case 4: return launch_build_n<4>(a, lay.M, st, nullptr, 0, true);
+    case 8: return launch_build_n<8>(a, lay.M, st, nullptr, 0, true);
     default: return cudaErrorInvalidValue;
   }
 }
