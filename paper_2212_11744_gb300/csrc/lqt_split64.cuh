@@ -39,6 +39,7 @@ struct Shared {
   double vec[8][N];
   uint4 dA[4 * 4 * ND * 32];  // (16 rows, 16-deep slab, digit, lane): an A fragment
   uint2 dB[8 * 4 * ND * 32];  // (8 columns, slab, digit, lane): a B fragment
+  unsigned eB[8 * 8 * 32];    // exponents of the right operand's entries, two a word: (8 columns, word, lane)
   alignas(16) float col[2][N];
   float rowp[N], scale[N];
   unsigned cand[8];
@@ -62,27 +63,45 @@ __device__ __forceinline__ Mat rows_of(const double* p, int ld) { return {p, ld,
 __device__ __forceinline__ Mat cols_of(const double* p, int ld) { return {p, 1, ld}; }
 
 // o(i, j) = sum_k a(i, k) b(k, j) + diag (i == j), or o -= the product
-// (kSubtract), o at o[i ld + j].  o may be one of the operands.  Returns the
+// (kSubtract), o at o[i ld + j].  o may be one of the operands.  Above the limit
+// the product is formed in FP64, or given up (kTry: see product16).  Returns the
 // largest biased exponent of the entries this warp set.
-static __device__ __noinline__ int product64(Shared& sm, Mat a, Mat b, double* o, int ld, int diag, int store) {
+static __device__ __noinline__ int product64(Shared& sm, Mat a, Mat b, double* o, int ld, int diag, int store,
+                                             int limit = split::kGradeLimit) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = lane >> 2, c = 2 * (lane & 3);
-  {
-    // warps 0 .. 7: rows 8 w + g of a; warps 8 .. 15: columns of b.  Entries k
-    // = 16 s + c, c + 1, c + 8, c + 9 of the vector and its largest exponent.
-    const bool left = warp < 8;
+  // warps 0 .. 7: rows 8 w + g of a; warps 8 .. 15: columns of b.  Entries k
+  // = 16 s + c, c + 1, c + 8, c + 9 of the vector and its largest exponent.
+  const bool left = warp < 8;
+  const int blk = warp & 7;
+  const int rb = warp >> 2, cb = warp & 3;
+  int top = 0;
+  bool graded = limit < 0;
+  if (!graded) {
+    unsigned xe[8];  // the entries' exponents, two a word
+    int e = 0;
     const Mat m = left ? a : b;
-    const int blk = warp & 7, v = 8 * blk + g;
+    const int v = 8 * blk + g;
     const double* p = m.p + (int64_t)v * m.sv + c * m.sk;
     double x[16];
-    int e = 0;
 #pragma unroll
     for (int q = 0; q < 16; ++q) x[q] = p[(16 * (q >> 2) + (q & 1) + 8 * ((q >> 1) & 1)) * m.sk];
+    unsigned bits = 0;
 #pragma unroll
-    for (int q = 0; q < 16; ++q) e = max(e, split::biased_exp(x[q]));
+    for (int q = 0; q < 16; q += 2) {
+      const int e0 = split::biased_exp(x[q]), e1 = split::biased_exp(x[q + 1]);
+      e = max(e, max(e0, e1));
+      bits |= split::magnitude_bits(x[q]) | split::magnitude_bits(x[q + 1]);
+      xe[q >> 1] = (unsigned)e0 | (unsigned)e1 << 16;
+    }
     e = max(e, __shfl_xor_sync(0xffffffffu, e, 1));
     e = max(e, __shfl_xor_sync(0xffffffffu, e, 2));
+    const bool odd = split::odd_vector(e, bits);
     if ((lane & 3) == 0) (left ? sm.rowE : sm.colE)[v] = e;
+    if (!left) {
+#pragma unroll
+      for (int w = 0; w < 8; ++w) sm.eB[(blk * 8 + w) * 32 + lane] = xe[w];
+    }
     // an A fragment's registers: rows g (k c .., k c + 8 ..), then rows g + 8
     uint2* d = left ? reinterpret_cast<uint2*>(sm.dA) + (((blk >> 1) * 4 * ND) * 32 + lane) * 2 + (blk & 1)
                     : sm.dB + (blk * 4 * ND) * 32 + lane;
@@ -95,10 +114,47 @@ static __device__ __noinline__ int product64(Shared& sm, Mat a, Mat b, double* o
       for (int i = 0; i < ND; ++i)
         d[(s * ND + i) * step] = make_uint2(split::digit_pair<C64>(u0, u1, i), split::digit_pair<C64>(u2, u3, i));
     }
+    __syncthreads();
+    // diagonal entry i = 8 blk + g: this lane of warp blk holds the k of row i that
+    // the same lane of warp 8 + blk holds of column i
+    int worst = 0;
+    if (left) {
+      unsigned term = 0;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) term = __vmaxu2(term, xe[w] + sm.eB[(blk * 8 + w) * 32 + lane]);
+      int t = max((int)(term & 0xffffu), (int)(term >> 16));
+      t = max(t, __shfl_xor_sync(0xffffffffu, t, 1));
+      t = max(t, __shfl_xor_sync(0xffffffffu, t, 2));
+      worst = split::grade(e, sm.colE[8 * blk + g], t);
+    }
+    graded = __syncthreads_or(odd || worst > limit) != 0;
   }
-  __syncthreads();
-  const int rb = warp >> 2, cb = warp & 3;
-  int top = 0;
+  if (graded) {
+    if (store == split::kTry) return split::kGraded;
+    double s[2][4] = {};
+#pragma unroll 1
+    for (int k = 0; k < N; ++k)
+#pragma unroll
+      for (int t = 0; t < 2; ++t)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int i = 16 * rb + g + 8 * (q >> 1), j = 16 * cb + 8 * t + c + (q & 1);
+          s[t][q] = fma(a.p[i * a.sv + k * a.sk], b.p[j * b.sv + k * b.sk], s[t][q]);
+        }
+    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < 2; ++t)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int i = 16 * rb + g + 8 * (q >> 1), j = 16 * cb + 8 * t + c + (q & 1);
+        const double v = s[t][q] + (i == j ? (double)diag : 0.0);
+        top = max(top, split::biased_exp(v));
+        double* w = o + (int64_t)i * ld + j;
+        *w = store == split::kSubtract ? *w - v : v;
+      }
+    __syncthreads();
+    return __reduce_max_sync(0xffffffffu, top);
+  }
   const uint4* fa = sm.dA + rb * 4 * ND * 32 + lane;
 #pragma unroll 1
   for (int t = 0; t < 2; ++t) {
@@ -261,14 +317,15 @@ static __device__ __noinline__ void inverse_f64(Shared& sm) {
 
 // sm.M <- sm.W^-1: the FP32 inverse and Newton steps M <- M - M (W M - I) until
 // the residual is below 2^-28 before the last step; where the residual does
-// not shrink, the FP64 inverse and one step.  E (row stride kLd) is scratch.
-__device__ __forceinline__ void inverse(Shared& sm, double* E) {
+// not shrink, the FP64 inverse and one step.  E (row stride kLd) is scratch;
+// limit: split::kAllFp64 or the products' own.
+__device__ __forceinline__ void inverse(Shared& sm, double* E, int limit) {
   constexpr int kExp1 = 1023;  // biased exponent of 1
-  bool fast = inverse_f32(sm);
+  bool fast = limit >= 0 && inverse_f32(sm);
   int last = kExp1 - 1;
   for (int it = 0; it < 4; ++it) {
     if (!fast) inverse_f64(sm);
-    const int top = product64(sm, rows_of(sm.W, kLd), cols_of(sm.M, kLd), E, kLd, -1, split::kSet);
+    const int top = product64(sm, rows_of(sm.W, kLd), cols_of(sm.M, kLd), E, kLd, -1, split::kSet, limit);
     // row sums: 64 entries below 2^(top - 1022)
     const bool done = __syncthreads_and(top <= kExp1 - 35) != 0 || !fast;
     const bool lost = __syncthreads_or(top > last - 3 || top > kExp1 - 7) != 0;
@@ -278,7 +335,8 @@ __device__ __forceinline__ void inverse(Shared& sm, double* E) {
       continue;
     }
     last = top;
-    product64(sm, rows_of(sm.M, kLd), cols_of(E, kLd), sm.M, kLd, 0, split::kSubtract);
+    product64(sm, rows_of(sm.M, kLd), cols_of(E, kLd), sm.M, kLd, 0, split::kSubtract,
+              limit < 0 ? limit : split::kNoLimit);
     if (done) break;
   }
 }
@@ -315,6 +373,14 @@ __device__ __forceinline__ double cta_sum(Shared& sm, double x) {
   return s;
 }
 
+// W = I + C J into sm.W, and the limit of the combination's other products: in
+// mixed units all of them are formed in FP64 (see split::kFoldLimit).
+__device__ __forceinline__ int product_w(Shared& sm, Mat c, Mat j) {
+  if (product64(sm, c, j, sm.W, kLd, 1, split::kTry, split::kFoldLimit) != split::kGraded) return split::kGradeLimit;
+  product64(sm, c, j, sm.W, kLd, 1, split::kSet, split::kAllFp64);
+  return split::kAllFp64;
+}
+
 // out = e1 (x) e2 (full elements in global memory; out aliases neither).
 __device__ inline void combine(Shared& sm, Slot sl, Rec<N> e1, Rec<N> e2, Rec<N> out) {
   using split::kSet;
@@ -324,8 +390,8 @@ __device__ inline void combine(Shared& sm, Slot sl, Rec<N> e1, Rec<N> e2, Rec<N>
   if (tid < N) b1[tid] = e1.b()[tid];
   else if (tid < 2 * N) eta2[tid - N] = e2.eta()[tid - N];
   // W = I + C1 J2, T1 = J2 A1 (C1, J2 symmetric)
-  product64(sm, rows_of(e1.C(), N), rows_of(e2.J(), N), sm.W, kLd, 1, kSet);
-  product64(sm, rows_of(e2.J(), N), cols_of(e1.A(), N), sl.T1, kLd, 0, kSet);
+  const int limit = product_w(sm, rows_of(e1.C(), N), rows_of(e2.J(), N));
+  product64(sm, rows_of(e2.J(), N), cols_of(e1.A(), N), sl.T1, kLd, 0, kSet, limit);
   {
     const double r = matvec(rows_of(e1.C(), N), eta2, b1[i]);
     const double w = matvec(rows_of(e2.J(), N), b1, 0.0);
@@ -335,10 +401,10 @@ __device__ inline void combine(Shared& sm, Slot sl, Rec<N> e1, Rec<N> e2, Rec<N>
     }
   }
   __syncthreads();
-  inverse(sm, sl.K1);
+  inverse(sm, sl.K1, limit);
   solve_refined(sm, rr, z0);
-  product64(sm, rows_of(sm.M, kLd), cols_of(e1.A(), N), sl.K1, kLd, 0, kSet);
-  product64(sm, rows_of(sm.M, kLd), rows_of(e1.C(), N), sm.W, kLd, 0, kSet);  // M C1
+  product64(sm, rows_of(sm.M, kLd), cols_of(e1.A(), N), sl.K1, kLd, 0, kSet, limit);
+  product64(sm, rows_of(sm.M, kLd), rows_of(e1.C(), N), sm.W, kLd, 0, kSet, limit);  // M C1
   // l0 = J2 z0 - eta2 ; zeta ; b = A2 z0 + b2 ; eta = K1^T wv + eta1
   {
     const double jz = matvec(rows_of(e2.J(), N), z0, 0.0);
@@ -355,10 +421,10 @@ __device__ inline void combine(Shared& sm, Slot sl, Rec<N> e1, Rec<N> e2, Rec<N>
     if (tid == 0) *out.zeta() = *e1.zeta() + *e2.zeta() + z;
   }
   // K1^T T1 ; A = A2 K1 ; A2 M C1 ; A2 M C1 A2^T
-  product64(sm, cols_of(sl.K1, kLd), cols_of(sl.T1, kLd), sm.M, kLd, 0, kSet);
-  product64(sm, rows_of(e2.A(), N), cols_of(sl.K1, kLd), out.A(), N, 0, kSet);
-  product64(sm, rows_of(e2.A(), N), cols_of(sm.W, kLd), sl.K1, kLd, 0, kSet);
-  product64(sm, rows_of(sl.K1, kLd), rows_of(e2.A(), N), sm.W, kLd, 0, kSet);
+  product64(sm, cols_of(sl.K1, kLd), cols_of(sl.T1, kLd), sm.M, kLd, 0, kSet, limit);
+  product64(sm, rows_of(e2.A(), N), cols_of(sl.K1, kLd), out.A(), N, 0, kSet, limit);
+  product64(sm, rows_of(e2.A(), N), cols_of(sm.W, kLd), sl.K1, kLd, 0, kSet, limit);
+  product64(sm, rows_of(sl.K1, kLd), rows_of(e2.A(), N), sm.W, kLd, 0, kSet, limit);
   // symmetric by taking the upper triangle
   double *oJ = out.J(), *oC = out.C();
   const double *J1 = e1.J(), *C2 = e2.C();
@@ -382,8 +448,8 @@ __device__ inline void combine_value(Shared& sm, Slot sl, Rec<N> e, const double
   double *b = sm.vec[0], *v2 = sm.vec[1], *rr = sm.vec[2], *wv = sm.vec[3], *alpha = sm.vec[4], *l0 = sm.vec[5];
   if (tid < N) b[tid] = e.b()[tid];
   else if (tid < 2 * N) v2[tid - N] = v2g[tid - N];
-  product64(sm, rows_of(e.C(), N), rows_of(S2, N), sm.W, kLd, 1, kSet);
-  product64(sm, rows_of(S2, N), cols_of(e.A(), N), sl.T1, kLd, 0, kSet);
+  const int limit = product_w(sm, rows_of(e.C(), N), rows_of(S2, N));
+  product64(sm, rows_of(S2, N), cols_of(e.A(), N), sl.T1, kLd, 0, kSet, limit);
   {
     const double r = matvec(rows_of(e.C(), N), v2, b[i]);
     const double w = matvec(rows_of(S2, N), b, 0.0);
@@ -393,10 +459,10 @@ __device__ inline void combine_value(Shared& sm, Slot sl, Rec<N> e, const double
     }
   }
   __syncthreads();
-  inverse(sm, sl.K1);
+  inverse(sm, sl.K1, limit);
   solve_refined(sm, rr, alpha);
-  product64(sm, rows_of(sm.M, kLd), cols_of(e.A(), N), sl.K1, kLd, 0, kSet);  // Psi
-  product64(sm, cols_of(sl.K1, kLd), cols_of(sl.T1, kLd), sm.W, kLd, 0, kSet);
+  product64(sm, rows_of(sm.M, kLd), cols_of(e.A(), N), sl.K1, kLd, 0, kSet, limit);  // Psi
+  product64(sm, cols_of(sl.K1, kLd), cols_of(sl.T1, kLd), sm.W, kLd, 0, kSet, limit);
   {
     const double sz = matvec(rows_of(S2, N), alpha, 0.0);
     if (own) l0[i] = sz - v2[i];

@@ -641,9 +641,10 @@ __device__ __forceinline__ bool inverse_f32(int lane, const double* W, double* M
 
 // Newton steps on Minv (row stride kWld), which holds the FP32 inverse of W
 // (row stride kWld) when `fast` (the same in every thread); E (row stride ld)
-// is scratch.
+// is scratch.  limit: split::kAllFp64 or the products' own.
 template <int NW>
-__device__ __forceinline__ void refine_inverse(const double* W, double* Minv, double* E, int ld, bool fast) {
+__device__ __forceinline__ void refine_inverse(const double* W, double* Minv, double* E, int ld, bool fast,
+                                               int limit) {
   constexpr int kExp1 = 1023;  // biased exponent of 1
   // at most four steps: |W M - I| < 2^-28 (row sum) before the last one
   int last = kExp1 - 1;
@@ -652,7 +653,8 @@ __device__ __forceinline__ void refine_inverse(const double* W, double* Minv, do
       if (NW == 1 || threadIdx.x < 32) inverse_f64(W, Minv);
       split::sync16<NW>();
     }
-    const int top = split::product16<NW>(rows_of(W, kWld), cols_of(Minv, kWld), rows_of(E, ld), -1, split::kSet);
+    const int top = split::product16<NW>(rows_of(W, kWld), cols_of(Minv, kWld), rows_of(E, ld), -1, split::kSet,
+                                           limit);
     // the residual must fall at least eightfold per step, from below 1/16
     bool done = top <= kExp1 - 32, lost = top > last - 3 || top > kExp1 - 5;
     if constexpr (NW > 1) {
@@ -666,7 +668,8 @@ __device__ __forceinline__ void refine_inverse(const double* W, double* Minv, do
       continue;
     }
     last = top;
-    split::product16<NW>(rows_of(Minv, kWld), cols_of(E, ld), rows_of(Minv, kWld), 0, split::kSubtract);
+    split::product16<NW>(rows_of(Minv, kWld), cols_of(E, ld), rows_of(Minv, kWld), 0, split::kSubtract,
+                         limit < 0 ? limit : split::kNoLimit);  // E is small: its products' errors are, too
     if (done) break;
   }
 }
@@ -703,6 +706,15 @@ __device__ __forceinline__ double saddle_term(double z, double Jz, double eta, d
   return fma(z, fma(0.5, Jz, -eta), l * ((b - z) - 0.5 * Cl));
 }
 
+// W = I + C J, and the limit of the combination's other products: in mixed units
+// all of them are formed in FP64 (see kFoldLimit).
+template <int NW>
+__device__ __forceinline__ int product_w(split::Mat16 c, split::Mat16 j, split::Mat16 w) {
+  if (split::product16<NW>(c, j, w, 1, split::kTry, split::kFoldLimit) != split::kGraded) return split::kGradeLimit;
+  split::product16<NW>(c, j, w, 1, split::kSet, split::kAllFp64);
+  return split::kAllFp64;
+}
+
 // Scratch of combine_split(): four 16 x 17 buffers and vectors.
 constexpr int kSplitBuf = 16 * kWld;
 constexpr int kSplitScratch = 4 * kSplitBuf + 6 * 16;
@@ -737,13 +749,13 @@ __device__ inline void combine_split(double* e1, const double* e2, double* scr) 
   const int lane = tid & 31, i = lane & 15, h = lane >> 4;
   const bool first = NW == 1 || tid < 32, second = NW == 1 || tid >= 32;
   // W = I + C1 J2, T1 = J2 A1 (C1, J2 symmetric: their rows are their columns)
-  product16<NW>(rows_of(C1, 16), rows_of(J2, 16), rows_of(W, kWld), 1, kSet);
+  const int limit = product_w<NW>(rows_of(C1, 16), rows_of(J2, 16), rows_of(W, kWld));
   if (first) {
-    const bool ok = inverse_f32(lane, W, Mi);
+    const bool ok = limit >= 0 && inverse_f32(lane, W, Mi);
     if (lane == 0) *fast = ok ? 1 : 0;
   }
   if (second) {
-    product16<1>(rows_of(J2, 16), cols_of(A1, 16), rows_of(T1, kWld), 0, kSet);
+    product16<1>(rows_of(J2, 16), cols_of(A1, 16), rows_of(T1, kWld), 0, kSet, limit);
     const double rv = matvec<double>(lane, [&](int r, int l) { return C1[l * 16 + r]; },
                                      [&](int l) { return eta2[l]; }, b1[i]);
     const double w = matvec<double>(lane, [&](int r, int l) { return -J2[l * 16 + r]; }, [&](int l) { return b1[l]; },
@@ -754,8 +766,8 @@ __device__ inline void combine_split(double* e1, const double* e2, double* scr) 
     }
   }
   sync16<NW>();
-  refine_inverse<NW>(W, Mi, K1, kWld, *fast != 0);
-  product16<NW>(rows_of(Mi, kWld), cols_of(A1, 16), rows_of(K1, kWld), 0, kSet);
+  refine_inverse<NW>(W, Mi, K1, kWld, *fast != 0, limit);
+  product16<NW>(rows_of(Mi, kWld), cols_of(A1, 16), rows_of(K1, kWld), 0, kSet, limit);
   double bo = 0.0, zs = 0.0, et = 0.0;
   if (first) {
     // z0 = M (b1 + C1 eta2), l0 = J2 z0 - eta2 ; zeta ; b = A2 z0 + b2
@@ -777,8 +789,8 @@ __device__ inline void combine_split(double* e1, const double* e2, double* scr) 
     // eta = K1^T wv + eta1 ; K1^T T1 ; A = A2 K1 (A1 was consumed by T1, K1)
     et = matvec<double>(lane, [&](int r, int l) { return K1[l * kWld + r]; }, [&](int l) { return wv[l]; },
                         e1[kOffEta + i]);
-    product16<1>(cols_of(K1, kWld), cols_of(T1, kWld), rows_of(T1, kWld), 0, kSet);
-    product16<1>(rows_of(A2, 16), cols_of(K1, kWld), rows_of(e1 + kOffA, 16), 0, kSet);
+    product16<1>(cols_of(K1, kWld), cols_of(T1, kWld), rows_of(T1, kWld), 0, kSet, limit);
+    product16<1>(rows_of(A2, 16), cols_of(K1, kWld), rows_of(e1 + kOffA, 16), 0, kSet, limit);
   }
   sync16<NW>();
   if (first) {
@@ -787,9 +799,9 @@ __device__ inline void combine_split(double* e1, const double* e2, double* scr) 
   }
   if (second && h == 0) e1[kOffEta + i] = et;
   // C = A2 (M C1) A2^T + C2
-  product16<NW>(rows_of(Mi, kWld), rows_of(C1, 16), rows_of(W, kWld), 0, kSet);
-  product16<NW>(rows_of(A2, 16), cols_of(W, kWld), rows_of(K1, kWld), 0, kSet);
-  product16<NW>(rows_of(K1, kWld), rows_of(A2, 16), rows_of(W, kWld), 0, kSet);
+  product16<NW>(rows_of(Mi, kWld), rows_of(C1, 16), rows_of(W, kWld), 0, kSet, limit);
+  product16<NW>(rows_of(A2, 16), cols_of(W, kWld), rows_of(K1, kWld), 0, kSet, limit);
+  product16<NW>(rows_of(K1, kWld), rows_of(A2, 16), rows_of(W, kWld), 0, kSet, limit);
   // symmetric by taking the upper triangle
   for (int e = tid; e < 256; e += 32 * NW) {
     const int r = e >> 4, c = e & 15;
@@ -823,12 +835,12 @@ __device__ inline void combine_value_split(const double* e, const double* V, dou
   const double* S2 = V;
   const double* v2 = V + 256;
   const int tid = threadIdx.x, lane = tid & 31, i = lane & 15, h = lane >> 4;
-  product16<NW>(rows_of(C, 16), rows_of(S2, 16), rows_of(W, kWld), 1, kSet);
+  const int limit = product_w<NW>(rows_of(C, 16), rows_of(S2, 16), rows_of(W, kWld));
   if (tid < 32) {
-    const bool ok = inverse_f32(lane, W, Mi);
+    const bool ok = limit >= 0 && inverse_f32(lane, W, Mi);
     if (lane == 0) *fast = ok ? 1 : 0;
   } else {
-    product16<1>(rows_of(S2, 16), cols_of(A, 16), rows_of(T1, kWld), 0, kSet);
+    product16<1>(rows_of(S2, 16), cols_of(A, 16), rows_of(T1, kWld), 0, kSet, limit);
     const double rv = matvec<double>(lane, [&](int r, int l) { return C[l * 16 + r]; }, [&](int l) { return v2[l]; },
                                      b[i]);
     const double w = matvec<double>(lane, [&](int r, int l) { return -S2[l * 16 + r]; }, [&](int l) { return b[l]; },
@@ -839,8 +851,8 @@ __device__ inline void combine_value_split(const double* e, const double* V, dou
     }
   }
   __syncthreads();
-  refine_inverse<NW>(W, Mi, Psi, 16, *fast != 0);
-  product16<NW>(rows_of(Mi, kWld), cols_of(A, 16), rows_of(Psi, 16), 0, kSet);
+  refine_inverse<NW>(W, Mi, Psi, 16, *fast != 0, limit);
+  product16<NW>(rows_of(Mi, kWld), cols_of(A, 16), rows_of(Psi, 16), 0, kSet, limit);
   if (tid < 32) {
     // alpha ; Sz = S2 alpha, l0 = Sz - v2 ; zeta
     solve_refined(lane, W, Mi, rr, alpha);
@@ -865,7 +877,7 @@ __device__ inline void combine_value_split(const double* e, const double* V, dou
     const double vo = matvec<double>(lane, [&](int r, int l) { return Psi[l * 16 + r]; },
                                      [&](int l) { return wv[l]; }, e[kOffEta + i]);
     if (h == 0) out[256 + i] = vo;
-    product16<1>(cols_of(Psi, 16), cols_of(T1, kWld), rows_of(T1, kWld), 0, kSet);
+    product16<1>(cols_of(Psi, 16), cols_of(T1, kWld), rows_of(T1, kWld), 0, kSet, limit);
   }
   __syncthreads();
   for (int q = tid; q < 256; q += 32 * NW) {
