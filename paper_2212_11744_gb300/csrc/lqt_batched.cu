@@ -126,9 +126,10 @@ __global__ void controls_cost_kernel(BatchDev bd, const double* S, const double*
 // Workspace layout of a batch.
 struct BatchLayout {
   int32_t B, n, m, K, M;
-  int64_t total, total_qr, maxT;
-  bool uniform;  // the constant-coefficient build applies to at least one problem
-  size_t off_probs, off_off, off_offqr, off_Lt, off_Ku, off_qr, off_el, off_team, off_inv, off_uni, off_scan, bytes;
+  int64_t total, total_qr;
+  int64_t chunks;  // of the constant-coefficient build; 0: it applies to no problem
+  size_t off_probs, off_off, off_offqr, off_chunk, off_Lt, off_Ku, off_qr, off_el, off_team, off_inv, off_uni, off_scan,
+      bytes;
 };
 
 static int32_t batch_factor_width(int n, int m) {
@@ -157,8 +158,7 @@ static lqt_status batch_validate(const lqt_batch* bt, BatchLayout& L) {
   const int maxM = n == 1 ? 1 : n == 2 ? 2 : n <= 4 ? 4 : n == 8 ? 8 : 16;
   if (L.M > maxM) return LQT_EUNSUPPORTED;
   int64_t total = 0, total_qr = 0;
-  L.maxT = 0;
-  L.uniform = false;
+  L.chunks = 0;
   for (int32_t b = 0; b < bt->count; ++b) {
     const lqt_problem& p = bt->problems[b];
     if (p.n != n || p.m != p0.m || p.nr != n || p.K != p0.K || p.T < 1) return LQT_EINVAL;
@@ -170,8 +170,7 @@ static lqt_status batch_validate(const lqt_batch* bt, BatchLayout& L) {
     const int32_t rm0 = p0.r.ptr ? p0.r.mode : LQT_CONST;
     if (rm != rm0 || (rm != LQT_CONST && rm != LQT_PER_INTERVAL && rm != LQT_PER_STAGE)) return LQT_EINVAL;
     if (!bt->x0[b]) return LQT_EINVAL;
-    if (p.T > L.maxT) L.maxT = p.T;
-    L.uniform = L.uniform || batch_uniform_member(p);
+    if (batch_uniform_member(p)) L.chunks += uniform_chunks(n, p.T);
     total += p.T + 1;
     total_qr += p.r.ptr ? sample_count(rm, p.T, p.K) : 1;
   }
@@ -181,6 +180,7 @@ static lqt_status batch_validate(const lqt_batch* bt, BatchLayout& L) {
   L.off_probs = off; off = bal(off + (size_t)L.B * sizeof(BatchProb));
   L.off_off = off; off = bal(off + ((size_t)L.B + 1) * sizeof(int64_t));
   L.off_offqr = off; off = bal(off + ((size_t)L.B + 1) * sizeof(int64_t));
+  L.off_chunk = off; off = bal(off + ((size_t)L.B + 1) * sizeof(int64_t));
   L.off_Lt = off; off = bal(off + (size_t)L.B * n * L.M * 8);
   L.off_Ku = off; off = bal(off + (size_t)L.B * L.m * n * 8);
   L.off_qr = off; off = bal(off + (size_t)total_qr * (n + 1) * 8);
@@ -193,7 +193,7 @@ static lqt_status batch_validate(const lqt_batch* bt, BatchLayout& L) {
   if (invariant_supported(n, L.M)) off = bal(off + (size_t)L.B * invariant_table_bytes(n, L.M, L.K));
   // per-problem tables of the constant-coefficient build
   L.off_uni = off;
-  if (L.uniform) off = bal(off + (size_t)L.B * uniform_table_bytes(n, L.M));
+  if (L.chunks) off = bal(off + (size_t)L.B * uniform_table_bytes(n, L.M));
   // The scans may run with any first-level chunk the caller's tuning picks;
   // the shortest chunk (2) needs the most level storage, so size for it.
   const int prev = scan_chunk_override();
@@ -213,6 +213,8 @@ static BatchDev batch_dev(const BatchLayout& L, char* ws) {
   d.off_qr = (const int64_t*)(ws + L.off_offqr);
   d.total = L.total;
   d.total_qr = L.total_qr;
+  d.off_chunk = (const int64_t*)(ws + L.off_chunk);
+  d.total_chunks = L.chunks;
   return d;
 }
 
@@ -254,8 +256,8 @@ lqt_status lqt_batch_plan(const lqt_batch* bt, void* ws, size_t ws_bytes, void* 
   if (!ws || ws_bytes < L.bytes) return LQT_EWORKSPACE;
   char* w = (char*)ws;
   std::vector<BatchProb> probs((size_t)L.B);
-  std::vector<int64_t> off((size_t)L.B + 1), offqr((size_t)L.B + 1);
-  int64_t o = 0, oq = 0;
+  std::vector<int64_t> off((size_t)L.B + 1), offqr((size_t)L.B + 1), offch((size_t)L.B + 1);
+  int64_t o = 0, oq = 0, oc = 0;
   for (int32_t b = 0; b < L.B; ++b) {
     const lqt_problem& p = bt->problems[b];
     BatchProb& P = probs[b];
@@ -280,16 +282,19 @@ lqt_status lqt_batch_plan(const lqt_batch* bt, void* ws, size_t ws_bytes, void* 
     P.cf.Ku = (const double*)(w + L.off_Ku) + (size_t)b * L.m * L.n;
     P.cf.Ku_per_boundary = 0;
     P.cf.M = L.M;
-    P.cf.uni = L.uniform && batch_uniform_member(p)
+    P.cf.uni = batch_uniform_member(p)
                    ? (const double*)(w + L.off_uni + (size_t)b * uniform_table_bytes(L.n, L.M))
                    : nullptr;
     off[b] = o;
     offqr[b] = oq;
+    offch[b] = oc;
+    if (P.cf.uni) oc += uniform_chunks(L.n, p.T);
     o += p.T + 1;
     oq += p.r.ptr ? sample_count(p.r.mode, p.T, p.K) : 1;
   }
   off[L.B] = o;
   offqr[L.B] = oq;
+  offch[L.B] = oc;
   cudaStream_t st = (cudaStream_t)stream;
   cudaError_t e = cudaMemcpyAsync(w + L.off_probs, probs.data(), probs.size() * sizeof(BatchProb),
                                   cudaMemcpyHostToDevice, st);
@@ -297,6 +302,8 @@ lqt_status lqt_batch_plan(const lqt_batch* bt, void* ws, size_t ws_bytes, void* 
     e = cudaMemcpyAsync(w + L.off_off, off.data(), off.size() * sizeof(int64_t), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(w + L.off_offqr, offqr.data(), offqr.size() * sizeof(int64_t), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(w + L.off_chunk, offch.data(), offch.size() * sizeof(int64_t), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // host tables go out of scope
   return e == cudaSuccess ? LQT_OK : LQT_ECUDA;
 }
@@ -321,7 +328,7 @@ lqt_status lqt_solve_batched(const lqt_batch* bt, const lqt_tuning* tune, double
   set_scan_chunk(chunk);
   cudaError_t e = batch_prepare(bd, st);
   const ElemPtrs el = batch_elements(L, w);
-  if (e == cudaSuccess && !invariant && L.uniform) e = batch_uniform(bd, L.maxT, el, st);
+  if (e == cudaSuccess && !invariant && L.chunks) e = batch_uniform(bd, el, st);
   if (e == cudaSuccess)
     e = invariant ? batch_build_invariant(bd, el, (double*)(w + L.off_inv), st)
                   : batch_build(bd, el, w + L.off_team, st);

@@ -117,6 +117,7 @@ bool uniform_eligible(const lqt_problem& p);
 size_t team_repeat_bytes(const lqt_problem& p, int32_t M, bool eligible);
 int64_t uniform_table_doubles(int n, int M);
 size_t uniform_table_bytes(int n, int M);
+int64_t uniform_chunks(int n, int64_t T);  // CTAs of the expansion
 cudaError_t launch_uniform_master(const lqt_problem& p, const Coefs& cf, cudaStream_t st);
 cudaError_t launch_uniform_expand(const lqt_problem& p, const Coefs& cf, const ElemPtrs& out, cudaStream_t st);
 // Reverse mode of that build (lqt_uniform_adjoint.cu).
@@ -253,6 +254,8 @@ struct BatchDev {
   const int64_t* off_qr;   // device [B+1]: qr sample offsets
   int64_t total;           // sum of (T_b + 1)
   int64_t total_qr;
+  const int64_t* off_chunk;  // device [B+1]: chunks of the constant-coefficient build before problem b
+  int64_t total_chunks;      // 0: no problem has a table
 };
 
 __host__ __device__ __forceinline__ int32_t batch_find(const int64_t* off, int32_t B, int64_t g) {
@@ -267,7 +270,7 @@ __host__ __device__ __forceinline__ int32_t batch_find(const int64_t* off, int32
 
 cudaError_t batch_prepare(const BatchDev& bd, cudaStream_t st);
 cudaError_t batch_build(const BatchDev& bd, const ElemPtrs& el, char* team_scratch, cudaStream_t st);
-cudaError_t batch_uniform(const BatchDev& bd, int64_t maxT, const ElemPtrs& out, cudaStream_t st);
+cudaError_t batch_uniform(const BatchDev& bd, const ElemPtrs& out, cudaStream_t st);
 cudaError_t batch_build_team(const BatchDev& bd, const ElemPtrs& el, double* gscratch, cudaStream_t st);
 cudaError_t batch_build_invariant(const BatchDev& bd, const ElemPtrs& el, double* tables, cudaStream_t st);
 void launch_inv_batch_build_warp(const BatchDev& bd, const double* tables, const ElemPtrs& out, cudaStream_t st);

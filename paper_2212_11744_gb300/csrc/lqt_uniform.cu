@@ -264,14 +264,15 @@ struct UniExpandArgs {
   const double* t;
   Coefs cf;
   ElemPtrs out;
-  // batches: problem b's chunks are blocks b chunks .. (b + 1) chunks - 1
+  // batches: the chunks of problem b are CTAs off_chunk[b] .. off_chunk[b + 1] - 1
   const BatchProb* probs;
-  int64_t chunks;
+  const int64_t* off_chunk;
+  int32_t B;
 };
 
 // Sub-intervals per CTA of the expansion.
-template <int N>
-constexpr int uni_chunk() { return N <= 8 ? 64 : 16; }
+__host__ __device__ constexpr int uni_chunk(int n) { return n <= 8 ? 64 : 16; }
+int64_t uniform_chunks(int n, int64_t T) { return (T + uni_chunk(n) - 1) / uni_chunk(n); }
 
 // The elements of one chunk of sub-intervals from the table: a thread holds
 // the entries e of A, C, J (value and slope) in registers and writes them for
@@ -279,18 +280,21 @@ constexpr int uni_chunk() { return N <= 8 ? 64 : 16; }
 // for eta, b and the rows of Z q a thread owns row i of one or more
 // sub-intervals.  Bound by the store of 3 n^2 + 2 n + 1 doubles per
 // sub-interval (n <= 8), by 18 n^2 FP64 operations above.
+// Batches: one CTA per chunk of a problem that has a table, found by the chunks'
+// prefix sum.  (A grid of the longest problem's chunks times B was 16.8 million
+// CTAs for one problem of T = 2^19 beside 2047 of T = 64, n = 4: 47.5 ms for the
+// batch, now 16.0; from 2^31 CTAs on it could not be launched.)
 template <int N>
 __global__ void __launch_bounds__(256) uniform_expand_kernel(UniExpandArgs a) {
-  constexpr int CH = uni_chunk<N>(), NN = N * N;
+  constexpr int CH = uni_chunk(N), NN = N * N;
   __shared__ double cj[CH], hk[CH], qs[CH * (N + 1)], zp[CH * N];
   __shared__ int near[CH];
-  const int64_t pb = a.probs ? blockIdx.x / a.chunks : 0;
-  const int64_t ch = a.probs ? blockIdx.x - pb * a.chunks : blockIdx.x;
+  const int32_t pb = a.probs ? batch_find(a.off_chunk, a.B, blockIdx.x) : 0;
+  const int64_t j0 = (blockIdx.x - (a.probs ? a.off_chunk[pb] : 0)) * CH;
   const Coefs& cf = a.probs ? a.probs[pb].cf : a.cf;
   const double* t = a.probs ? a.probs[pb].t : a.t;
   const int64_t T = a.probs ? a.probs[pb].T : a.T;
   const int64_t off = a.probs ? a.probs[pb].off : 0;
-  const int64_t j0 = ch * CH;
   const double* tab = cf.uni;
   if (tab == nullptr || tab[0] == 0.0 || j0 >= T) return;
   const int cnt = T - j0 < CH ? (int)(T - j0) : CH;
@@ -411,11 +415,8 @@ cudaError_t launch_uniform_master(const lqt_problem& p, const Coefs& cf, cudaStr
   return launch_master(a, 1, st);
 }
 
-static cudaError_t launch_expand(int n, const UniExpandArgs& a, int64_t problems, int64_t maxT, cudaStream_t st) {
-  UniExpandArgs b = a;
-  const int ch = n <= 8 ? 64 : 16;
-  b.chunks = (maxT + ch - 1) / ch;
-  const unsigned grid = (unsigned)(b.chunks * problems);
+static cudaError_t launch_expand(int n, const UniExpandArgs& b, int64_t chunks, cudaStream_t st) {
+  const unsigned grid = (unsigned)chunks;
   switch (n) {
     case 1: uniform_expand_kernel<1><<<grid, 256, 0, st>>>(b); break;
     case 2: uniform_expand_kernel<2><<<grid, 256, 0, st>>>(b); break;
@@ -433,17 +434,17 @@ static cudaError_t launch_expand(int n, const UniExpandArgs& a, int64_t problems
 cudaError_t launch_uniform_expand(const lqt_problem& p, const Coefs& cf, const ElemPtrs& out, cudaStream_t st) {
   UniExpandArgs a{};
   a.K = p.K; a.T = p.T; a.t = p.t; a.cf = cf; a.out = out;
-  return launch_expand(p.n, a, 1, p.T, st);
+  return launch_expand(p.n, a, uniform_chunks(p.n, p.T), st);
 }
 
-cudaError_t batch_uniform(const BatchDev& bd, int64_t maxT, const ElemPtrs& out, cudaStream_t st) {
+cudaError_t batch_uniform(const BatchDev& bd, const ElemPtrs& out, cudaStream_t st) {
   UniArgs a{};
   a.n = bd.n; a.M = bd.M; a.K = bd.K; a.B = bd.B; a.probs = bd.probs;
   const cudaError_t e = launch_master(a, bd.B, st);
   if (e != cudaSuccess) return e;
   UniExpandArgs x{};
-  x.K = bd.K; x.out = out; x.probs = bd.probs;
-  return launch_expand(bd.n, x, bd.B, maxT, st);
+  x.K = bd.K; x.out = out; x.probs = bd.probs; x.off_chunk = bd.off_chunk; x.B = bd.B;
+  return launch_expand(bd.n, x, bd.total_chunks, st);
 }
 
 }  // namespace lqt
