@@ -137,11 +137,21 @@ static int32_t batch_factor_width(int n, int m) {
   return padded_M(m);
 }
 
-// Whether problem p of a batch has a table of the constant-coefficient build.
-// A table costs one element's integration per problem, so short problems keep
-// the general build; n = 64 tables (MBs each) are left to single problems.
+// Whether problem p of a batch has a table of the constant-coefficient build,
+// given that the batch uses them.  A table costs one element's integration per
+// problem, so short problems keep the general build; n = 64 tables (MBs each) are
+// left to single problems.  Whole batches, general build -> tables, us: n = 1: 512
+// problems of T = 512 462 -> 488, 128 of 2048 493 -> 406; n = 2: 2048 of 128 1077 ->
+// 1202, 1024 of 256 1069 -> 885; n = 3: 1024 of 64 925 -> 926, 1024 of 256 2158 ->
+// 1268; n = 16: 1024 of 64 42306 -> 12252.
+static int64_t batch_uniform_min_T(int n) { return n == 1 ? 1024 : n == 2 ? 256 : 64; }
+// ... and the fewest sub-intervals of such problems for which they are used: below
+// it the general build takes one element's latency, as a table does (n = 1: 64 of
+// 1024 289 -> 305; n = 2: 64 of 256 295 -> 323, 64 of 512 373 -> 359).
+static int64_t batch_uniform_min_total(int n) { return n == 1 ? 131072 : n == 2 ? 32768 : 0; }
+
 static bool batch_uniform_member(const lqt_problem& p) {
-  return p.n <= 16 && p.T >= 64 && !p.c.ptr && (!p.r.ptr || p.r.mode != LQT_PER_STAGE);
+  return p.n <= 16 && p.T >= batch_uniform_min_T(p.n) && !p.c.ptr && (!p.r.ptr || p.r.mode != LQT_PER_STAGE);
 }
 
 static lqt_status batch_validate(const lqt_batch* bt, BatchLayout& L) {
@@ -157,7 +167,7 @@ static lqt_status batch_validate(const lqt_batch* bt, BatchLayout& L) {
   L.M = batch_factor_width(n, p0.m);
   const int maxM = n == 1 ? 1 : n == 2 ? 2 : n <= 4 ? 4 : n == 8 ? 8 : 16;
   if (L.M > maxM) return LQT_EUNSUPPORTED;
-  int64_t total = 0, total_qr = 0;
+  int64_t total = 0, total_qr = 0, served = 0;
   L.chunks = 0;
   for (int32_t b = 0; b < bt->count; ++b) {
     const lqt_problem& p = bt->problems[b];
@@ -170,10 +180,14 @@ static lqt_status batch_validate(const lqt_batch* bt, BatchLayout& L) {
     const int32_t rm0 = p0.r.ptr ? p0.r.mode : LQT_CONST;
     if (rm != rm0 || (rm != LQT_CONST && rm != LQT_PER_INTERVAL && rm != LQT_PER_STAGE)) return LQT_EINVAL;
     if (!bt->x0[b]) return LQT_EINVAL;
-    if (batch_uniform_member(p)) L.chunks += uniform_chunks(n, p.T);
+    if (batch_uniform_member(p)) {
+      L.chunks += uniform_chunks(n, p.T);
+      served += p.T;
+    }
     total += p.T + 1;
     total_qr += p.r.ptr ? sample_count(rm, p.T, p.K) : 1;
   }
+  if (served < batch_uniform_min_total(n)) L.chunks = 0;
   L.total = total;
   L.total_qr = total_qr;
   size_t off = 0;
@@ -282,7 +296,7 @@ lqt_status lqt_batch_plan(const lqt_batch* bt, void* ws, size_t ws_bytes, void* 
     P.cf.Ku = (const double*)(w + L.off_Ku) + (size_t)b * L.m * L.n;
     P.cf.Ku_per_boundary = 0;
     P.cf.M = L.M;
-    P.cf.uni = batch_uniform_member(p)
+    P.cf.uni = L.chunks && batch_uniform_member(p)
                    ? (const double*)(w + L.off_uni + (size_t)b * uniform_table_bytes(L.n, L.M))
                    : nullptr;
     off[b] = o;

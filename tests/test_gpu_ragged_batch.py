@@ -4,7 +4,6 @@ number.  Against the oracle, and the long problem against itself in a batch of
 its own."""
 import dataclasses
 
-import numpy as np
 import pytest
 import torch
 
@@ -16,12 +15,14 @@ pytestmark = pytest.mark.gpu
 
 
 def member(n, T, seed=3):
-    if n > 1:
+    """A member of the workloads' batch; n = 1 and 3: its first states, one input."""
+    if n not in (1, 3):
         return W.batched_member(seed, T=T, n=n)
-    p = W.batched_member(seed, T=T, n=2)
-    return dataclasses.replace(p, n=1, nr=1, F=W.const(p.F.values[0][:1, :1]), L=W.const(np.array([[0.7]])),
-                               X=W.const(np.array([[1.3]])), r=W.Coef(p.r.values[:, :1].copy(), p.r.mode),
-                               Xf=np.array([[1.3]]), rf=p.rf[:1], x0=p.x0[:1])
+    p = W.batched_member(seed, T=T, n=n + 1)
+    cut = lambda c: W.const(c.values[0][:n, :n])
+    return dataclasses.replace(p, n=n, nr=n, m=1, F=cut(p.F), L=W.const(p.L.values[0][:n, :1]), X=cut(p.X),
+                               U=W.const(p.U.values[0][:1, :1]), r=W.Coef(p.r.values[:, :n].copy(), p.r.mode),
+                               Xf=p.Xf[:n, :n], rf=p.rf[:n], x0=p.x0[:n])
 
 
 @pytest.mark.parametrize("n", [1, 2, 8, 16])
@@ -58,3 +59,20 @@ def test_longest_times_count_beyond_the_grid_limit():
     got = b.problem_slice(out, B - 1)
     for k in ("S", "v", "x", "u"):
         assert rel(to_np(got[k]), to_np(want[k])) <= TOL, k
+
+
+# n, T, problems: either side of the shortest problem that has a table, and of
+# the fewest sub-intervals for which a batch makes tables
+@pytest.mark.parametrize("n,T,B", [(1, 1023, 129), (1, 1024, 127), (1, 1024, 128), (2, 255, 129), (2, 256, 127),
+                                   (2, 256, 128), (3, 63, 3), (3, 64, 3)])
+def test_lines_of_the_table_rule(n, T, B):
+    from paper_2212_11744_gb300.batch import Batch
+    p = member(n, T)
+    b = Batch([p] * B)
+    out = b.solve()
+    torch.cuda.synchronize()
+    ref = oracle.solve(p)
+    for i in (0, B // 2, B - 1):
+        got = b.problem_slice(out, i)
+        for k in ("S", "v", "zeta", "x", "u"):
+            assert rel(to_np(got[k]), ref[k]) <= TOL, (i, k)
