@@ -464,9 +464,14 @@ template <int P, int Q, bool kValues>
 cudaError_t launch_tiles(const GridArgs& a, const double* A, const double* B, double* out, double* X0, double* X1,
                          int l, int64_t ncols, const double2* tab, cudaStream_t st) {
   const int kc = a.G < kKC ? ((a.G + 3) & ~3) : kKC;
-  const size_t smem = (size_t)(16 * P + 16 * Q) * screen_stride(kc) * sizeof(float);  // at most 58 KB
+  constexpr size_t per_stride = (size_t)(16 * P + 16 * Q) * sizeof(float);
+  const size_t smem = per_stride * screen_stride(kc);  // at most 58 KB
   const auto kernel = grid_minplus_kernel<P, Q, kValues>;
-  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the limit of the largest G, whatever this G: the attribute belongs to all of
+  // the process's threads, and one with a small G must not lower it between
+  // another's call here and its launch
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)(per_stride * screen_stride(kKC)));
   if (e != cudaSuccess) return e;
   const dim3 grid(cdiv_u(ncols, 16 * Q), cdiv_u(a.G, 16 * P));
   kernel<<<grid, kThreads, smem, st>>>(a, A, B, out, X0, X1, l, ncols, tab);

@@ -368,10 +368,12 @@ cudaError_t launch_uniform_adjoint(const UniAdjArgs& a, cudaStream_t st) {
   const int nn = a.n * a.n;
   uniform_adjoint_sums_kernel<<<(unsigned)a.parts, 256, 0, st>>>(a);
   count_launch();
-  // n = 8, K = 8: 65 KB
-  const size_t smem = (size_t)(12 + 6 + 6 + 3 + 3 + 12 * a.K) * nn * sizeof(double);
+  // the limit of the largest n and K (8, 8: 65 KB), whatever these: the attribute
+  // belongs to all of the process's threads (lqt_grid.cu, launch_tiles)
+  auto bytes = [](int K, int n) { return (size_t)(12 + 6 + 6 + 3 + 3 + 12 * K) * n * n * sizeof(double); };
+  const size_t smem = bytes(a.K, a.n);
   const cudaError_t e = cudaFuncSetAttribute(uniform_adjoint_sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
+                                             (int)bytes(8, 8));
   if (e != cudaSuccess) return e;
   uniform_adjoint_sweep_kernel<<<3, 256, smem, st>>>(a);
   count_launch();
