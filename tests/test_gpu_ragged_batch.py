@@ -9,7 +9,7 @@ import torch
 
 import oracle
 import workloads as W
-from tests.test_gpu_parity import TOL, relerr as rel, to_np
+from tests.test_gpu_parity import TOL, relerr as rel, relerr_one, to_np
 
 pytestmark = pytest.mark.gpu
 
@@ -56,9 +56,10 @@ def test_longest_times_count_beyond_the_grid_limit():
         got = b.problem_slice(out, i)
         for k in ("S", "v", "zeta", "x", "u"):
             assert rel(to_np(got[k]), ref[k]) <= TOL, (i, k)
+    # scalars that cross zero: against the whole trajectory's norm
     got = b.problem_slice(out, B - 1)
     for k in ("S", "v", "x", "u"):
-        assert rel(to_np(got[k]), to_np(want[k])) <= TOL, k
+        assert relerr_one(to_np(got[k]), to_np(want[k])) <= TOL, k
 
 
 # n, T, problems: either side of the shortest problem that has a table, and of
