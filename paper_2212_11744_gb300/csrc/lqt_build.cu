@@ -471,12 +471,12 @@ struct NoExchange {
   __device__ __forceinline__ void take(double*, double*) {}
 };
 
-template <int N, int M, int ROLE = kBothSides, class X = NoExchange>
-__device__ __forceinline__ void element_rhs(const Elem<N>& y, const double* __restrict__ F,
-                                            const double* __restrict__ c, const double* __restrict__ Lt,
-                                            const double* __restrict__ Q, const double* __restrict__ qr,
-                                            Elem<N>& k, unsigned long long nzF, unsigned long long nzL,
-                                            X xch = X()) {
+template <int N, int M, int ROLE, class X>
+__device__ __forceinline__ void element_rhs_by_entry(const Elem<N>& y, const double* __restrict__ F,
+                                                     const double* __restrict__ c, const double* __restrict__ Lt,
+                                                     const double* __restrict__ Q, const double* __restrict__ qr,
+                                                     Elem<N>& k, unsigned long long nzF, unsigned long long nzL,
+                                                     X xch) {
   constexpr bool kFlow = (ROLE & kFlowSide) != 0, kCost = (ROLE & kCostSide) != 0;
   double AL[N * M], P[N * M], w[M];
 #pragma unroll
@@ -583,6 +583,143 @@ __device__ __forceinline__ void element_rhs(const Elem<N>& y, const double* __re
       for (int l = 0; l < N; ++l) z = fma(y.eta[l], c[l], z);
     }
     k.zeta = z;
+  }
+}
+
+// The same without the branches around each entry, output by output: at n = 8 a
+// thread's fields are mostly spilled, and with every bit set the order above,
+// which keeps whole products in flight, was slower (n = 8, uneven grid, T = 40000:
+// 8.29 ms against 6.94 so; the same sums in the same order, so the same bits).
+template <int N, int M>
+__device__ __forceinline__ void element_rhs_dense(const Elem<N>& y, const double* __restrict__ F,
+                                                  const double* __restrict__ c, const double* __restrict__ Lt,
+                                                  const double* __restrict__ Q, const double* __restrict__ qr,
+                                                  Elem<N>& k) {
+  double AL[N * M], P[N * M], w[M];
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+#pragma unroll
+    for (int a = 0; a < M; ++a) {
+      double s1 = 0.0, s2 = 0.0;
+#pragma unroll
+      for (int l = 0; l < N; ++l) {
+        const double lt = Lt[l * M + a];
+        s1 = fma(y.A[i * N + l], lt, s1);
+        s2 = fma(y.J[sidx<N>(i, l)], lt, s2);
+      }
+      AL[i * M + a] = s1;
+      P[i * M + a] = s2;
+    }
+#pragma unroll
+  for (int a = 0; a < M; ++a) {
+    double s = 0.0;
+#pragma unroll
+    for (int l = 0; l < N; ++l) s = fma(Lt[l * M + a], y.eta[l], s);
+    w[a] = s;
+  }
+  // dA = AL P^T - A F
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      double s = 0.0;
+#pragma unroll
+      for (int a = 0; a < M; ++a) s = fma(AL[i * M + a], P[j * M + a], s);
+#pragma unroll
+      for (int l = 0; l < N; ++l) s = fma(-y.A[i * N + l], F[l * N + j], s);
+      k.A[i * N + j] = s;
+    }
+  // db = -AL w - A c
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    double s = 0.0;
+#pragma unroll
+    for (int a = 0; a < M; ++a) s = fma(-AL[i * M + a], w[a], s);
+    if (c) {
+#pragma unroll
+      for (int l = 0; l < N; ++l) s = fma(-y.A[i * N + l], c[l], s);
+    }
+    k.b[i] = s;
+  }
+  // dC = -AL AL^T
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+#pragma unroll
+    for (int j = i; j < N; ++j) {
+      double s = 0.0;
+#pragma unroll
+      for (int a = 0; a < M; ++a) s = fma(-AL[i * M + a], AL[j * M + a], s);
+      k.C[sidx<N>(i, j)] = s;
+    }
+  // deta = -q - F^T eta + J c + P w
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    double s = -qr[i];
+#pragma unroll
+    for (int l = 0; l < N; ++l) s = fma(-F[l * N + i], y.eta[l], s);
+    if (c) {
+#pragma unroll
+      for (int l = 0; l < N; ++l) s = fma(y.J[sidx<N>(i, l)], c[l], s);
+    }
+#pragma unroll
+    for (int a = 0; a < M; ++a) s = fma(P[i * M + a], w[a], s);
+    k.eta[i] = s;
+  }
+  // dJ = -Q - JF - (JF)^T + P P^T
+  double JF[N * N];
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      double s = 0.0;
+#pragma unroll
+      for (int l = 0; l < N; ++l) s = fma(y.J[sidx<N>(i, l)], F[l * N + j], s);
+      JF[i * N + j] = s;
+    }
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+#pragma unroll
+    for (int j = i; j < N; ++j) {
+      double s = -Q[i * N + j] - JF[i * N + j] - JF[j * N + i];
+#pragma unroll
+      for (int a = 0; a < M; ++a) s = fma(P[i * M + a], P[j * M + a], s);
+      k.J[sidx<N>(i, j)] = s;
+    }
+  // dzeta
+  double z = -0.5 * qr[N];
+#pragma unroll
+  for (int a = 0; a < M; ++a) z = fma(0.5 * w[a], w[a], z);
+  if (c) {
+#pragma unroll
+    for (int l = 0; l < N; ++l) z = fma(y.eta[l], c[l], z);
+  }
+  k.zeta = z;
+}
+
+// n = 8 out of line: its fields are in local memory either way, and inlined at
+// each of the four stages the two forms took minutes to compile.
+template <int M, bool kDense>
+static __device__ __noinline__ void element_rhs8(const Elem<8>& y, const double* F, const double* c, const double* Lt,
+                                                 const double* Q, const double* qr, Elem<8>& k,
+                                                 unsigned long long nzF, unsigned long long nzL) {
+  if constexpr (kDense)
+    element_rhs_dense<8, M>(y, F, c, Lt, Q, qr, k);
+  else
+    element_rhs_by_entry<8, M, kBothSides>(y, F, c, Lt, Q, qr, k, nzF, nzL, NoExchange());
+}
+
+template <int N, int M, int ROLE, class X>
+__device__ __forceinline__ void element_rhs(const Elem<N>& y, const double* __restrict__ F,
+                                            const double* __restrict__ c, const double* __restrict__ Lt,
+                                            const double* __restrict__ Q, const double* __restrict__ qr,
+                                            Elem<N>& k, unsigned long long nzF, unsigned long long nzL, X xch) {
+  if constexpr (N == 8) {
+    if (8 * __popcll(nzF) >= 7 * N * N)  // F (nearly) full
+      element_rhs8<M, true>(y, F, c, Lt, Q, qr, k, nzF, nzL);
+    else
+      element_rhs8<M, false>(y, F, c, Lt, Q, qr, k, nzF, nzL);
+  } else {
+    element_rhs_by_entry<N, M, ROLE>(y, F, c, Lt, Q, qr, k, nzF, nzL, xch);
   }
 }
 
