@@ -137,6 +137,42 @@ __device__ __forceinline__ void control_at(const DenseArgs& a, int64_t j, int32_
   control_from<N, M>(L, U, a.m, e, u);
 }
 
+// The right-hand sides by entry, or whole where F is (nearly) full; n = 8 out of
+// line, as its state is in local memory either way.
+template <int N, int M>
+__device__ __forceinline__ void dense_riccati_inl(const RicState<N>& y, const double* F, const double* c,
+                                                  const double* Lt, const double* Q, const double* qr,
+                                                  RicState<N>& k, unsigned long long nzF, unsigned long long nzL) {
+  if (8 * __popcll(nzF) >= 7 * N * N)
+    riccati_rhs<N, M>(y, F, c, Lt, Q, qr, k);
+  else
+    riccati_rhs_by_entry<N, M>(y, F, c, Lt, Q, qr, k, nzF, nzL);
+}
+template <int M>
+static __device__ __noinline__ void dense_riccati8(const RicState<8>& y, const double* F, const double* c,
+                                                   const double* Lt, const double* Q, const double* qr,
+                                                   RicState<8>& k, unsigned long long nzF, unsigned long long nzL) {
+  dense_riccati_inl<8, M>(y, F, c, Lt, Q, qr, k, nzF, nzL);
+}
+template <int N, int M>
+__device__ __forceinline__ void dense_riccati(const RicState<N>& y, const double* F, const double* c,
+                                              const double* Lt, const double* Q, const double* qr, RicState<N>& k,
+                                              unsigned long long nzF, unsigned long long nzL) {
+  if constexpr (N == 8)
+    dense_riccati8<M>(y, F, c, Lt, Q, qr, k, nzF, nzL);
+  else
+    dense_riccati_inl<N, M>(y, F, c, Lt, Q, qr, k, nzF, nzL);
+}
+template <int N, int M>
+__device__ __forceinline__ void dense_closed_loop(const double* S, const double* v, const double* x, const double* F,
+                                                  const double* c, const double* Lt, double* dx,
+                                                  unsigned long long nzF, unsigned long long nzL) {
+  if (8 * __popcll(nzF) >= 7 * N * N)
+    closed_loop_rhs<N, M>(S, v, x, F, c, Lt, dx);
+  else
+    closed_loop_rhs_by_entry<N, M>(S, v, x, F, c, Lt, dx, nzF, nzL);
+}
+
 template <int N, int M>
 __global__ void __launch_bounds__(128) densify_kernel(DenseArgs a) {
   constexpr int NS = Dim<N>::NS;
@@ -162,17 +198,17 @@ __global__ void __launch_bounds__(128) densify_kernel(DenseArgs a) {
         Q[q] = cf.Q.ptr + sample_index(cf.Q.mode, j, ps[q], K) * N * N;
         qr[q] = cf.qr.ptr + sample_index(cf.qr.mode, j, ps[q], K) * (N + 1);
       }
-      riccati_rhs<N, M>(y, F[0], c[0], Lt[0], Q[0], qr[0], k, nzF, nzL);
+      dense_riccati<N, M>(y, F[0], c[0], Lt[0], Q[0], qr[0], k, nzF, nzL);
       D[i + 1] = k;
       ric_axpy(yn, y, -h / 6.0, k);
       ric_axpy(yt, y, -0.5 * h, k);
-      riccati_rhs<N, M>(yt, F[1], c[1], Lt[1], Q[1], qr[1], k, nzF, nzL);
+      dense_riccati<N, M>(yt, F[1], c[1], Lt[1], Q[1], qr[1], k, nzF, nzL);
       ric_axpy(yn, yn, -h / 3.0, k);
       ric_axpy(yt, y, -0.5 * h, k);
-      riccati_rhs<N, M>(yt, F[1], c[1], Lt[1], Q[1], qr[1], k, nzF, nzL);
+      dense_riccati<N, M>(yt, F[1], c[1], Lt[1], Q[1], qr[1], k, nzF, nzL);
       ric_axpy(yn, yn, -h / 3.0, k);
       ric_axpy(yt, y, -h, k);
-      riccati_rhs<N, M>(yt, F[2], c[2], Lt[2], Q[2], qr[2], k, nzF, nzL);
+      dense_riccati<N, M>(yt, F[2], c[2], Lt[2], Q[2], qr[2], k, nzF, nzL);
       ric_axpy(y, yn, -h / 6.0, k);
       if (i > 0) ok = store_values<N>(y, a.Sd + (g0 + i) * N * N, a.vd + (g0 + i) * N, a.zd + g0 + i) && ok;
     }
@@ -183,7 +219,7 @@ __global__ void __launch_bounds__(128) densify_kernel(DenseArgs a) {
       const double* Lt = cf.Lt.ptr + sample_index(cf.Lt.mode, j, 0, K) * N * M;
       const double* Q = cf.Q.ptr + sample_index(cf.Q.mode, j, 0, K) * N * N;
       const double* qr = cf.qr.ptr + sample_index(cf.qr.mode, j, 0, K) * (N + 1);
-      riccati_rhs<N, M>(y, F, c, Lt, Q, qr, D[0], nzF, nzL);
+      dense_riccati<N, M>(y, F, c, Lt, Q, qr, D[0], nzF, nzL);
     }
     // boundary point t_j: the given solution
     double x[N];
@@ -218,25 +254,25 @@ __global__ void __launch_bounds__(128) densify_kernel(DenseArgs a) {
         Lt[q] = cf.Lt.ptr + sample_index(cf.Lt.mode, j, ps[q], K) * N * M;
       }
       double kx[N], ax[N], xt[N];
-      closed_loop_rhs<N, M>(y0.S, y0.v, x, F[0], c[0], Lt[0], kx, nzF, nzL);
+      dense_closed_loop<N, M>(y0.S, y0.v, x, F[0], c[0], Lt[0], kx, nzF, nzL);
 #pragma unroll
       for (int q = 0; q < N; ++q) {
         ax[q] = fma(h / 6.0, kx[q], x[q]);
         xt[q] = fma(0.5 * h, kx[q], x[q]);
       }
-      closed_loop_rhs<N, M>(ym.S, ym.v, xt, F[1], c[1], Lt[1], kx, nzF, nzL);
+      dense_closed_loop<N, M>(ym.S, ym.v, xt, F[1], c[1], Lt[1], kx, nzF, nzL);
 #pragma unroll
       for (int q = 0; q < N; ++q) {
         ax[q] = fma(h / 3.0, kx[q], ax[q]);
         xt[q] = fma(0.5 * h, kx[q], x[q]);
       }
-      closed_loop_rhs<N, M>(ym.S, ym.v, xt, F[1], c[1], Lt[1], kx, nzF, nzL);
+      dense_closed_loop<N, M>(ym.S, ym.v, xt, F[1], c[1], Lt[1], kx, nzF, nzL);
 #pragma unroll
       for (int q = 0; q < N; ++q) {
         ax[q] = fma(h / 3.0, kx[q], ax[q]);
         xt[q] = fma(h, kx[q], x[q]);
       }
-      closed_loop_rhs<N, M>(y1.S, y1.v, xt, F[2], c[2], Lt[2], kx, nzF, nzL);
+      dense_closed_loop<N, M>(y1.S, y1.v, xt, F[2], c[2], Lt[2], kx, nzF, nzL);
 #pragma unroll
       for (int q = 0; q < N; ++q) {
         x[q] = fma(h / 6.0, kx[q], ax[q]);

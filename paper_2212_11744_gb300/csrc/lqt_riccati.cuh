@@ -24,14 +24,109 @@ __host__ __device__ constexpr int ric_doubles() {
 // dS/dt = -(SF)^T - SF - Q + (S Lt)(S Lt)^T
 // dv/dt = -q + S c - F^T v + (S Lt)(Lt^T v)
 // dz/dt = -rho/2 + |Lt^T v|^2 / 2 + v^T c
-// nzF, nzL: the entries of F and Lt that may be nonzero (nonzero_bits); the
-// others are skipped.
 template <int N, int M>
 __device__ __forceinline__ void riccati_rhs(const RicState<N>& y, const double* __restrict__ F,
                                             const double* __restrict__ c, const double* __restrict__ Lt,
                                             const double* __restrict__ Q, const double* __restrict__ qr,
-                                            RicState<N>& k, unsigned long long nzF = ~0ull,
-                                            unsigned long long nzL = ~0ull) {
+                                            RicState<N>& k) {
+  double SL[N * M], w[M], SF[N * N];
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+#pragma unroll
+    for (int a = 0; a < M; ++a) {
+      double s = 0.0;
+#pragma unroll
+      for (int l = 0; l < N; ++l) s = fma(y.S[sidx<N>(i, l)], Lt[l * M + a], s);
+      SL[i * M + a] = s;
+    }
+#pragma unroll
+  for (int a = 0; a < M; ++a) {
+    double s = 0.0;
+#pragma unroll
+    for (int l = 0; l < N; ++l) s = fma(Lt[l * M + a], y.v[l], s);
+    w[a] = s;
+  }
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      double s = 0.0;
+#pragma unroll
+      for (int l = 0; l < N; ++l) s = fma(y.S[sidx<N>(i, l)], F[l * N + j], s);
+      SF[i * N + j] = s;
+    }
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+#pragma unroll
+    for (int j = i; j < N; ++j) {
+      double s = -Q[i * N + j] - SF[i * N + j] - SF[j * N + i];
+#pragma unroll
+      for (int a = 0; a < M; ++a) s = fma(SL[i * M + a], SL[j * M + a], s);
+      k.S[sidx<N>(i, j)] = s;
+    }
+  double z = -0.5 * qr[N];
+#pragma unroll
+  for (int a = 0; a < M; ++a) z = fma(0.5 * w[a], w[a], z);
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    double s = -qr[i];
+    if (c) {
+#pragma unroll
+      for (int l = 0; l < N; ++l) s = fma(y.S[sidx<N>(i, l)], c[l], s);
+    }
+#pragma unroll
+    for (int l = 0; l < N; ++l) s = fma(-F[l * N + i], y.v[l], s);
+#pragma unroll
+    for (int a = 0; a < M; ++a) s = fma(SL[i * M + a], w[a], s);
+    k.v[i] = s;
+    if (c) z = fma(y.v[i], c[i], z);
+  }
+  k.zeta = z;
+}
+
+// dx/dt = F x - Lt Lt^T (S x - v) + c
+template <int N, int M>
+__device__ __forceinline__ void closed_loop_rhs(const double* __restrict__ S, const double* __restrict__ v,
+                                                const double* __restrict__ x, const double* __restrict__ F,
+                                                const double* __restrict__ c, const double* __restrict__ Lt,
+                                                double* __restrict__ dx) {
+  double e[N], w[M];
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    double s = -v[i];
+#pragma unroll
+    for (int l = 0; l < N; ++l) s = fma(S[sidx<N>(i, l)], x[l], s);
+    e[i] = s;
+  }
+#pragma unroll
+  for (int a = 0; a < M; ++a) {
+    double s = 0.0;
+#pragma unroll
+    for (int l = 0; l < N; ++l) s = fma(Lt[l * M + a], e[l], s);
+    w[a] = s;
+  }
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    double s = c ? c[i] : 0.0;
+#pragma unroll
+    for (int l = 0; l < N; ++l) s = fma(F[i * N + l], x[l], s);
+#pragma unroll
+    for (int a = 0; a < M; ++a) s = fma(-Lt[i * M + a], w[a], s);
+    dx[i] = s;
+  }
+}
+
+// The two for constant F and Lt with zeros in them: entries whose bit in nzF, nzL
+// (nonzero_bits) is clear are skipped, each behind a branch.  Where every entry
+// counts the branches are a loss, so a full F takes the forms above (densification,
+// every coefficient per stage: n = 4, T = 20000 763 us by entry, 744 whole; n = 8
+// 6.66 and 6.23 ms; the sequential solve, point mass, T = 20000: 4.14 and 3.73 s).
+template <int N, int M>
+__device__ __forceinline__ void riccati_rhs_by_entry(const RicState<N>& y, const double* __restrict__ F,
+                                                     const double* __restrict__ c, const double* __restrict__ Lt,
+                                                     const double* __restrict__ Q, const double* __restrict__ qr,
+                                                     RicState<N>& k, unsigned long long nzF,
+                                                     unsigned long long nzL) {
   double SL[N * M], w[M], SF[N * N], Fv[N];
 #pragma unroll
   for (int e = 0; e < N * M; ++e) SL[e] = 0.0;
@@ -91,13 +186,13 @@ __device__ __forceinline__ void riccati_rhs(const RicState<N>& y, const double* 
   k.zeta = z;
 }
 
-// dx/dt = F x - Lt Lt^T (S x - v) + c
 template <int N, int M>
-__device__ __forceinline__ void closed_loop_rhs(const double* __restrict__ S, const double* __restrict__ v,
-                                                const double* __restrict__ x, const double* __restrict__ F,
-                                                const double* __restrict__ c, const double* __restrict__ Lt,
-                                                double* __restrict__ dx, unsigned long long nzF = ~0ull,
-                                                unsigned long long nzL = ~0ull) {
+__device__ __forceinline__ void closed_loop_rhs_by_entry(const double* __restrict__ S, const double* __restrict__ v,
+                                                         const double* __restrict__ x,
+                                                         const double* __restrict__ F,
+                                                         const double* __restrict__ c,
+                                                         const double* __restrict__ Lt, double* __restrict__ dx,
+                                                         unsigned long long nzF, unsigned long long nzL) {
   double e[N], w[M];
 #pragma unroll
   for (int i = 0; i < N; ++i) {
