@@ -163,10 +163,11 @@ struct Operands {
 // FP64 sum g_k + f_k equals the FP64 minimum has lo_k <= U; every k with
 // lo_k > U has a larger FP64 sum.  So the exact minimum, with the lowest-index
 // rule, is taken over the survivors lo_k <= U alone, in ascending k, in FP64.
-// Where no operand of the tile is negative, t_k is s_k itself, so that U = s_min
-// + c s_min and lo_k <= U is a bound on s_k: a candidate then costs one
-// addition and one minimum, and one addition and one comparison in the second
-// pass (a bound rounded up keeps a few candidates more, never fewer).
+// Where no operand of a stage is negative, t_k is s_k itself, so that the smallest
+// hi_k of the stage is s_min + c s_min, and with none negative in the whole tile
+// lo_k <= U is a bound on s_k: a candidate then costs one addition and one
+// minimum, and one addition and one comparison in the second pass (a bound
+// rounded up keeps a few candidates more, never fewer).
 // Operands of magnitude >= 2^100 (or not finite) fall outside the screen's
 // float range: a CTA that meets one evaluates every candidate in FP64.
 constexpr float kScreenC = 9.5367431640625e-07f;  // 2^-20
@@ -217,8 +218,8 @@ __device__ __forceinline__ int stage_float(const Operands<kValues>& op, float* A
     if (gk < G) {
       v = 0.0f;
       if (live) {
-        bad |= (screen_range(x) ? 0 : 1) | (x < 0.0 ? 2 : 0);
-        v = screen_float(x);
+        v = screen_float(x);  // (signs compared in float: an FP64 comparison takes 64 cycles)
+        bad |= (screen_range(x) ? 0 : 1) | (v < 0.0f ? 2 : 0);
       }
     }
     *dst = v;
@@ -274,10 +275,12 @@ __device__ __forceinline__ int stage_float(const Operands<kValues>& op, float* A
 // store.  Bound by the FP32 and ALU instructions of the two passes and, per
 // output, by some 30 FP64 instructions of the refinement (its three divisions)
 // at 64 cycles each.  One output per thread, with staging again in the second
-// pass, took 4.43 ms for the block and the values at G = 201, T = 10^4; this
-// 2.59 ms (2 x 4 outputs and two CTAs on an SM, loads one by one: 3.09).
+// pass, took 4.43 ms for the block and the values at G = 201, T = 10^4, 2 x 4 outputs
+// and two CTAs on an SM 3.09, 2 x 2 and three CTAs 2.59, and with the operands'
+// signs compared in float instead of FP64 2.29 (G = 60, T = 10^4, the values alone:
+// 670 us with one output per thread, 710 with the FP64 comparisons, 668).
 template <int P, int Q, bool kValues>
-__global__ void __launch_bounds__(kThreads, P * Q <= 4 ? 3 : 2)
+__global__ void __launch_bounds__(kThreads, 3)
     grid_minplus_kernel(GridArgs a, const double* __restrict__ A, const double* Bm, double* Om, double* X0,
                         double* X1, int l, int64_t ncols, const double2* __restrict__ tab) {
   constexpr int TR = 16 * P, TC = 16 * Q;
@@ -297,28 +300,48 @@ __global__ void __launch_bounds__(kThreads, P * Q <= 4 ? 3 : 2)
   for (int p = 0; p < P; ++p)
 #pragma unroll
     for (int q = 0; q < Q; ++q) U[p][q] = __int_as_float(0x7f800000);  // +inf
-  // pass 1, as if nothing were negative: the smallest sum
+  // pass 1: the smallest upper bracket, where a stage holds nothing negative by
+  // way of its smallest sum (the bracket grows with it)
+  bool neg = false;
   for (int k0 = 0; k0 < G; k0 += kc) {
     if (k0) __syncthreads();
-    bad |= stage_float<TR, TC>(op, As, Bs, S, t, i0, c0, ncols, k0, kc);
-    __syncthreads();
-    for (int kk = 0; kk < kc; kk += 4) {
-      float4 x[P], y[Q];
+    const int here = stage_float<TR, TC>(op, As, Bs, S, t, i0, c0, ncols, k0, kc);
+    bad |= here;
+    const bool signs = __syncthreads_or(here & 2) != 0;
+    neg = neg || signs;
+    float m[P][Q];
 #pragma unroll
-      for (int p = 0; p < P; ++p) x[p] = *reinterpret_cast<const float4*>(As + (ti + 16 * p) * S + kk);
+    for (int p = 0; p < P; ++p)
 #pragma unroll
-      for (int q = 0; q < Q; ++q) y[q] = *reinterpret_cast<const float4*>(Bs + (tc + 16 * q) * S + kk);
+      for (int q = 0; q < Q; ++q) m[p][q] = __int_as_float(0x7f800000);
+    auto pass1 = [&](auto sum) {
+      for (int kk = 0; kk < kc; kk += 4) {
+        float4 x[P], y[Q];
 #pragma unroll
-      for (int p = 0; p < P; ++p)
+        for (int p = 0; p < P; ++p) x[p] = *reinterpret_cast<const float4*>(As + (ti + 16 * p) * S + kk);
 #pragma unroll
-        for (int q = 0; q < Q; ++q) {
-          const float m0 = fminf(__fadd_rn(x[p].x, y[q].x), __fadd_rn(x[p].y, y[q].y));
-          const float m1 = fminf(__fadd_rn(x[p].z, y[q].z), __fadd_rn(x[p].w, y[q].w));
-          U[p][q] = fminf(U[p][q], fminf(m0, m1));
-        }
-    }
+        for (int q = 0; q < Q; ++q) y[q] = *reinterpret_cast<const float4*>(Bs + (tc + 16 * q) * S + kk);
+#pragma unroll
+        for (int p = 0; p < P; ++p)
+#pragma unroll
+          for (int q = 0; q < Q; ++q) {
+            const float m0 = fminf(sum(x[p].x, y[q].x), sum(x[p].y, y[q].y));
+            const float m1 = fminf(sum(x[p].z, y[q].z), sum(x[p].w, y[q].w));
+            m[p][q] = fminf(m[p][q], fminf(m0, m1));
+          }
+      }
+    };
+    if (signs)
+      pass1([](float x, float y) { return screen_hi(x, y); });
+    else
+      pass1([](float x, float y) { return __fadd_rn(x, y); });
+#pragma unroll
+    for (int p = 0; p < P; ++p)
+#pragma unroll
+      for (int q = 0; q < Q; ++q)
+        U[p][q] = fminf(U[p][q], signs ? m[p][q] : __fmaf_rn(kScreenC, m[p][q], m[p][q]));
   }
-  const bool range = __syncthreads_or(bad & 1) != 0, neg = __syncthreads_or(bad & 2) != 0;
+  const bool range = __syncthreads_or(bad & 1) != 0;
   unsigned long long pk[P][Q];  // survivors' indices, 16 bits each (G <= 16384)
   int ns[P][Q];
 #pragma unroll
@@ -339,7 +362,7 @@ __global__ void __launch_bounds__(kThreads, P * Q <= 4 ? 3 : 2)
     for (int p = 0; p < P; ++p)
 #pragma unroll
       for (int q = 0; q < Q; ++q) {
-        const float ub = __fadd_ru(__fmaf_rn(kScreenC, U[p][q], U[p][q]), kScreenD);
+        const float ub = __fadd_ru(U[p][q], kScreenD);
         thr[p][q] = __fmaf_ru(2.0f * kScreenC, ub, ub);
       }
     for (int k0 = 0; k0 < G; k0 += kc) {
@@ -370,30 +393,30 @@ __global__ void __launch_bounds__(kThreads, P * Q <= 4 ? 3 : 2)
       }
     }
   } else if (!range) {
-    // negative operands: the brackets with their own t_k
+    // negative operands: the brackets with their own t_k (a padded k's is far
+    // above every bound)
+    for (int k0 = 0; k0 < G; k0 += kc) {
+      if (G > kc) {
+        __syncthreads();
+        stage_float<TR, TC>(op, As, Bs, S, t, i0, c0, ncols, k0, kc);
+        __syncthreads();
+      }
+      for (int kk = 0; kk < kc; kk += 4) {
+        float4 x[P], y[Q];
 #pragma unroll
-    for (int p = 0; p < P; ++p)
+        for (int p = 0; p < P; ++p) x[p] = *reinterpret_cast<const float4*>(As + (ti + 16 * p) * S + kk);
 #pragma unroll
-      for (int q = 0; q < Q; ++q) U[p][q] = __int_as_float(0x7f800000);
-    for (int pass = 0; pass < 2; ++pass) {
-      for (int k0 = 0; k0 < G; k0 += kc) {
-        if (G > kc) {
-          __syncthreads();
-          stage_float<TR, TC>(op, As, Bs, S, t, i0, c0, ncols, k0, kc);
-          __syncthreads();
-        }
-        const int kend = G - k0 < kc ? G - k0 : kc;
-        for (int kk = 0; kk < kend; ++kk)
+        for (int q = 0; q < Q; ++q) y[q] = *reinterpret_cast<const float4*>(Bs + (tc + 16 * q) * S + kk);
 #pragma unroll
-          for (int p = 0; p < P; ++p)
+        for (int p = 0; p < P; ++p)
 #pragma unroll
-            for (int q = 0; q < Q; ++q) {
-              const float x = As[(ti + 16 * p) * S + kk], y = Bs[(tc + 16 * q) * S + kk];
-              if (pass == 0)
-                U[p][q] = fminf(U[p][q], screen_hi(x, y));
-              else if (screen_lo(x, y) <= __fadd_ru(U[p][q], kScreenD))
-                push(p, q, k0 + kk);
-            }
+          for (int q = 0; q < Q; ++q) {
+            const float ub = __fadd_ru(U[p][q], kScreenD);
+            if (screen_lo(x[p].x, y[q].x) <= ub) push(p, q, k0 + kk);
+            if (screen_lo(x[p].y, y[q].y) <= ub) push(p, q, k0 + kk + 1);
+            if (screen_lo(x[p].z, y[q].z) <= ub) push(p, q, k0 + kk + 2);
+            if (screen_lo(x[p].w, y[q].w) <= ub) push(p, q, k0 + kk + 3);
+          }
       }
     }
   }
