@@ -76,9 +76,7 @@ static Layout make_layout(const lqt_problem& p) {
   L.uniform = uniform_eligible(p);
   L.off_uni = off;
   if (L.uniform) off += uniform_table_bytes(p.n, L.M);
-  L.off_repeat = off;
   L.repeat_bytes = team_repeat_bytes(p, L.M, L.uniform);
-  off = align_up(off + L.repeat_bytes);
   L.coef_bytes = off;
   return L;
 }
@@ -124,9 +122,11 @@ size_t lqt_workspace_size(const lqt_problem* p, int32_t which) {
       return b ? b : 256;
     }
     case LQT_WS_TRAJ: return L.coef_bytes + scan_workspace_bytes(p->n, p->T, true);
-    case LQT_WS_SOLVE:
+    case LQT_WS_SOLVE: {
+      const size_t scan = scan_workspace_bytes(p->n, p->T, true);
       return L.coef_bytes + element_bytes(*p) + align_up(T1 * 8) + team_build_scratch_bytes(p->n) +
-             scan_workspace_bytes(p->n, p->T, true);
+             (L.repeat_bytes > scan ? L.repeat_bytes : scan);
+    }
     case LQT_WS_SEQUENTIAL: return L.coef_bytes + align_up(sequential_workspace_bytes(p->n, p->T, p->K));
     case LQT_WS_BACKWARD: return backward_workspace_bytes(*p, L, element_bytes(*p)) + 4096;
     case LQT_WS_DENSIFY: return L.coef_bytes;
@@ -212,8 +212,10 @@ lqt_status lqt_solve(const lqt_problem* p, const double* x0, double* S, double* 
   double* zbuf = (double*)(base + L.coef_bytes + element_bytes(*p));
   double* zout = zeta ? zeta : zbuf;
   char* team_scr = base + L.coef_bytes + element_bytes(*p) + align_up(((size_t)p->T + 1) * 8);
-  if (launch_build(*p, L, cf, el, st, (double*)team_scr) != cudaSuccess) return LQT_ECUDA;
   char* scan = team_scr + team_build_scratch_bytes(p->n);
+  // the mixed build by repeated lengths works in the scan's region before the scan does
+  if (mixed_precision() && L.repeat_bytes) cf.repeat = scan;
+  if (launch_build(*p, L, cf, el, st, (double*)team_scr) != cudaSuccess) return LQT_ECUDA;
   return from_cuda(run_value_and_traj(*p, L, cf, el, S, v, zout, x0, x, u, cost, true, true, nullptr, nullptr, scan,
                                       ws_bytes - (scan - base), st));
 }

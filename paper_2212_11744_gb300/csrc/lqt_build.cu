@@ -435,7 +435,6 @@ cudaError_t launch_prepare_coefs(const lqt_problem& p, const Layout& lay, char* 
   const cudaError_t e = launch_prepare_into(p, lay, (double*)(ws + lay.off_Lt), (double*)(ws + lay.off_Q),
                                             (double*)(ws + lay.off_qr), (double*)(ws + lay.off_Ku), cf, st);
   if (lay.uniform) cf.uni = (const double*)(ws + lay.off_uni);
-  if (lay.repeat_bytes) cf.repeat = ws + lay.off_repeat;
   return e;
 }
 

@@ -64,7 +64,7 @@ struct Coefs {
   // table of the constant-coefficient build (lqt_uniform.cu); NULL: the
   // general build makes every element
   const double* uni;
-  // workspace of the build by repeated lengths (lqt_team.cu), n = 64; NULL: none
+  // workspace of the mixed solve's build by repeated lengths (lqt_team.cu), n = 64; NULL: none
   char* repeat;
 };
 
@@ -80,7 +80,7 @@ struct Layout {
   // byte offsets inside the workspace
   size_t off_Lt, off_Q, off_qr, off_Ku, off_uni;
   bool uniform;  // the constant-coefficient build applies (lqt_uniform.cu)
-  size_t off_repeat, repeat_bytes;  // the build by repeated lengths (0 bytes: does not apply)
+  size_t repeat_bytes;  // the mixed solve's build by repeated lengths (0: does not apply), not in coef_bytes
   size_t coef_bytes;  // end of the coefficient region
 };
 
