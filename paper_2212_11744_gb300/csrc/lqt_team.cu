@@ -78,12 +78,12 @@ struct TeamCfg<64> {
 // Doubles of per-slot scratch of each kernel.
 template <int N, int M>
 constexpr int build_slot_doubles() { return Rec<N>::SIZE + 3 * Rec<N>::FLOW + 2 * N * M + M + 8; }
+// (the mixed n = 64 combinations: two records and T1; two value records, the chunk
+// composite with its scratch and T1)
 template <int N>
-constexpr int reduce_slot_doubles() { return 2 * Rec<N>::SIZE + team::combine_scratch_doubles<N>() + 8; }
+constexpr int reduce_slot_doubles() { return 2 * Rec<N>::SIZE + N * N; }
 template <int N>
-constexpr int down_slot_doubles() {
-  return 2 * team::val_doubles<N>() + team::value_scratch_doubles<N>() + 3 * (N * N + N) + N * N + N + 8;
-}
+constexpr int down_slot_doubles() { return 2 * team::val_doubles<N>() + 2 * (N * N + N) + N * N; }
 template <int N>
 constexpr int maps_slot_doubles() { return 3 * (N * N + N) + 2 * N + 8; }
 
@@ -506,10 +506,8 @@ __global__ void __launch_bounds__(TeamCfg<N>::TEAM) build_forward_team_kernel(Te
 // stage (b): reduce / down-sweep of the value scan
 // ---------------------------------------------------------------------------
 
-// The FP32 products of the n = 64 combinations run on the tensor core.
-template <int N, typename GT>
-constexpr bool kTensorProducts = (N == 64 && std::is_same<GT, float>::value);
-// The FP64 combinations of n = 64 run on split products (lqt_split64.cuh).
+// The FP64 combinations of n = 64 run on split products (lqt_split64.cuh), the
+// mixed ones' FP32 products on the tensor core (lqt_tc64.cuh).
 template <int N, typename GT>
 constexpr bool kSplit64 = (N == 64 && std::is_same<GT, double>::value);
 // The tensor-core instances: the operand tiles, then W, R and the vectors
@@ -545,31 +543,23 @@ __device__ __forceinline__ Rec<N> level_elem(const TeamScanArgs& a, int64_t k, d
   return Rec<N>::pub(a.el, k, zero);
 }
 
-template <int N, typename GT = double>
-__global__ void __launch_bounds__(TeamCfg<N>::TEAM, TeamCfg<N>::SCAN_MIN) reduce_team_kernel(TeamScanArgs a) {
-  constexpr int TEAM = TeamCfg<N>::TEAM;
-  constexpr int SD = reduce_slot_doubles<N>();
+// The mixed-precision combinations of n = 64, one CTA each.
+__global__ void __launch_bounds__(TeamCfg<64>::TEAM, TeamCfg<64>::SCAN_MIN) reduce_team_kernel(TeamScanArgs a) {
+  constexpr int N = 64, TEAM = TeamCfg<N>::TEAM;
   __shared__ double fs[2 * TEAM];
   __shared__ int is[TEAM];
   __shared__ double zero;
+  __shared__ uint32_t tmem_slot;
+  __shared__ unsigned long long tc_bar;
+  extern __shared__ __align__(16) unsigned char tc_smem[];
   const int lane = threadIdx.x;
   if (lane == 0) zero = 0.0;
-  double* base = slot_base<N>(a.gscratch, SD);
-  double* bufA = base;
+  double* bufA = slot_base<N>(a.gscratch, reduce_slot_doubles<N>());
   double* bufB = bufA + Rec<N>::SIZE;
-  double* scr = bufB + Rec<N>::SIZE;
-  double* t1 = nullptr;
-  tc::Ctx* tcx = nullptr;
-  tc::Ctx tc_ctx;
-  if constexpr (kTensorProducts<N, GT>) {
-    extern __shared__ __align__(16) unsigned char tc_smem[];
-    __shared__ uint32_t tmem_slot;
-    __shared__ unsigned long long tc_bar;
-    tc::init(tc_ctx, &tmem_slot, &tc_bar, tc_smem);
-    tcx = &tc_ctx;
-    t1 = scr + N * N + N * (2 * N + 1);
-    scr = reinterpret_cast<double*>(tc_smem + tc::kSmemBytes);
-  }
+  double* t1 = bufB + Rec<N>::SIZE;
+  tc::Ctx tcx;
+  tc::init(tcx, &tmem_slot, &tc_bar, tc_smem);
+  double* scr = reinterpret_cast<double*>(tc_smem + tc::kSmemBytes);
   team::sync<TEAM>();
   const int64_t groups = tdiv(a.cnt, a.G);
   for (int64_t g = blockIdx.x; g < groups; g += gridDim.x) {
@@ -578,51 +568,41 @@ __global__ void __launch_bounds__(TeamCfg<N>::TEAM, TeamCfg<N>::SCAN_MIN) reduce
     Rec<N> acc = Rec<N>::packed(bufA), nxt = Rec<N>::packed(bufB);
     team::copy_rec<N, TEAM>(lane, acc, level_elem<N>(a, last, &zero));
     for (int64_t k = last - 1; k >= first; --k) {
-      team::combine<N, TEAM, GT>(lane, level_elem<N>(a, k, &zero), acc, nxt, scr, fs, is, tcx, t1);
+      team::combine<N, TEAM, float>(lane, level_elem<N>(a, k, &zero), acc, nxt, scr, fs, is, &tcx, t1);
       const Rec<N> t = acc;
       acc = nxt;
       nxt = t;
     }
     team::copy_rec<N, TEAM>(lane, Rec<N>::packed(a.agg + g * Rec<N>::SIZE), acc);
   }
-  if constexpr (kTensorProducts<N, GT>) tc::release(tc_ctx);
+  tc::release(tcx);
 }
 
-template <int N, bool Level0, typename GT = double>
-__global__ void __launch_bounds__(TeamCfg<N>::TEAM, TeamCfg<N>::SCAN_MIN) down_team_kernel(TeamScanArgs a) {
-  constexpr int TEAM = TeamCfg<N>::TEAM;
-  constexpr int SD = down_slot_doubles<N>();
+template <bool Level0>
+__global__ void __launch_bounds__(TeamCfg<64>::TEAM, TeamCfg<64>::SCAN_MIN) down_team_kernel(TeamScanArgs a) {
+  constexpr int N = 64, TEAM = TeamCfg<N>::TEAM;
   constexpr int VS = team::val_doubles<N>();
   constexpr int PM = N * N + N;
   __shared__ double fs[2 * TEAM];
   __shared__ int is[TEAM];
   __shared__ double zero;
   __shared__ double zinc;
+  __shared__ uint32_t tmem_slot;
+  __shared__ unsigned long long tc_bar;
+  extern __shared__ __align__(16) unsigned char tc_smem[];
   const int lane = threadIdx.x;
   if (lane == 0) zero = 0.0;
-  double* base = slot_base<N>(a.gscratch, SD);
-  double* c0 = base;
+  double* c0 = slot_base<N>(a.gscratch, down_slot_doubles<N>());
   double* c1 = c0 + VS;
-  double* scr = c1 + VS;
-  double* Psi = scr + team::value_scratch_doubles<N>();
-  double* alpha = Psi + N * N;
-  double* P = alpha + N;
+  double* P = c1 + VS;
   double* pv = P + N * N;
   double* Tm = pv + N;
-  double* t1 = nullptr;
-  tc::Ctx* tcx = nullptr;
-  tc::Ctx tc_ctx;
-  if constexpr (kTensorProducts<N, GT>) {
-    extern __shared__ __align__(16) unsigned char tc_smem[];
-    __shared__ uint32_t tmem_slot;
-    __shared__ unsigned long long tc_bar;
-    tc::init(tc_ctx, &tmem_slot, &tc_bar, tc_smem);
-    tcx = &tc_ctx;
-    t1 = scr + N * N + N * (N + 1);
-    scr = reinterpret_cast<double*>(tc_smem + tc::kSmemBytes);
-    Psi = scr + N * N + N * (N + 1) + 3 * N;
-    alpha = Psi + N * N;
-  }
+  double* t1 = Tm + PM;
+  tc::Ctx tcx;
+  tc::init(tcx, &tmem_slot, &tc_bar, tc_smem);
+  double* scr = reinterpret_cast<double*>(tc_smem + tc::kSmemBytes);
+  double* Psi = scr + N * N + N * (N + 1) + 3 * N;
+  double* alpha = Psi + N * N;
   team::sync<TEAM>();
   const int64_t groups = tdiv(a.cnt, a.G);
   for (int64_t g = blockIdx.x; g < groups; g += gridDim.x) {
@@ -639,7 +619,8 @@ __global__ void __launch_bounds__(TeamCfg<N>::TEAM, TeamCfg<N>::SCAN_MIN) down_t
       }
     team::sync<TEAM>();
     for (int64_t k = last; k >= first; --k) {
-      team::combine_value<N, TEAM, GT>(lane, level_elem<N>(a, k, &zero), carry, nv, Psi, alpha, scr, fs, is, &zinc, tcx, t1);
+      team::combine_value<N, TEAM, float>(lane, level_elem<N>(a, k, &zero), carry, nv, Psi, alpha, scr, fs, is, &zinc,
+                                          &tcx, t1);
       if (Level0) {
         bool ok = true;
         for (int e = lane; e < VS; e += TEAM) {
@@ -666,7 +647,7 @@ __global__ void __launch_bounds__(TeamCfg<N>::TEAM, TeamCfg<N>::SCAN_MIN) down_t
       for (int e = lane; e < PM; e += TEAM) a.comp[g * PM + e] = e < N * N ? P[e] : pv[e - N * N];
     team::sync<TEAM>();
   }
-  if constexpr (kTensorProducts<N, GT>) tc::release(tc_ctx);
+  tc::release(tcx);
 }
 
 __device__ __forceinline__ bool finite_bits(double x) {
@@ -1192,13 +1173,12 @@ static void launch_reduce(const TeamScanArgs& a, int64_t groups, cudaStream_t st
     cudaFuncSetAttribute(reduce_s64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(s64::Shared));
     reduce_s64_kernel<<<team_grid<N>(groups, TeamCfg<N>::SCAN_SLOTS), s64::kThreads, sizeof(s64::Shared), st>>>(a);
     count_launch();
-  } else if constexpr (kTensorProducts<N, GT>) {
-    constexpr size_t smem = kTcReduceSmemBytes<N>;
-    cudaFuncSetAttribute(reduce_team_kernel<N, GT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    reduce_team_kernel<N, GT><<<team_grid<N>(groups, TeamCfg<N>::SCAN_SLOTS), TeamCfg<N>::TEAM, smem, st>>>(a);
-    count_launch();
   } else {
-    team_launch<N>(reduce_team_kernel<N, GT>, groups, reduce_slot_doubles<N>(), a, st, TeamCfg<N>::SCAN_SLOTS);
+    static_assert(N == 64, "n = 16 and 64");
+    constexpr size_t smem = kTcReduceSmemBytes<N>;
+    cudaFuncSetAttribute(reduce_team_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    reduce_team_kernel<<<team_grid<N>(groups, TeamCfg<N>::SCAN_SLOTS), TeamCfg<N>::TEAM, smem, st>>>(a);
+    count_launch();
   }
 }
 
@@ -1215,13 +1195,12 @@ static void launch_down(const TeamScanArgs& a, int64_t groups, cudaStream_t st) 
     down_s64_kernel<Level0>
         <<<team_grid<N>(groups, TeamCfg<N>::SCAN_SLOTS), s64::kThreads, sizeof(s64::Shared), st>>>(a);
     count_launch();
-  } else if constexpr (kTensorProducts<N, GT>) {
-    constexpr size_t smem = kTcDownSmemBytes<N>;
-    cudaFuncSetAttribute(down_team_kernel<N, Level0, GT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    down_team_kernel<N, Level0, GT><<<team_grid<N>(groups, TeamCfg<N>::SCAN_SLOTS), TeamCfg<N>::TEAM, smem, st>>>(a);
-    count_launch();
   } else {
-    team_launch<N>(down_team_kernel<N, Level0, GT>, groups, down_slot_doubles<N>(), a, st, TeamCfg<N>::SCAN_SLOTS);
+    static_assert(N == 64, "n = 16 and 64");
+    constexpr size_t smem = kTcDownSmemBytes<N>;
+    cudaFuncSetAttribute(down_team_kernel<Level0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    down_team_kernel<Level0><<<team_grid<N>(groups, TeamCfg<N>::SCAN_SLOTS), TeamCfg<N>::TEAM, smem, st>>>(a);
+    count_launch();
   }
 }
 
@@ -1478,27 +1457,18 @@ void team_prefix_maps(const double* maps, int64_t cnt, const double* x_in, doubl
 template <int N, typename GT>
 void team_upper_reduce(const double* src, int64_t cnt, double* agg, cudaStream_t st) {
   static_assert(Rec<N>::SIZE == full_elem_doubles<N>(), "record layouts differ");
-  if constexpr (N == 4 || N == 8) {
+  // (no level of n <= 3 is below its line: lqt_scan.cu, team_level_below)
+  if constexpr (N == 4 || N == 8)
     team_launch<N>(reduce_w8_kernel<N, GT>, tdiv(cnt, 2), 0, src, st, TeamCfg<N>::SLOTS, cnt, agg);
-  } else {
-    TeamScanArgs a{};
-    a.src = src; a.cnt = cnt; a.G = 2; a.agg = agg;
-    team_launch<N>(reduce_team_kernel<N, GT>, tdiv(cnt, 2), reduce_slot_doubles<N>(), a, st);
-  }
 }
 
 template <int N, typename GT>
 void team_upper_down(const double* src, int64_t cnt, const double* above, int64_t cnt_above, double* vals,
                      cudaStream_t st) {
   static_assert(team::val_doubles<N>() == full_val_doubles<N>(), "value layouts differ");
-  if constexpr (N == 4 || N == 8) {
+  if constexpr (N == 4 || N == 8)
     team_launch<N>(down_w8_kernel<N, GT>, tdiv(cnt, 2), 0, src, st, TeamCfg<N>::SLOTS, cnt, above, cnt_above,
                    vals);
-  } else {
-    TeamScanArgs a{};
-    a.src = src; a.cnt = cnt; a.G = 2; a.above = above; a.cnt_above = cnt_above; a.vals = vals;
-    team_launch<N>(down_team_kernel<N, false, GT>, tdiv(cnt, 2), down_slot_doubles<N>(), a, st);
-  }
 }
 
 template <int N>
@@ -1731,7 +1701,7 @@ static TeamPrefixPlan<N> team_prefix_plan(int64_t T) {
   pl.off_scratch = off;
   if (!TeamCfg<N>::SMEM) {
     size_t sd = m2_slot_doubles<N>();
-    if ((size_t)reduce_slot_doubles<N>() > sd) sd = reduce_slot_doubles<N>();
+    if ((size_t)kS64SlotDoubles > sd) sd = kS64SlotDoubles;  // launch_reduce<64, double>
     if ((size_t)prefix_slot_doubles<N>() > sd) sd = prefix_slot_doubles<N>();
     off = tal(off + (size_t)TeamCfg<N>::SLOTS * sd * sizeof(double));
   }
