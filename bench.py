@@ -969,10 +969,23 @@ def run_ours(args):
             "clocks": clocks,
             "rows": rows,
         }
-        print(json.dumps(line))
+        print(json.dumps(line), file=sys.stderr)
+        print(json.dumps(result_line(line)))
     if ws_ > 1:
         import torch.distributed as dist
         dist.destroy_process_group()
+
+
+def result_line(full):
+    """The one line on stdout: the result and what qualifies it, below 2000
+    characters, so that a reader of a log's tail gets it whole.  The full record,
+    with every row's notes, is one JSON line on stderr."""
+    pick = lambda d, *keys: {k: d[k] for k in keys} if d else d
+    line = {k: v for k, v in full.items() if k not in ("roofline_step", "pipes_measured", "rows")}
+    line["roofline"] = pick(full["roofline"], "bound", "kernel", "achieved", "peak", "unit", "frac", "traffic")
+    line["sequential_gpu"] = pick(full["sequential_gpu"], "value", "unit", "T_timed", "speedup_parallel_over_sequential")
+    line["cpu_baseline"] = pick(full["cpu_baseline"], "value", "unit", "cores")
+    return line
 
 
 def main():
