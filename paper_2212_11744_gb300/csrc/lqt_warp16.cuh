@@ -646,7 +646,8 @@ template <int NW>
 __device__ __forceinline__ void refine_inverse(const double* W, double* Minv, double* E, int ld, bool fast,
                                                int limit) {
   constexpr int kExp1 = 1023;  // biased exponent of 1
-  // at most four steps: |W M - I| < 2^-28 (row sum) before the last one
+  // at most four steps: |W M - I| < 2^-28 (row sum: sixteen entries below 2^-32)
+  // before the last one
   int last = kExp1 - 1;
   for (int it = 0; it < 4; ++it) {
     if (!fast) {
@@ -656,7 +657,7 @@ __device__ __forceinline__ void refine_inverse(const double* W, double* Minv, do
     const int top = split::product16<NW>(rows_of(W, kWld), cols_of(Minv, kWld), rows_of(E, ld), -1, split::kSet,
                                            limit);
     // the residual must fall at least eightfold per step, from below 1/16
-    bool done = top <= kExp1 - 32, lost = top > last - 3 || top > kExp1 - 5;
+    bool done = top <= kExp1 - 33, lost = top > last - 3 || top > kExp1 - 5;
     if constexpr (NW > 1) {
       done = __syncthreads_and(done) != 0;
       lost = __syncthreads_or(lost) != 0;
