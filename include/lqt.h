@@ -34,7 +34,11 @@
  *    and lqt_solve_host().
  *  - Matrices are row-major and dense; symmetric outputs are written in full.
  *    Arrays indexed by boundary run over k = 0..T (T+1 entries).
- *  - FP64 throughout.
+ *  - FP64 throughout (lqt_solve_mixed apart).  At n = 16 and 64 the products of
+ *    the combinations are formed from 16-bit digits on the tensor cores, exact
+ *    sums rounded once, wherever that is as accurate as FP64 multiplication,
+ *    and in FP64 elsewhere (states in mixed units, subnormal or infinite
+ *    entries).
  *  - Errors: invalid arguments are rejected on the host before any launch and
  *    returned directly.  Numerical trouble found on the device (a non-finite
  *    value in an output; a singular system) is recorded in a per-device status

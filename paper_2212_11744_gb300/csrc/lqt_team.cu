@@ -743,9 +743,9 @@ __global__ void __launch_bounds__(s64::kThreads, 1) down_s64_kernel(TeamScanArgs
   }
 }
 
-// n = 16: one warp per combination with the register Gauss-Jordan solve and
-// TMA-staged element operands (lqt_warp16.cuh).  Same levels, groups and
-// records as the kernels above.
+// n = 16, TMA-staged element operands (lqt_warp16.cuh): FP64 by two warps on split
+// products, mixed by one warp with a register Gauss-Jordan solve.  Same levels,
+// groups and records as the n = 64 kernels.
 template <typename GT>
 constexpr bool kSplit16 = std::is_same<GT, double>::value;  // FP64: split products (lqt_split.cuh)
 template <typename GT>

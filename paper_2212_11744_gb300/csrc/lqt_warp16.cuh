@@ -1,17 +1,22 @@
-// One warp per combination for n = 16: the combination rule of Sec. IV-A (eq.
-// lqt_comb, full and value form) with the warp's 32 lanes used on every FP64
-// instruction, and the linear solve of I + C1 J2 (App. B) as a register
-// resident Gauss-Jordan elimination.
+// The combinations for n = 16 (the rule of Sec. IV-A, eq. lqt_comb, full and value
+// form; the linear solve of I + C1 J2, App. B).  On this GPU a warp's FP64
+// instruction occupies its sub-partition for 64 cycles whatever the number of
+// active lanes, which decides both forms here:
 //
-// Why: on this GPU a warp's FP64 instruction occupies its sub-partition for
-// 64 cycles whatever the number of active lanes, and the solve is a chain of
-// 16 dependent pivot steps.  Written as an LU in shared memory with a barrier
-// after every step (and a second pass for the back substitution), the chain
-// left the FP64 pipe idle most of the time.  Here each lane owns one column of
-// [W | X1] in registers (lanes 0..15: W, lanes 16..31: X1) and one row slice
-// of X2 and of the vector x, so one pass of 16 steps solves
-// W [X1 | X2 | x] = [X1 | X2 | x]_in with 16-26 independent FMAs per lane per
-// step, no shared-memory traffic and no barriers inside the elimination.
+// FP64 (combine_split, combine_value_split): the 16^3 products on the FP16 tensor
+// cores as split products (lqt_split.cuh) and an inverse made in FP32 and refined
+// by Newton steps; two warps per combination in the scans, one in Method 2's
+// fold.  See the section's own comment below.
+//
+// Mixed precision (combine, combine_value): FP32 products by one warp, and the
+// solve as a register resident FP64 Gauss-Jordan elimination.  The elimination is
+// a chain of 16 dependent pivot steps.  Written as an LU in shared memory with a
+// barrier after every step (and a second pass for the back substitution), the
+// chain left the FP64 pipe idle most of the time.  Here each lane owns one column
+// of [W | X1] in registers (lanes 0..15: W, lanes 16..31: X1) and one row slice of
+// X2 and of the vector x, so one pass of 16 steps solves W [X1 | X2 | x] = [X1 | X2
+// | x]_in with 16-26 independent FMAs per lane per step, no shared-memory traffic
+// and no barriers inside the elimination.
 //
 // The element operand of every combination is staged in shared memory by the
 // TMA unit (cp.async.bulk, completion on an mbarrier with a bounded wait),
@@ -492,7 +497,9 @@ __device__ __forceinline__ void compose_right(int lane, double* P, double* p, co
 // Where an FP32 pivot falls below 2^-10 of its row or the residual does not
 // shrink (cond(W) beyond some 1e5), the inverse is made in FP64 with the
 // pivots and the SINGULAR test of gauss_jordan, and the Newton step polishes
-// that one.
+// that one.  In states of mixed units (split::kFoldLimit) the inverse and all
+// products are FP64, the Newton step too: it takes out what the elimination's
+// pivots, which feel the units, leave.
 
 // x[k], k = 0..7, without indexing a local array.
 template <typename X>
