@@ -3,17 +3,19 @@
 //
 // What bounds it: in FP64 a full combination is 2.0 M multiply-adds, 500 us on
 // one SM's FP64 pipe (820 us as measured, with the barriers of the LU).  Here
-// its fourteen 64^3 products are FP16 tensor-core products of seven digits;
-// per product the splitting of 8 k entries and the assembly of 4 k results
-// (integer work) take about as long as the 28 digit products.  Each entry is split
-// once, by the warp that owns eight rows of the left or columns of the right
-// operand, and the digits are kept in shared memory in fragment order; each of
-// the sixteen warps then forms 16 x 16 outputs: 23.7 k cycles a product, 398 k a
-// combination, of which the FP32 inverse takes 64 k.  (Eight warps with the left
-// digits in registers, split twice: 27 k a product.)  W = I + C1 J2 is
-// inverted in FP32 (Gauss-Jordan in registers) and refined by Newton steps, as
-// for n = 16 (lqt_warp16.cuh), with the FP64 elimination behind it where that
-// does not converge.
+// its fourteen 64^3 products are FP16 tensor-core products of seven digits.  A
+// full combination takes 0.24 ms, alone or 66 at once (ncu, 512 threads on an SM): the
+// ALU pipe is 31% busy (splitting 8 k entries and assembling 4 k results a
+// product), the FP64 pipe 24% (vectors), the
+// tensor pipe 18%, and the warps wait on one another's digits and on shared
+// memory.  Each entry is split once, by the warp that owns eight rows of the left
+// or columns of the right operand, and the digits are kept in shared memory in
+// fragment order; each of the sixteen warps then forms 16 x 16 outputs.  (Eight
+// warps with the left digits in registers, split twice, took 27 k cycles a
+// product against 23.7 k.)  W = I + C1 J2 is inverted in FP32 (Gauss-Jordan in
+// registers, 64 k cycles) and refined by Newton steps, as for n = 16
+// (lqt_warp16.cuh), with the FP64 elimination behind it where that does not
+// converge, and in FP64 altogether in mixed units (lqt_split.cuh).
 #pragma once
 
 #include <cuda_runtime.h>

@@ -20,8 +20,8 @@
 // partly uniform.
 //
 // What bounds it: the general build is bound by the FP64 pipe (K (40 n^3 +
-// 60 n^2) flop per sub-interval); here a sub-interval costs 6 n^2 + 12 n^2
-// flop and the store of its element.  One CTA per step value holds the
+// 60 n^2) flop per sub-interval); here a sub-interval costs 18 n^2 FP64
+// operations and the store of its element.  One CTA per step value holds the
 // integrated element in shared memory (n <= 16); at n = 64, where one
 // element's integration is 70 Mflop, a cluster of eight CTAs shares it through
 // its workspace (L2) with a cluster barrier between the phases of a stage.
@@ -278,8 +278,9 @@ int64_t uniform_chunks(int n, int64_t T) { return (T + uni_chunk(n) - 1) / uni_c
 // the entries e of A, C, J (value and slope) in registers and writes them for
 // every sub-interval of the chunk (consecutive lanes, consecutive addresses);
 // for eta, b and the rows of Z q a thread owns row i of one or more
-// sub-intervals.  Bound by the store of 3 n^2 + 2 n + 1 doubles per
-// sub-interval (n <= 8), by 18 n^2 FP64 operations above.
+// sub-intervals.  Bound by its 18 n^2 FP64 operations per sub-interval (FP64 pipe
+// 81% busy at n = 16, T = 4104), which at 64 cycles a warp instruction take longer
+// than the store of 3 n^2 + 2 n + 1 doubles at every n.
 // Batches: one CTA per chunk of a problem that has a table, found by the chunks'
 // prefix sum.  (A grid of the longest problem's chunks times B was 16.8 million
 // CTAs for one problem of T = 2^19 beside 2047 of T = 64, n = 4: 47.5 ms for the

@@ -486,7 +486,7 @@ __device__ __forceinline__ void compose_right(int lane, double* P, double* p, co
 // the FP64 combinations: split products (lqt_split.cuh) and an inverse
 // ---------------------------------------------------------------------------
 //
-// What bounds a combination is the FP64 pipe, at 64 cycles a warp
+// Done in FP64, a combination is bound by that pipe, at 64 cycles a warp
 // instruction: five to six 16^3 products took 128 instructions each and the
 // elimination of 2 n + 1 right-hand sides 530.  The products now run on the
 // tensor core (about 800 cycles of a sub-partition each, integer work, against
@@ -500,6 +500,9 @@ __device__ __forceinline__ void compose_right(int lane, double* P, double* p, co
 // that one.  In states of mixed units (split::kFoldLimit) the inverse and all
 // products are FP64, the Newton step too: it takes out what the elimination's
 // pivots, which feel the units, leave.
+// Level 0 of a scan, T = 4104 (ncu, 6.8 CTAs on an SM): the ALU pipe, which splits
+// and assembles, is 50% busy, the FP64 pipe (vectors, inverse) 40%, the tensor pipe
+// 6%; the warps wait on their own results and on instruction fetches.
 
 // x[k], k = 0..7, without indexing a local array.
 template <typename X>
