@@ -278,9 +278,11 @@ __device__ __forceinline__ int stage_float(const Operands<kValues>& op, float* A
 // pass, took 4.43 ms for the block and the values at G = 201, T = 10^4, 2 x 4 outputs
 // and two CTAs on an SM 3.09, 2 x 2 and three CTAs 2.59, and with the operands'
 // signs compared in float instead of FP64 2.29 (G = 60, T = 10^4, the values alone:
-// 670 us with one output per thread, 710 with the FP64 comparisons, 668).
+// 670 us with one output per thread, 710 with the FP64 comparisons, 668).  The
+// small tiles take four CTAs on an SM: the values at T = 10^4 in one graph 408 -> 369 us
+// at G = 20, 489 -> 477 at 40, 609 -> 558 at 60.
 template <int P, int Q, bool kValues>
-__global__ void __launch_bounds__(kThreads, 3)
+__global__ void __launch_bounds__(kThreads, P * Q == 1 ? 4 : 3)
     grid_minplus_kernel(GridArgs a, const double* __restrict__ A, const double* Bm, double* Om, double* X0,
                         double* X1, int l, int64_t ncols, const double2* __restrict__ tab) {
   constexpr int TR = 16 * P, TC = 16 * Q;
